@@ -79,6 +79,8 @@ struct ferrox_ctx {
   double* Fbuf = nullptr;
   double* phi_prev = nullptr;         // previous step's potential (guess = 1)
   void* e_arena = nullptr;
+  float* eb_arena = nullptr;          // black corrections between the legs of a V-cycle
+  bool legs = false;                  // FP32 levels run one launch per leg (leg_device.cuh)
   void* e_alt = nullptr;              // second error array of the fused sweeps (largest such level)
   void* r_arena = nullptr;
   void* s_arena = nullptr;
@@ -86,7 +88,8 @@ struct ferrox_ctx {
   PlaneCoef<double>* coef0 = nullptr; // level 0 in FP64 (outer residual)
   PlaneCoef<double>* coef0s = nullptr; // level 0 divided by the diagonal (direct form's sweeps)
   double* bs = nullptr;                // b / diag (direct form's fine sweeps)
-  void* sinv0 = nullptr;               // 1 / (diag + s) on level 0 (T; with a Newton shift)
+  void* sinv0 = nullptr;               // 1 / (diag + s) on level 0 (T; with a Newton shift), with
+                                       // legs on every level
   PlaneCoefDF* coef_df = nullptr;     // level 0 as double-float pairs (double-float residual)
   bool df_resid = false;              // the mixed form's outer residual in double-float
   PlaneTDGL* planes_d = nullptr;
@@ -504,11 +507,25 @@ bool rb_sweeps(const ferrox_ctx* c, int l, int nu) {
   return c->e_alt && nu % 2 == 0 && smooth_rb_tile<T>(c->lv[l], c->shift) > 0;
 }
 
+// Levels whose smoothing and transfers run as one launch per V-cycle leg
+bool leg_at(const ferrox_ctx* c, int l) { return c->legs && l < c->tail_first && leg_level(c->lv[l]); }
+
 // kernels of one smoothing of level l with nu sweeps
 int smoothing_launches(const ferrox_ctx* c, int l, int nu) {
   const bool rb = c->num.precision == FERROX_MIXED ? rb_sweeps<float>(c, l, nu)
                                                    : rb_sweeps<double>(c, l, nu);
   return rb ? nu : 2 * nu;
+}
+
+bool separate_update(const ferrox_ctx* c);
+
+// algorithmic bytes of one leg: r (and s) once, the black corrections written or read,
+// the coarse arrays, a starting correction's black half, and e or phi at the end
+double leg_bytes(const ferrox_ctx* c, int l, bool down, bool first, bool fold) {
+  const double n = (double)c->lv[l].ncell, nc = (double)c->lv[l + 1].ncell;
+  double b = n * 4.0 * (c->shift ? 2.0 : 1.0) + n * 2.0 + nc * 4.0;
+  if (down) return b + (l == 0 && !first ? n * 2.0 : 0.0);
+  return b + (l == 0 && fold ? n * 16.0 : n * 4.0);
 }
 
 // first: the fine level starts from a zero correction; last: phi += e rides on
@@ -525,9 +542,39 @@ void enqueue_levels(ferrox_ctx* c, cudaStream_t s, W wrap, int l0, bool first, b
   const int constant = 0;
   const int lt = c->tail_first, L = (int)c->lv.size() - 1;
   T* alt = static_cast<T*>(c->e_alt);
+  const UpdateArgs upd{c->phi, c->stats_d, update_clamp(c)};
+  // the fine level's e is wanted whole where phi is not updated by its last sweep
+  const bool fold = last && !separate_update(c);
+  auto leg_args = [&](int l) {
+    const LevelDesc &F = c->lv[l], &C = c->lv[l + 1];
+    LegArgs g{};
+    if constexpr (sizeof(T) == sizeof(float)) {
+      g.r = a.r + F.off;
+      g.s = a.s ? a.s + F.off : nullptr;
+      g.sinv = a.s ? static_cast<const float*>(c->sinv0) + F.off : nullptr;
+      g.e_in = l == 0 && !first ? a.e : nullptr;
+      g.eb = c->eb_arena + F.off / 2;
+      g.rc = a.r + C.off;
+      // the shift is fixed between two residuals: restricted by the first V-cycle after one
+      g.sc = a.s && (first || adapt_max(c) > 0) ? a.s + C.off : nullptr;
+      g.sinvc = g.sc && leg_at(c, l + 1) ? static_cast<float*>(c->sinv0) + C.off : nullptr;
+      g.coefc = a.coef + C.coef_off;
+      g.ec = a.e + C.off;
+      g.e_out = a.e + F.off;
+      g.coef = a.coef + F.coef_off;
+    }
+    g.nx = F.nx; g.ny = F.ny; g.nz = F.nz; g.crz = F.crz; g.ncz = C.nz;
+    g.seq = C.ncell > kSmallTransfer;
+    return g;
+  };
   for (int l = l0; l < lt; ++l) {
     const int ks = l == 0 ? FERROX_K_SMOOTH0 : FERROX_K_SMOOTHC;
     const double sb = sweep_bytes<T>(c, c->lv[l]);
+    if (leg_at(c, l)) {
+      wrap(l == 0 ? FERROX_K_SMOOTH0 : FERROX_K_RESTRICT, leg_bytes(c, l, true, first, fold),
+           [&] { launch_leg_down(leg_args(l), s); });
+      continue;
+    }
     if (rb_sweeps<T>(c, l, nu1)) {
       T* own = a.e + c->lv[l].off;
       for (int sw = 0; sw < nu1; ++sw) {
@@ -562,9 +609,13 @@ void enqueue_levels(ferrox_ctx* c, cudaStream_t s, W wrap, int l0, bool first, b
     for (int l = lt; l <= L; ++l) tb += 2.0 * (double)c->lv[l].ncell * sizeof(T);
     wrap(FERROX_K_TAIL, tb, [&] { launch_tail<T>(a, ta, c->tail_smem, s); });
   }
-  const UpdateArgs upd{c->phi, c->stats_d, update_clamp(c)};
   for (int l = lt - 1; l >= l0; --l) {
     const int ks = l == 0 ? FERROX_K_SMOOTH0 : FERROX_K_SMOOTHC;
+    if (leg_at(c, l)) {
+      wrap(l == 0 ? FERROX_K_SMOOTH0 : FERROX_K_PROLONG, leg_bytes(c, l, false, first, fold),
+           [&] { launch_leg_up(leg_args(l), l == 0 && fold ? &upd : nullptr, s); });
+      continue;
+    }
     // the tiled form where FP64 arithmetic bounds the launch: the fine level
     const bool tiled = sizeof(T) == sizeof(double) && l == 0;
     wrap(FERROX_K_PROLONG, prolong_bytes<T>(c->lv[l], c->lv[l + 1]),
@@ -696,7 +747,7 @@ bool separate_update(const ferrox_ctx* c) {
 int vcycle_launches(const ferrox_ctx* c) {
   int n = 1;   // the tail or the dense bottom solve
   for (int l = 0; l < c->tail_first; ++l)
-    n += smoothing_launches(c, l, c->num.nu1) + 1 + 1 + smoothing_launches(c, l, c->num.nu2);
+    n += leg_at(c, l) ? 2 : smoothing_launches(c, l, c->num.nu1) + 1 + 1 + smoothing_launches(c, l, c->num.nu2);
   return n;
 }
 
@@ -1184,7 +1235,7 @@ void release(ferrox_ctx* c) {
   cudaGraph_t gr[4] = {c->gr_step, c->gr_solve, c->gr_tdgl, c->gr_step_nn};
   for (auto g : ge) if (g) cudaGraphExecDestroy(g);
   for (auto g : gr) if (g) cudaGraphDestroy(g);
-  void* ptrs[] = {c->b, c->Pbuf, c->Fbuf, c->phi_prev, c->e_arena, c->e_alt, c->r_arena, c->s_arena, c->coef, c->coef0, c->coef0s, c->bs, c->sinv0, c->coef_df,
+  void* ptrs[] = {c->b, c->Pbuf, c->Fbuf, c->phi_prev, c->e_arena, c->eb_arena, c->e_alt, c->r_arena, c->s_arena, c->coef, c->coef0, c->coef0s, c->bs, c->sinv0, c->coef_df,
                   c->planes_d, c->planes_f32_d, c->lv_d, c->lvt_d, c->nn_scale, c->phi_guess, c->nn_pf, c->nn_stats, c->params_d, c->stats_d, c->partials_d, c->charge_d,
                   c->charge_part_d, c->dense_d, c->dense_wide_d};
   for (void* p : ptrs) if (p) cudaFree(p);
@@ -1319,14 +1370,19 @@ ferrox_status ferrox_init_geometry(ferrox_ctx** out, const ferrox_geometry* geom
     FX_INIT_CK(cudaMemset(ctx->phi_prev, 0, N * sizeof(double)));
   }
   FX_INIT_CK(cudaMalloc(&ctx->e_arena, ctx->arena * tsz));
-  // FERROX_RB_SWEEPS=0 in the environment keeps the colour-by-colour sweeps
+  // FERROX_RB_SWEEPS=0 in the environment keeps the colour-by-colour launches
   // (same results; for comparing the two paths)
   const char* rb_env = std::getenv("FERROX_RB_SWEEPS");
+  ctx->legs = mixed && ctx->num.nu1 == 2 && ctx->num.nu2 == 2 && !(rb_env && rb_env[0] == '0');
+  if (ctx->legs) {
+    FX_INIT_CK(cudaMalloc(&ctx->eb_arena, (ctx->arena / 2 + 32) * sizeof(float)));
+    FX_INIT_CK(leg_prepare());
+  }
   if (mixed && !(rb_env && rb_env[0] == '0')) {
     // the fused red-black sweeps alternate between a level's array and e_alt
     long long alt = 0;
     for (int l = 0; l < ctx->tail_first; ++l)
-      if (smooth_rb_tile<float>(ctx->lv[l], ctx->shift) > 0) alt = std::max(alt, ctx->lv[l].ncell);
+      if (!leg_at(ctx, l) && smooth_rb_tile<float>(ctx->lv[l], ctx->shift) > 0) alt = std::max(alt, ctx->lv[l].ncell);
     if (alt > 0) {
       FX_INIT_CK(cudaMalloc(&ctx->e_alt, alt * tsz));
       FX_INIT_CK(smooth_rb_prepare<float>());
@@ -1334,7 +1390,7 @@ ferrox_status ferrox_init_geometry(ferrox_ctx** out, const ferrox_geometry* geom
   }
   FX_INIT_CK(cudaMalloc(&ctx->r_arena, ctx->arena * tsz));
   if (ctx->shift) FX_INIT_CK(cudaMalloc(&ctx->s_arena, ctx->arena * tsz));
-  if (ctx->shift) FX_INIT_CK(cudaMalloc(&ctx->sinv0, ctx->lv[0].ncell * tsz));
+  if (ctx->shift) FX_INIT_CK(cudaMalloc(&ctx->sinv0, (ctx->legs ? ctx->arena : ctx->lv[0].ncell) * tsz));
   FX_INIT_CK(cudaMalloc(&ctx->planes_d, ctx->nz * sizeof(PlaneTDGL)));
   FX_INIT_CK(cudaMalloc(&ctx->lv_d, ctx->lv.size() * sizeof(LevelDesc)));
   FX_INIT_CK(cudaMalloc(&ctx->params_d, sizeof(DevParams)));

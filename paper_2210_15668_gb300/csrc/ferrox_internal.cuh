@@ -55,6 +55,12 @@ constexpr int kDenseWide = 512;         // a first tail level up to this size (s
                                         // carriers) is solved by its inverse across the SMs
                                         // instead of the tail V-cycle
 constexpr int kTailMaxSmem = 200 * 1024; // shared memory available to the tail CTA
+// Latency-bound FP32 levels: the per-thread chains of the one-thread-per-coarse-
+// cell transfers dominate up to this size.  Measured on 256x256x32, 500 steps
+// (Mcell-steps/s, mixed / fast form): none 1781 / 2735, up to 4096 cells
+// 1799 / 2761, up to 32768 cells 1804 / 2775; larger FP32 levels lose.  FP64
+// levels use the split kernels at every size (+2.2% FP64).
+constexpr long long kSmallTransfer = 32768;
 constexpr int kResidBX = 32, kResidBY = 8; // residual: one thread per (x, y) column
 constexpr int kTdglTileX = 32, kTdglTileY = 2, kTdglChunks = 4;  // batched TDGL: column tile, z chunks
 
@@ -248,6 +254,33 @@ void launch_scale_rhs(const double* b, const PlaneCoef<double>* coef, int nx, in
 template <typename T>
 void launch_smooth_rb(const MGArgs<T>& a, const LevelDesc& L, const T* e_in, T* e_out,
                       int zero_init, const UpdateArgs* upd, cudaStream_t s);
+// One leg of a V-cycle on one FP32 level (leg_device.cuh); all arrays start at the
+// level's (coarse level's) first cell.
+struct LegArgs {
+  const float* r;           // right-hand side
+  const float* s;           // Newton shift (null without)
+  const float* sinv;        // 1 / (diag + s)
+  const float* e_in;        // down: starting corrections (null: zero)
+  float* eb;                // black corrections between the legs: [nz][ny][nx / 2]
+  float* rc;                // down: coarse right-hand side ...
+  float* sc;                // ... and coarse shift (null: keep) ...
+  float* sinvc;             // ... and 1 / (diag + s) there (null where no leg reads it)
+  const PlaneCoef<float>* coefc;  // the coarse level's planes
+  const float* ec;          // up: coarse corrections
+  float* e_out;             // up: corrections of the level (when phi is not updated)
+  const PlaneCoef<float>* coef;
+  int nx, ny, nz, crz;      // crz: the level is coarsened in z too (always in x and y)
+  int ncz;                  // planes of the coarse level
+  int kz;                   // planes per block (even)
+  int phi_vec;              // up: phi is 16-byte aligned
+  int seq;                  // down: the children are summed one after another (restrict_kernel's
+                            // order), else as four columns (restrict4_kernel's)
+};
+// whether a level takes the legs: FP32 with two sweeps each way, coarsened in x and y
+bool leg_level(const LevelDesc& L);
+cudaError_t leg_prepare();
+void launch_leg_down(const LegArgs& a, cudaStream_t s);
+void launch_leg_up(const LegArgs& a, const UpdateArgs* upd, cudaStream_t s);
 dim3 check_grid(const LevelDesc& C);
 void launch_restrict_check(const MGArgs<double>& fa, double* rc, const LevelDesc& F,
                            const LevelDesc& C, int nu1, const CheckArgs& ck, cudaStream_t s);

@@ -1,0 +1,151 @@
+// Launches of the V-cycle legs of leg_device.cuh on one device stack.
+#include <cuda_runtime.h>
+#include <math.h>
+
+#include <algorithm>
+
+#include "ferrox_internal.cuh"
+#include "leg_device.cuh"
+
+namespace fx {
+
+namespace {
+
+using namespace dev;
+
+// Blocks per SM the register allocation has to allow: with a Newton shift 16 warps
+// (128 registers instead of 130 to 150, one 240-thread block per SM otherwise); without
+// one the kernels keep the 72 to 124 registers they ask for (80 forced: 256x256x32
+// mixed step 5.65 -> 6.14 ms for five solves)
+constexpr int min_blocks(int threads, bool sc) {
+  const int w = (threads + 31) / 32;
+  return sc && w < 16 ? 16 / w : 1;
+}
+
+template <int TX, int TY, bool SC, bool CONT>
+__global__ void __launch_bounds__(LegDown<TX, TY, SC, CONT>::G::THREADS, min_blocks(LegDown<TX, TY, SC, CONT>::G::THREADS, SC)) leg_down_kernel(LegArgs a) {
+  extern __shared__ __align__(16) unsigned char leg_smem[];
+  pdl_enter();
+  LegDown<TX, TY, SC, CONT>::run(a, blockIdx.x, blockIdx.y, blockIdx.z, leg_smem);
+}
+
+template <int TX, int TY, bool SC, bool PHI>
+__global__ void __launch_bounds__(LegUp<TX, TY, SC, PHI>::G::THREADS, min_blocks(LegUp<TX, TY, SC, PHI>::G::THREADS, SC)) leg_up_kernel(LegArgs a, Upd u, const DevStats* st) {
+  extern __shared__ __align__(16) unsigned char leg_smem[];
+  pdl_enter();
+  if (PHI) u.zero = st->zero_phi;
+  LegUp<TX, TY, SC, PHI>::run(a, u, blockIdx.x, blockIdx.y, blockIdx.z, leg_smem);
+}
+
+struct Plan {
+  int tile, kz;
+};
+
+#ifdef FX_LEG_BENCH
+Plan g_plan;
+Plan leg_plan(const LegArgs&, bool) { return g_plan; }
+#else
+// Tile and planes per block by the level's size, from the legs timed one by one in a
+// graph (us, down / up; tile/kz): small levels want blocks on every SM more than they
+// mind the recomputed halo,
+//   32x32x4      16x16/2 2.9 / 4.4, 32x16/4 3.4 / 4.7        64x64x8  16x16/2 3.5 / 5.6, 32x16/4 4.4 / 6.5
+//   128x128x16   32x16/4 4.6 / 7.5, 16x16/4 5.2 / 7.7, 32x16/16 6.6 / 9.7,
+// large ones the smaller halo share of long columns,
+//   256x256x32   32x16/32 11.4 / 18.0, 32x16/16 12.3 / 16.8, 32x16/8 15.5 / 22.8
+//   512x512x128 (shift)  32x16/128 297 / 217, 32x16/32 287 / 232, 32x16/16 325 / 281,
+// and with a shift the down leg that continues a correction (six registers more per
+// cell) the larger tile: 256x256x64 32x32/32 37, 32x16/32 50.
+Plan leg_plan(const LegArgs& a, bool wide) {
+  const long long cells = (long long)a.nx * a.ny * a.nz;
+  if (cells < (1 << 17)) return {2, 2};
+  if (cells < (1 << 20)) return {1, 4};
+  const long long tiles = (long long)((a.nx + 31) / 32) * ((a.ny + 15) / 16);
+  int kz = 32;
+  while (kz < 128 && tiles * ((a.nz + kz - 1) / kz) > 600) kz *= 2;
+  return {wide ? 0 : 1, kz};
+}
+#endif
+
+template <int TX, int TY>
+dim3 leg_grid(const LegArgs& a) {
+  return dim3((a.nx + TX - 1) / TX, (a.ny + TY - 1) / TY, (a.nz + a.kz - 1) / a.kz);
+}
+
+template <int TX, int TY, bool SC, bool CONT>
+void down(const LegArgs& a, cudaStream_t s) {
+  using K = LegDown<TX, TY, SC, CONT>;
+  launch_k(leg_down_kernel<TX, TY, SC, CONT>, leg_grid<TX, TY>(a), dim3(K::G::THREADS), K::smem_bytes(a.kz), s, a);
+}
+
+template <int TX, int TY, bool SC, bool PHI>
+void up(const LegArgs& a, const UpdateArgs* upd, cudaStream_t s) {
+  using K = LegUp<TX, TY, SC, PHI>;
+  Upd u{nullptr, 0.0, 0, 0.0f};
+  const DevStats* st = nullptr;
+  if (upd) { u.phi = upd->phi; u.clamp = upd->clamp; u.clampf = (float)upd->clamp; st = upd->stats; }
+  launch_k(leg_up_kernel<TX, TY, SC, PHI>, leg_grid<TX, TY>(a), dim3(K::G::THREADS), K::smem_bytes(a.kz), s, a, u, st);
+}
+
+template <int TX, int TY>
+cudaError_t prepare_tile() {
+  const int lim = 227 * 1024;
+  const cudaFuncAttribute m = cudaFuncAttributeMaxDynamicSharedMemorySize;
+  cudaError_t e = cudaSuccess;
+  auto set = [&](const void* f) {
+    const cudaError_t r = cudaFuncSetAttribute(f, m, lim);
+    if (e == cudaSuccess) e = r;
+  };
+  set((const void*)leg_down_kernel<TX, TY, false, false>);
+  set((const void*)leg_down_kernel<TX, TY, false, true>);
+  set((const void*)leg_down_kernel<TX, TY, true, false>);
+  set((const void*)leg_down_kernel<TX, TY, true, true>);
+  set((const void*)leg_up_kernel<TX, TY, false, false>);
+  set((const void*)leg_up_kernel<TX, TY, false, true>);
+  set((const void*)leg_up_kernel<TX, TY, true, false>);
+  set((const void*)leg_up_kernel<TX, TY, true, true>);
+  return e;
+}
+
+template <int TX, int TY>
+void down_tile(const LegArgs& a, cudaStream_t s) {
+  if (a.s) a.e_in ? down<TX, TY, true, true>(a, s) : down<TX, TY, true, false>(a, s);
+  else a.e_in ? down<TX, TY, false, true>(a, s) : down<TX, TY, false, false>(a, s);
+}
+
+template <int TX, int TY>
+void up_tile(const LegArgs& a, const UpdateArgs* upd, cudaStream_t s) {
+  if (a.s) upd ? up<TX, TY, true, true>(a, upd, s) : up<TX, TY, true, false>(a, upd, s);
+  else upd ? up<TX, TY, false, true>(a, upd, s) : up<TX, TY, false, false>(a, upd, s);
+}
+
+}  // namespace
+
+bool leg_level(const LevelDesc& L) { return L.crx && L.cry && !(L.nx & 1) && !(L.ny & 1); }
+
+cudaError_t leg_prepare() {
+  cudaError_t e;
+  if ((e = prepare_tile<32, 32>()) != cudaSuccess) return e;
+  if ((e = prepare_tile<32, 16>()) != cudaSuccess) return e;
+  return prepare_tile<16, 16>();
+}
+
+void launch_leg_down(const LegArgs& a_in, cudaStream_t s) {
+  LegArgs a = a_in;
+  const Plan p = leg_plan(a, a.s && a.e_in);
+  a.kz = std::min(p.kz, a.nz + (a.nz & 1));
+  if (p.tile == 0) down_tile<32, 32>(a, s);
+  else if (p.tile == 1) down_tile<32, 16>(a, s);
+  else down_tile<16, 16>(a, s);
+}
+
+void launch_leg_up(const LegArgs& a_in, const UpdateArgs* upd, cudaStream_t s) {
+  LegArgs a = a_in;
+  const Plan p = leg_plan(a, false);
+  a.kz = std::min(p.kz, a.nz + (a.nz & 1));
+  a.phi_vec = upd && reinterpret_cast<uintptr_t>(upd->phi) % 16 == 0;
+  if (p.tile == 0) up_tile<32, 32>(a, upd, s);
+  else if (p.tile == 1) up_tile<32, 16>(a, upd, s);
+  else up_tile<16, 16>(a, upd, s);
+}
+
+}  // namespace fx

@@ -39,6 +39,14 @@ __device__ __forceinline__ T gs_numerator(const T* e, const T* r, const PlaneCoe
   return acc;
 }
 
+// a numerator over the shifted diagonal d = diag + s; in FP32 by the reciprocal, as
+// level 0 does with its stored 1 / (diag + s) and the V-cycle legs at every level
+template <typename T>
+__device__ __forceinline__ T over_shifted(T num, T d) {
+  if constexpr (sizeof(T) == sizeof(float)) return num * (T(1) / d);
+  else return num / d;
+}
+
 struct Upd {
   double* phi;      // fine-level potential (null: no fused update)
   double clamp;     // |e| limit of one update (infinite without carriers)
@@ -81,7 +89,7 @@ __device__ __forceinline__ void smooth_pair(const MGArgs<T>& a, const LevelDesc&
       ev = a.r[id] * d;
     } else {
       const T num = gs_numerator(a.e, a.r, c, L, i, j, k, id);
-      ev = c.has_s ? (a.sinv ? num * a.sinv[id - L.off] : num / (c.diag + a.s[id])) : num * c.invdiag;
+      ev = c.has_s ? (a.sinv ? num * a.sinv[id - L.off] : over_shifted<T>(num, c.diag + a.s[id])) : num * c.invdiag;
     }
     a.e[id] = ev;
   }

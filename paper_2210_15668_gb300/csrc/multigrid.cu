@@ -108,7 +108,7 @@ __global__ void __launch_bounds__(256) smooth_kz_kernel(MGArgs<T> a, LevelDesc L
     acc = fma(c[q].czhi, v[q][6], acc);
     if constexpr (SCALED) a.e[id] = acc;
     else if (!c[q].has_s) a.e[id] = acc * c[q].invdiag;
-    else a.e[id] = a.sinv ? acc * a.sinv[id - L.off] : acc / (c[q].diag + a.s[id]);
+    else a.e[id] = a.sinv ? acc * a.sinv[id - L.off] : over_shifted<T>(acc, c[q].diag + a.s[id]);
   }
 }
 
@@ -276,7 +276,7 @@ __global__ void __launch_bounds__(256) smooth_rb_kernel(RBArgs<float> a) {
           acc = fmaf(c.cy, Ec[e - kRbW] + Ec[e + kRbW], acc);
           acc = fmaf(c.czlo, Ed[e], acc);
           acc = fmaf(c.czhi, Eu[e], acc);
-          ev = c.has_s ? (a.sinv ? acc * S[q] : acc / (c.diag + S[q])) : acc * c.invdiag;
+          ev = c.has_s ? (a.sinv ? acc * S[q] : over_shifted(acc, c.diag + S[q])) : acc * c.invdiag;
         }
         R[q] = ev;
       }
@@ -298,7 +298,7 @@ __global__ void __launch_bounds__(256) smooth_rb_kernel(RBArgs<float> a) {
       acc = fmaf(c.cy, Rc[qb - kRbW] + Rc[qb + kRbW], acc);
       acc = fmaf(c.czlo, Rd[qb], acc);
       acc = fmaf(c.czhi, Ru[qb], acc);
-      const float eb = c.has_s ? (a.sinv ? acc * S[qb] : acc / (c.diag + S[qb])) : acc * c.invdiag;
+      const float eb = c.has_s ? (a.sinv ? acc * S[qb] : over_shifted(acc, c.diag + S[qb])) : acc * c.invdiag;
       const float er = Rc[q0 + 1 - second];
       const int id = pb * plane + gy_b * nx + x0 + 2 * bk;
       const float2 v = second ? make_float2(er, eb) : make_float2(eb, er);
@@ -789,13 +789,6 @@ void launch_restrict_check(const MGArgs<double>& fa, double* rc, const LevelDesc
   launch_k(restrict_check_kernel<double>, grid, block, 0, s, fa, rc, F, C,
            black_residual_zero(F, nu1), ck);
 }
-
-// Latency-bound FP32 levels: the per-thread chains of the one-thread-per-coarse-
-// cell transfers dominate up to this size.  Measured on 256x256x32, 500 steps
-// (Mcell-steps/s, mixed / fast form): none 1781 / 2735, up to 4096 cells
-// 1799 / 2761, up to 32768 cells 1804 / 2775; larger FP32 levels lose.  FP64
-// levels use the split kernels at every size (+2.2% FP64).
-constexpr long long kSmallTransfer = 32768;
 
 template <typename T>
 void launch_restrict(const MGArgs<T>& a, const LevelDesc& F, const LevelDesc& C, int nu1,

@@ -228,7 +228,7 @@ __device__ __forceinline__ void smooth_rows(const MGArgs<T>& a, const LevelDesc&
         const T d = cf.has_s ? (a.sinv ? a.sinv[t - L.off] : T(1) / (cf.diag + sv[rr])) : cf.invdiag;
         ev = num[rr] * d;
       } else {
-        ev = cf.has_s ? (a.sinv ? num[rr] * a.sinv[t - L.off] : num[rr] / (cf.diag + sv[rr]))
+        ev = cf.has_s ? (a.sinv ? num[rr] * a.sinv[t - L.off] : over_shifted<T>(num[rr], cf.diag + sv[rr]))
                       : num[rr] * cf.invdiag;
       }
       a.e[t] = ev;
