@@ -1848,6 +1848,10 @@ struct ferrox_batch {
   void* r = nullptr;
   void* s = nullptr;
   void* coef = nullptr;
+  float* eb = nullptr;                // FP32 legs: black corrections, 1 / (diag + s), block prefixes
+  float* sinv = nullptr;
+  int* leg_pre = nullptr;
+  int leg_blocks[kMaxLegLevels] = {}, leg_tile[kMaxLegLevels] = {}, leg_kz[kMaxLegLevels] = {};
   void* dense = nullptr;              // T: inverses of the instances' dense tail levels
   PlaneCoef<double>* coef0 = nullptr;
   PlaneTDGL* planes = nullptr;
@@ -1941,6 +1945,12 @@ BatchArgs batch_args(ferrox_batch* B, int mode) {
   a.ticket = B->ticket;
   a.tile_pre = B->tile_pre;
   a.ntiles = B->ntiles;
+  a.eb = B->eb; a.sinv = B->sinv; a.leg_pre = B->leg_pre;
+  for (int l = 0; l < kMaxLegLevels; ++l) {
+    a.leg_blocks[l] = B->leg_blocks[l];
+    a.leg_tile[l] = B->leg_tile[l];
+    a.leg_kz[l] = B->leg_kz[l];
+  }
   return a;
 }
 
@@ -2204,7 +2214,7 @@ void batch_release(ferrox_batch* B) {
   if (B->ge_solve) cudaGraphExecDestroy(B->ge_solve);
   if (B->gr_step) cudaGraphDestroy(B->gr_step);
   if (B->gr_solve) cudaGraphDestroy(B->gr_solve);
-  void* ptrs[] = {B->b, B->Pbuf, B->backup, B->e, B->r, B->s, B->coef, B->dense, B->coef0, B->planes, B->lv,
+  void* ptrs[] = {B->b, B->Pbuf, B->backup, B->e, B->r, B->s, B->eb, B->sinv, B->leg_pre, B->coef, B->dense, B->coef0, B->planes, B->lv,
                   B->lvt, B->pre, B->partials, B->active, B->bar, B->grp_d, B->status, B->ticket, B->tile_pre, B->any_d, B->nsteps_d, B->dbg, B->params,
                   B->stats, B->inst, B->charge_part, B->charge_out};
   for (void* p : ptrs) if (p) cudaFree(p);
@@ -2340,6 +2350,44 @@ ferrox_status ferrox_init_batch(ferrox_batch** out, int n, const ferrox_geometry
     FX_BINIT(cudaMalloc(&B->tile_pre, (n + 1) * sizeof(int)));
     FX_BINIT(cudaMemcpy(B->tile_pre, tp.data(), (n + 1) * sizeof(int), cudaMemcpyHostToDevice));
   }
+  if (B->mixed && num->nu1 == 2 && num->nu2 == 2) {
+    // levels every instance that holds them can take as legs (the graph engine)
+    const int nl = std::min(B->Ldown, kMaxLegLevels);
+    std::vector<int> lp((size_t)std::max(1, nl) * (n + 1), 0);
+    for (int l = 0; l < nl; ++l) {
+      long long total = 0;
+      int nx = 0, ny = 0, nz = 0;
+      bool ok = true;
+      for (const auto& p : B->plans) {
+        if (l >= p.c.tail_first) continue;
+        const LevelDesc& L = p.c.lv[l];
+        ok = ok && leg_level(L);
+        total += L.ncell;
+        nx = std::max(nx, L.nx); ny = std::max(ny, L.ny); nz = std::max(nz, L.nz);
+      }
+      if (!ok) break;   // the levels below can halve no more than this one
+      const LegPlan lpl = leg_plan(total, nx, ny, nz, false);
+      const int tw = lpl.tile == kLegTile16x16 ? 16 : 32;
+      B->leg_tile[l] = lpl.tile;
+      B->leg_kz[l] = std::min(lpl.kz, nz + (nz & 1));
+      for (int i = 0; i < n; ++i) {
+        const ferrox_ctx& c = B->plans[i].c;
+        int blocks = 0;
+        if (l < c.tail_first) {
+          const LevelDesc& L = c.lv[l];
+          blocks = ((L.nx + tw - 1) / tw) * ((L.ny + 15) / 16) * ((L.nz + B->leg_kz[l] - 1) / B->leg_kz[l]);
+        }
+        lp[(size_t)l * (n + 1) + i + 1] = lp[(size_t)l * (n + 1) + i] + blocks;
+      }
+      B->leg_blocks[l] = lp[(size_t)l * (n + 1) + n];
+    }
+    if (nl > 0 && B->leg_blocks[0] > 0) {
+      FX_BINIT(cudaMalloc(&B->eb, (arena / 2 + 32) * sizeof(float)));
+      if (has_sc) FX_BINIT(cudaMalloc(&B->sinv, arena * sizeof(float)));
+      FX_BINIT(cudaMalloc(&B->leg_pre, lp.size() * sizeof(int)));
+      FX_BINIT(cudaMemcpy(B->leg_pre, lp.data(), lp.size() * sizeof(int), cudaMemcpyHostToDevice));
+    }
+  }
   FX_BINIT(cudaMalloc(&B->nsteps_d, sizeof(int)));
   FX_BINIT(cudaMalloc(&B->dbg, (8 + 1024) * sizeof(int)));
   FX_BINIT(cudaMemset(B->dbg, 0, (8 + 1024) * sizeof(int)));
@@ -2405,6 +2453,7 @@ ferrox_status ferrox_init_batch(ferrox_batch** out, int n, const ferrox_geometry
     ra.nx = c.nx; ra.ny = c.ny; ra.nz = c.nz;
     ra.r_out = static_cast<char*>(B->r) + (size_t)p.arena_off * tsz;
     ra.s_out = has_sc && c.has_sc ? static_cast<char*>(B->s) + (size_t)p.arena_off * tsz : nullptr;
+    ra.sinv_out = ra.s_out && B->sinv ? B->sinv + p.arena_off : nullptr;
     ra.carriers = carrier_kind(&c);
     // FP64 residual: measured, the double-float form is slower in the batched
     // residual, whose columns give too few threads to hide its longer chains (64

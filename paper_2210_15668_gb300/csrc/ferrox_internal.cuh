@@ -47,6 +47,7 @@ inline cudaError_t launch_k(void (*kern)(K...), dim3 grid, dim3 block, size_t sm
 }
 
 constexpr int kMaxLevels = 24;
+constexpr int kMaxLegLevels = 8;        // batched levels that may run as legs
 constexpr int kTailMaxCells = 4096;     // levels at or below this size run in one CTA (FP32)
 constexpr int kTailMaxCellsFP64 = 512;  // the same for FP64 corrections
 constexpr int kTailThreads = 1024;
@@ -278,6 +279,13 @@ struct LegArgs {
 };
 // whether a level takes the legs: FP32 with two sweeps each way, coarsened in x and y
 bool leg_level(const LevelDesc& L);
+enum { kLegTile32x32 = 0, kLegTile32x16 = 1, kLegTile16x16 = 2 };
+// lateral tile and planes per block for a level, or for `cells` in all of several levels
+// in one launch; wide: the down leg that continues a correction with a shift
+struct LegPlan {
+  int tile, kz;
+};
+LegPlan leg_plan(long long cells, int nx, int ny, int nz, bool wide);
 cudaError_t leg_prepare();
 void launch_leg_down(const LegArgs& a, cudaStream_t s);
 void launch_leg_up(const LegArgs& a, const UpdateArgs* upd, cudaStream_t s);
@@ -459,6 +467,13 @@ struct BatchArgs {
   int max_cycles, nu1, nu2, rows_per_unit, any_full_tail, pad;
   int* dbg;             // optional self-check record (null: off)
   unsigned int* ticket; // graph engine: blocks of the decision kernel done (0 between launches)
+  // graph engine, FP32 with two sweeps each way: levels that run as V-cycle legs
+  float* eb;            // black corrections between the legs (half an arena; null: no legs)
+  float* sinv;          // 1 / (diag + s) arena (with semiconductor instances)
+  const int* leg_pre;   // per leg level: prefix of its blocks per instance
+  int leg_blocks[kMaxLegLevels];  // per level: blocks in all (0: colour sweeps and transfers)
+  int leg_tile[kMaxLegLevels];    // ... lateral tile (kLegTile*)
+  int leg_kz[kMaxLegLevels];      // ... planes per block
   int* any_out;         // eager phase replay: "any instance active" after each decision (else null)
 };
 

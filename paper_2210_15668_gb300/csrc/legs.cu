@@ -9,62 +9,28 @@
 
 namespace fx {
 
+#ifdef FX_LEG_BENCH
+LegPlan g_plan;
+#endif
+
 namespace {
 
 using namespace dev;
 
-// Blocks per SM the register allocation has to allow: with a Newton shift 16 warps
-// (128 registers instead of 130 to 150, one 240-thread block per SM otherwise); without
-// one the kernels keep the 72 to 124 registers they ask for (80 forced: 256x256x32
-// mixed step 5.65 -> 6.14 ms for five solves)
-constexpr int min_blocks(int threads, bool sc) {
-  const int w = (threads + 31) / 32;
-  return sc && w < 16 ? 16 / w : 1;
-}
-
 template <int TX, int TY, bool SC, bool CONT>
-__global__ void __launch_bounds__(LegDown<TX, TY, SC, CONT>::G::THREADS, min_blocks(LegDown<TX, TY, SC, CONT>::G::THREADS, SC)) leg_down_kernel(LegArgs a) {
+__global__ void __launch_bounds__(LegDown<TX, TY, SC, CONT>::G::THREADS, leg_min_blocks(LegDown<TX, TY, SC, CONT>::G::THREADS, SC)) leg_down_kernel(LegArgs a) {
   extern __shared__ __align__(16) unsigned char leg_smem[];
   pdl_enter();
   LegDown<TX, TY, SC, CONT>::run(a, blockIdx.x, blockIdx.y, blockIdx.z, leg_smem);
 }
 
 template <int TX, int TY, bool SC, bool PHI>
-__global__ void __launch_bounds__(LegUp<TX, TY, SC, PHI>::G::THREADS, min_blocks(LegUp<TX, TY, SC, PHI>::G::THREADS, SC)) leg_up_kernel(LegArgs a, Upd u, const DevStats* st) {
+__global__ void __launch_bounds__(LegUp<TX, TY, SC, PHI>::G::THREADS, leg_min_blocks(LegUp<TX, TY, SC, PHI>::G::THREADS, SC)) leg_up_kernel(LegArgs a, Upd u, const DevStats* st) {
   extern __shared__ __align__(16) unsigned char leg_smem[];
   pdl_enter();
   if (PHI) u.zero = st->zero_phi;
   LegUp<TX, TY, SC, PHI>::run(a, u, blockIdx.x, blockIdx.y, blockIdx.z, leg_smem);
 }
-
-struct Plan {
-  int tile, kz;
-};
-
-#ifdef FX_LEG_BENCH
-Plan g_plan;
-Plan leg_plan(const LegArgs&, bool) { return g_plan; }
-#else
-// Tile and planes per block by the level's size, from the legs timed one by one in a
-// graph (us, down / up; tile/kz): small levels want blocks on every SM more than they
-// mind the recomputed halo,
-//   32x32x4      16x16/2 2.9 / 4.4, 32x16/4 3.4 / 4.7        64x64x8  16x16/2 3.5 / 5.6, 32x16/4 4.4 / 6.5
-//   128x128x16   32x16/4 4.6 / 7.5, 16x16/4 5.2 / 7.7, 32x16/16 6.6 / 9.7,
-// large ones the smaller halo share of long columns,
-//   256x256x32   32x16/32 11.4 / 18.0, 32x16/16 12.3 / 16.8, 32x16/8 15.5 / 22.8
-//   512x512x128 (shift)  32x16/128 297 / 217, 32x16/32 287 / 232, 32x16/16 325 / 281,
-// and with a shift the down leg that continues a correction (six registers more per
-// cell) the larger tile: 256x256x64 32x32/32 37, 32x16/32 50.
-Plan leg_plan(const LegArgs& a, bool wide) {
-  const long long cells = (long long)a.nx * a.ny * a.nz;
-  if (cells < (1 << 17)) return {2, 2};
-  if (cells < (1 << 20)) return {1, 4};
-  const long long tiles = (long long)((a.nx + 31) / 32) * ((a.ny + 15) / 16);
-  int kz = 32;
-  while (kz < 128 && tiles * ((a.nz + kz - 1) / kz) > 600) kz *= 2;
-  return {wide ? 0 : 1, kz};
-}
-#endif
 
 template <int TX, int TY>
 dim3 leg_grid(const LegArgs& a) {
@@ -120,6 +86,28 @@ void up_tile(const LegArgs& a, const UpdateArgs* upd, cudaStream_t s) {
 
 }  // namespace
 
+// Tile and planes per block by the level's size, from the legs timed one by one in a
+// graph (us, down / up; tile/kz): small levels want blocks on every SM more than they
+// mind the recomputed halo,
+//   32x32x4      16x16/2 2.9 / 4.4, 32x16/4 3.4 / 4.7        64x64x8  16x16/2 3.5 / 5.6, 32x16/4 4.4 / 6.5
+//   128x128x16   32x16/4 4.6 / 7.5, 16x16/4 5.2 / 7.7, 32x16/16 6.6 / 9.7,
+// large ones the smaller halo share of long columns,
+//   256x256x32   32x16/32 11.4 / 18.0, 32x16/16 12.3 / 16.8, 32x16/8 15.5 / 22.8
+//   512x512x128 (shift)  32x16/128 297 / 217, 32x16/32 287 / 232, 32x16/16 325 / 281,
+// and with a shift the down leg that continues a correction (six registers more per
+// cell) the larger tile: 256x256x64 32x32/32 37, 32x16/32 50.
+LegPlan leg_plan(long long cells, int nx, int ny, int nz, bool wide) {
+#ifdef FX_LEG_BENCH
+  return g_plan;
+#endif
+  if (cells < (1 << 17)) return {kLegTile16x16, 2};
+  if (cells < (1 << 20)) return {kLegTile32x16, 4};
+  const long long tiles = (long long)((nx + 31) / 32) * ((ny + 15) / 16);
+  int kz = 32;
+  while (kz < 128 && tiles * ((nz + kz - 1) / kz) > 600) kz *= 2;
+  return {wide ? kLegTile32x32 : kLegTile32x16, kz};
+}
+
 bool leg_level(const LevelDesc& L) { return L.crx && L.cry && !(L.nx & 1) && !(L.ny & 1); }
 
 cudaError_t leg_prepare() {
@@ -131,20 +119,20 @@ cudaError_t leg_prepare() {
 
 void launch_leg_down(const LegArgs& a_in, cudaStream_t s) {
   LegArgs a = a_in;
-  const Plan p = leg_plan(a, a.s && a.e_in);
+  const LegPlan p = leg_plan((long long)a.nx * a.ny * a.nz, a.nx, a.ny, a.nz, a.s && a.e_in);
   a.kz = std::min(p.kz, a.nz + (a.nz & 1));
-  if (p.tile == 0) down_tile<32, 32>(a, s);
-  else if (p.tile == 1) down_tile<32, 16>(a, s);
+  if (p.tile == kLegTile32x32) down_tile<32, 32>(a, s);
+  else if (p.tile == kLegTile32x16) down_tile<32, 16>(a, s);
   else down_tile<16, 16>(a, s);
 }
 
 void launch_leg_up(const LegArgs& a_in, const UpdateArgs* upd, cudaStream_t s) {
   LegArgs a = a_in;
-  const Plan p = leg_plan(a, false);
+  const LegPlan p = leg_plan((long long)a.nx * a.ny * a.nz, a.nx, a.ny, a.nz, false);
   a.kz = std::min(p.kz, a.nz + (a.nz & 1));
   a.phi_vec = upd && reinterpret_cast<uintptr_t>(upd->phi) % 16 == 0;
-  if (p.tile == 0) up_tile<32, 32>(a, upd, s);
-  else if (p.tile == 1) up_tile<32, 16>(a, upd, s);
+  if (p.tile == kLegTile32x32) up_tile<32, 32>(a, upd, s);
+  else if (p.tile == kLegTile32x16) up_tile<32, 16>(a, upd, s);
   else up_tile<16, 16>(a, upd, s);
 }
 

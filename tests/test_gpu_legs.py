@@ -42,3 +42,25 @@ def test_legs_bit_identical(stack, shape, form, monkeypatch):
     assert np.array_equal(Pa, Pb) and np.array_equal(pa, pb)
     assert sa["vcycles"] == sb["vcycles"] and sa["cycles"] == sb["cycles"]
     assert sb["launches"] < sa["launches"]
+
+
+def test_batched_legs_equal_the_persistent_launch():
+    """The graph engine's legs against the persistent launch's colour sweeps: a batch with
+    and without carriers, with short, ragged and odd instances."""
+    from paper_2210_15668_gb300 import ferrox
+    geoms = [I.make_geometry(nx, ny, I.mfim_stack(nz, n_fe=4) if k == 0 else I.mfism_stack(nz, n_fe=3, n_ox=1))
+             for nx, ny, nz, k in [(64, 48, 16, 0), (36, 20, 9, 1), (112, 80, 14, 1), (16, 144, 12, 0), (96, 96, 21, 1)]]
+    P0 = [I.random_polarization(g, seed=40 + i, amp=0.05) for i, g in enumerate(geoms)]
+    out = []
+    for engine in (0, 1):
+        b = ferrox.Batch(geoms, P0, ferrox.make_numerics(4e-13, tol=1e-10, precision=ferrox.MIXED))
+        b.set_engine(engine)
+        b.set_bias(0.0, [0.5, -0.4, 0.2, 1.0, -0.1])
+        b.solve_poisson()
+        b.step(2)
+        out.append(([b.state(i) for i in range(len(geoms))], [s["cycles"] for s in b.stats()]))
+        b.close()
+    (sa, ca), (sb, cb) = out
+    assert ca == cb
+    for (Pa, pa), (Pb, pb) in zip(sa, sb):
+        assert np.array_equal(Pa, Pb) and np.array_equal(pa, pb)
