@@ -221,9 +221,10 @@ ferrox_status ferrox_charge(ferrox_ctx* ctx, ferrox_charge_t* out);
  * the finite-volume form, scaled by h^2/eps0) for the current state: b is formed
  * from the current P and bias, rho from the current Phi.  r_host is a host array
  * of Nz*Ny*Nx doubles.  arithmetic selects how the stencil is evaluated:
- * FERROX_RESID_FP64 (the FP64 forms' outer residual) or
- * FERROX_RESID_DOUBLE_FLOAT (the mixed form's outer residual: double-float pairs
- * on the FP32 pipe, about 48 significant bits; r = h + l).  A diagnostic: it
+ * FERROX_RESID_FP64 (the outer residual's stencil in every form) or
+ * FERROX_RESID_DOUBLE_FLOAT (double-float pairs on the FP32 pipe, about 48
+ * significant bits; r = h + l; the solves use this arithmetic for the mixed form's
+ * Boltzmann carriers only).  A diagnostic: it
  * allocates a device buffer, synchronises, and leaves the state unchanged (b is
  * recomputed from P, as every step does). */
 enum { FERROX_RESID_FP64 = 0, FERROX_RESID_DOUBLE_FLOAT = 1 };

@@ -91,7 +91,8 @@ struct ferrox_ctx {
   void* sinv0 = nullptr;               // 1 / (diag + s) on level 0 (T; with a Newton shift), with
                                        // legs on every level
   PlaneCoefDF* coef_df = nullptr;     // level 0 as double-float pairs (double-float residual)
-  bool df_resid = false;              // the mixed form's outer residual in double-float
+  PlaneCarrierDF* carriers_df = nullptr;
+  bool df_resid = false;              // the mixed form's Boltzmann carriers in double-float
   PlaneTDGL* planes_d = nullptr;
   PlaneF32* planes_f32_d = nullptr;   // FP32 TDGL arithmetic only
   LevelDesc* lv_d = nullptr;
@@ -436,13 +437,24 @@ double update_clamp(const ferrox_ctx* c) {
   return 10.0 * kKB * tmax / kQ;
 }
 
-// a plane's FP64 coefficients as double-float pairs: h = the nearest float, l = the
-// nearest float to the remainder
+// an FP64 value as a double-float pair: h = the nearest float, l = the nearest float to
+// the remainder
+void split(double x, float& h, float& l) {
+  h = (float)x;
+  l = (float)(x - (double)h);
+}
+
+PlaneCarrierDF split_carriers_df(const PlaneTDGL& p) {
+  PlaneCarrierDF d;
+  split(p.inv_vt, d.inv_vt_h, d.inv_vt_l);
+  split(p.kqn0, d.kqn0_h, d.kqn0_l);
+  split(p.kqp0, d.kqp0_h, d.kqp0_l);
+  split(p.kqN, d.kqN_h, d.kqN_l);
+  return d;
+}
+
+// a plane's FP64 coefficients as double-float pairs
 PlaneCoefDF split_coef_df(const PlaneCoef<double>& q) {
-  auto split = [](double x, float& h, float& l) {
-    h = (float)x;
-    l = (float)(x - (double)h);
-  };
   PlaneCoefDF d;
   split(q.cx, d.cx_h, d.cx_l);
   split(q.cy, d.cy_h, d.cy_l);
@@ -452,8 +464,8 @@ PlaneCoefDF split_coef_df(const PlaneCoef<double>& q) {
   return d;
 }
 
-// the mixed form evaluates its outer residual in double-float arithmetic unless
-// FERROX_DF_RESID=0 is set in the environment (FP64 residual; for comparisons)
+// the mixed form evaluates its Boltzmann carriers in double-float arithmetic unless
+// FERROX_DF_RESID=0 is set in the environment (FP64 carriers; for comparisons)
 bool df_resid_enabled() {
   const char* v = std::getenv("FERROX_DF_RESID");
   return !(v && v[0] == '0');
@@ -772,9 +784,9 @@ void enqueue_resid(ferrox_ctx* c, cudaStream_t s, int first, int set_cond,
   a.s_out = c->shift ? c->s_arena : nullptr;
   a.sinv_out = c->shift ? c->sinv0 : nullptr;
   a.carriers = carrier_kind(c);
-  a.coef_df = c->df_resid ? c->coef_df : nullptr;
+  a.carriers_df = c->df_resid ? c->carriers_df : nullptr;
   a.partials = c->partials_d;
-  a.kchunk = c->df_resid ? c->resid_kchunk_df : c->resid_kchunk;
+  a.kchunk = c->resid_kchunk;
   a.stats = c->stats_d;
   a.tol = c->num.tol;
   a.max_cycles = c->num.max_cycles;
@@ -992,11 +1004,11 @@ void enqueue_nn_features(ferrox_ctx* c, cudaStream_t s, __nv_bfloat16* x) {
   a.s_out = c->shift ? c->s_arena : nullptr;
   a.sinv_out = c->shift ? c->sinv0 : nullptr;
   a.carriers = carrier_kind(c);
-  a.coef_df = c->df_resid ? c->coef_df : nullptr;
+  a.carriers_df = c->df_resid ? c->carriers_df : nullptr;
   a.stats = c->stats_d;
   a.partials = c->partials_d;
   a.norm_out = c->nn_scale + 1;   // ||r|| of the guess, for the check of the correction
-  a.kchunk = c->df_resid ? c->resid_kchunk_df : c->resid_kchunk;
+  a.kchunk = c->resid_kchunk;
   launch_resid<T>(a, s);
   T* r = static_cast<T*>(c->r_arena);
   nn_bridge_restrict<T>(r, c->lv, c->nn_level, s);
@@ -1235,7 +1247,7 @@ void release(ferrox_ctx* c) {
   cudaGraph_t gr[4] = {c->gr_step, c->gr_solve, c->gr_tdgl, c->gr_step_nn};
   for (auto g : ge) if (g) cudaGraphExecDestroy(g);
   for (auto g : gr) if (g) cudaGraphDestroy(g);
-  void* ptrs[] = {c->b, c->Pbuf, c->Fbuf, c->phi_prev, c->e_arena, c->eb_arena, c->e_alt, c->r_arena, c->s_arena, c->coef, c->coef0, c->coef0s, c->bs, c->sinv0, c->coef_df,
+  void* ptrs[] = {c->b, c->Pbuf, c->Fbuf, c->phi_prev, c->e_arena, c->eb_arena, c->e_alt, c->r_arena, c->s_arena, c->coef, c->coef0, c->coef0s, c->bs, c->sinv0, c->coef_df, c->carriers_df,
                   c->planes_d, c->planes_f32_d, c->lv_d, c->lvt_d, c->nn_scale, c->phi_guess, c->nn_pf, c->nn_stats, c->params_d, c->stats_d, c->partials_d, c->charge_d,
                   c->charge_part_d, c->dense_d, c->dense_wide_d};
   for (void* p : ptrs) if (p) cudaFree(p);
@@ -1429,6 +1441,12 @@ ferrox_status ferrox_init_geometry(ferrox_ctx** out, const ferrox_geometry* geom
     FX_INIT_CK(cudaMemcpy(ctx->coef_df, cdf.data(), ctx->nz * sizeof(PlaneCoefDF),
                           cudaMemcpyHostToDevice));
     ctx->df_resid = mixed && df_resid_enabled();
+    if (ctx->df_resid && ctx->has_sc) {
+      std::vector<PlaneCarrierDF> ccd(ctx->nz);
+      for (int k = 0; k < ctx->nz; ++k) ccd[k] = split_carriers_df(ctx->planes[k]);
+      FX_INIT_CK(cudaMalloc(&ctx->carriers_df, ctx->nz * sizeof(PlaneCarrierDF)));
+      FX_INIT_CK(cudaMemcpy(ctx->carriers_df, ccd.data(), ctx->nz * sizeof(PlaneCarrierDF), cudaMemcpyHostToDevice));
+    }
   }
   ctx->dense_lev = dense_level(ctx);
   if (mixed) {
@@ -1870,6 +1888,8 @@ struct ferrox_batch {
   int* any_d = nullptr;               // phase profile: "any instance active" (device / pinned host)
   int* any_h = nullptr;
   int ntiles = 0;
+  int* rt_pre = nullptr;              // graph engine's residual: prefix of its blocks per instance
+  int rtiles = 0, rrows = 2;
   int* nsteps_d = nullptr;
   int* dbg = nullptr;
   DevParams* params = nullptr;
@@ -1945,6 +1965,9 @@ BatchArgs batch_args(ferrox_batch* B, int mode) {
   a.ticket = B->ticket;
   a.tile_pre = B->tile_pre;
   a.ntiles = B->ntiles;
+  a.rt_pre = B->rt_pre;
+  a.rtiles = B->rtiles;
+  a.rrows = B->rrows;
   a.eb = B->eb; a.sinv = B->sinv; a.leg_pre = B->leg_pre;
   for (int l = 0; l < kMaxLegLevels; ++l) {
     a.leg_blocks[l] = B->leg_blocks[l];
@@ -2215,7 +2238,7 @@ void batch_release(ferrox_batch* B) {
   if (B->gr_step) cudaGraphDestroy(B->gr_step);
   if (B->gr_solve) cudaGraphDestroy(B->gr_solve);
   void* ptrs[] = {B->b, B->Pbuf, B->backup, B->e, B->r, B->s, B->eb, B->sinv, B->leg_pre, B->coef, B->dense, B->coef0, B->planes, B->lv,
-                  B->lvt, B->pre, B->partials, B->active, B->bar, B->grp_d, B->status, B->ticket, B->tile_pre, B->any_d, B->nsteps_d, B->dbg, B->params,
+                  B->lvt, B->pre, B->partials, B->active, B->bar, B->grp_d, B->status, B->ticket, B->tile_pre, B->rt_pre, B->any_d, B->nsteps_d, B->dbg, B->params,
                   B->stats, B->inst, B->charge_part, B->charge_out};
   for (void* p : ptrs) if (p) cudaFree(p);
   if (B->host_pinned) cudaFreeHost(B->host_pinned);
@@ -2331,7 +2354,19 @@ ferrox_status ferrox_init_batch(ferrox_batch** out, int n, const ferrox_geometry
   FX_BINIT(cudaMalloc(&B->lv, (size_t)nlv * sizeof(LevelDesc)));
   FX_BINIT(cudaMalloc(&B->lvt, (size_t)nlvt * sizeof(LevelDesc)));
   FX_BINIT(cudaMalloc(&B->pre, (size_t)(1 + 2 * B->Ldown) * (n + 1) * sizeof(int)));
-  FX_BINIT(cudaMalloc(&B->partials, (size_t)3 * B->nrows * sizeof(double)));
+  {
+    std::vector<int> rp(n + 1, 0);
+    for (int i = 0; i < n; ++i) {
+      const ferrox_ctx& c = B->plans[i].c;
+      if (c.ny % 2) B->rrows = 1;
+      rp[i + 1] = rp[i] + ((c.nx + kResidBX - 1) / kResidBX) * ((c.ny + kResidBY - 1) / kResidBY) *
+                              ((c.nz + kResidBatchKZ - 1) / kResidBatchKZ);
+    }
+    B->rtiles = rp[n];
+    FX_BINIT(cudaMalloc(&B->rt_pre, (n + 1) * sizeof(int)));
+    FX_BINIT(cudaMemcpy(B->rt_pre, rp.data(), (n + 1) * sizeof(int), cudaMemcpyHostToDevice));
+  }
+  FX_BINIT(cudaMalloc(&B->partials, (size_t)3 * std::max(B->nrows, B->rtiles) * sizeof(double)));
   FX_BINIT(cudaMalloc(&B->active, n * sizeof(int)));
   FX_BINIT(cudaMalloc(&B->bar, (size_t)n * sizeof(GridBar)));
   FX_BINIT(cudaMalloc(&B->grp_d, 2 * (size_t)(n + 1) * sizeof(int)));

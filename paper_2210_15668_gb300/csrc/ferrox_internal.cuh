@@ -62,7 +62,8 @@ constexpr int kTailMaxSmem = 200 * 1024; // shared memory available to the tail 
 // 1799 / 2761, up to 32768 cells 1804 / 2775; larger FP32 levels lose.  FP64
 // levels use the split kernels at every size (+2.2% FP64).
 constexpr long long kSmallTransfer = 32768;
-constexpr int kResidBX = 32, kResidBY = 8; // residual: one thread per (x, y) column
+constexpr int kResidBX = 32, kResidBY = 8; // residual: columns of a block (two rows per thread)
+constexpr int kResidBatchKZ = 8;           // planes per block of the batched graph engine's residual
 constexpr int kTdglTileX = 32, kTdglTileY = 2, kTdglChunks = 4;  // batched TDGL: column tile, z chunks
 
 // Copy of a read-only table entry through the read-only data path (8-byte
@@ -103,6 +104,13 @@ struct PlaneTDGL {
   double Nc, Nv, eta_e0, eta_p0;
   // kq n0, kq p0, kq Nnet (the double-float residual forms rho from these)
   double kqn0, kqp0, kqN;
+};
+
+// a semiconductor plane's 1/VT, kq n0, kq p0 and kq Nnet as double-float pairs (nearest
+// floats of the value and of the rest), a table of its own: PlaneTDGL's stride is the
+// TDGL kernel's (256 bytes instead of 224 cost it 8%)
+struct PlaneCarrierDF {
+  float inv_vt_h, inv_vt_l, kqn0_h, kqn0_l, kqp0_h, kqp0_l, kqN_h, kqN_l;
 };
 
 // ---- per-plane multigrid coefficients of one level ----------------------------------
@@ -186,6 +194,8 @@ struct ResidArgs {
   int carriers;                      // carrier charge: 0 none, 1 Boltzmann planes only, 2 with
                                      // Fermi-Dirac planes
   const PlaneCoefDF* coef_df;        // non-null: stencil in double-float arithmetic (FP32 pipe)
+  const PlaneCarrierDF* carriers_df; // non-null: Boltzmann carriers in double-float beside the
+                                     // FP64 stencil
   void* sinv_out;                    // with s_out: 1 / (diag + s) of level 0 (float or double)
   int warp_rows;                     // nx is a multiple of 32: each warp holds 32 cells of a row
 };
@@ -454,6 +464,8 @@ struct BatchArgs {
   const int* pre;       // unit prefix tables: rows, smoothing rows per level, coarse rows per level
   const int* tile_pre;  // graph engine's TDGL: prefix of 32 x 2 column tiles per instance
   int ntiles;           // ... and their total
+  const int* rt_pre;    // graph engine's residual: prefix of its blocks per instance
+  int rtiles, rrows;    // ... their total, rows per thread (2, or 1 with a one-cell-wide instance)
   int Ldown;            // deepest multi-block level count over instances
   double* partials;     // 3 per row unit
   int* active;          // per instance

@@ -493,6 +493,30 @@ __device__ __forceinline__ double fd_half(double eta, double& dF) {
   return F;
 }
 
+// Carrier charge rho = kq (p - n + Nnet) of a semiconductor cell and the Newton shift
+// -d rho/d phi, FP64.  Every rounding is spelled out, so that the residual's variants
+// (and the two batched engines) agree bit for bit whatever they are inlined into.
+template <int SC>
+__device__ __forceinline__ void carrier_charge(const PlaneTDGL& pt, double phi, double& rho, double& shift) {
+  const double u = __dmul_rn(phi, pt.inv_vt);
+  double diff, sum;   // p - n; dp + dn in units of 1 / V_T
+  if (SC == 2 && pt.fd) {
+    // n = Nc F(eta_e0 + u), p = Nv F(eta_p0 - u); -d rho/d phi = kq (dn + dp)/VT
+    double dn, dp;
+    const double n = __dmul_rn(pt.Nc, fd_half(__dadd_rn(pt.eta_e0, u), dn));
+    diff = fma(pt.Nv, fd_half(__dadd_rn(pt.eta_p0, -u), dp), -n);
+    sum = fma(pt.Nc, dn, __dmul_rn(pt.Nv, dp));
+  } else {
+    double ep, em;
+    exp_pm(u, ep, em);
+    const double n = __dmul_rn(pt.n0, ep);
+    diff = fma(pt.p0, em, -n);
+    sum = fma(pt.p0, em, n);
+  }
+  rho = __dmul_rn(pt.kq, __dadd_rn(diff, pt.Nnet));
+  shift = __dmul_rn(__dmul_rn(pt.kq, sum), pt.inv_vt);
+}
+
 // FP64 residual of planes [k0, k1) of one (x, y) column, marching up with a
 // register window; accumulates r^2, b^2 (first residual of a solve only) and
 // rho^2.  SC = 0 compiles out the carrier term (stacks without a semiconductor
@@ -548,26 +572,13 @@ __device__ __forceinline__ void resid_column(const ResidArgs& a, int i, int j, i
     }
     double rho = 0.0;
     if (SC && pt.sc) {
-      if (SC == 2 && pt.fd) {
-        // n = Nc F(eta_e0 + u), p = Nv F(eta_p0 - u); -d rho/d phi = kq (dn + dp)/VT
-        const double u = pc * pt.inv_vt;
-        double dn, dp;
-        const double n = pt.Nc * fd_half(pt.eta_e0 + u, dn);
-        const double p = pt.Nv * fd_half(pt.eta_p0 - u, dp);
-        rho = pt.kq * (p - n + pt.Nnet);
-        if (s_out) put_shift<T>(a, t, pt.kq * fma(pt.Nc, dn, pt.Nv * dp) * pt.inv_vt, (T)c.diag);
-      } else {
-        double ep, em;
-        exp_pm(pc * pt.inv_vt, ep, em);
-        const double n = pt.n0 * ep;
-        const double p = pt.p0 * em;
-        rho = pt.kq * (p - n + pt.Nnet);
-        if (s_out) put_shift<T>(a, t, pt.kq * (n + p) * pt.inv_vt, (T)c.diag);
-      }
+      double s;
+      carrier_charge<SC>(pt, pc, rho, s);
+      if (s_out) put_shift<T>(a, t, s, (T)c.diag);
       acc_rho = fma(rho, rho, acc_rho);
     }
     // r = b + rho - A phi = (b + rho) - diag phi + couplings * neighbours
-    double r = fma(-c.diag, pc, SC ? bb + rho : bb);
+    double r = fma(-c.diag, pc, SC ? __dadd_rn(bb, rho) : bb);
     r = fma(c.czhi, pu, r);
     r = fma(c.czlo, pd, r);
     r = fma(c.cy, sy, r);
@@ -580,14 +591,146 @@ __device__ __forceinline__ void resid_column(const ResidArgs& a, int i, int j, i
   }
 }
 
-// The same residual with the stencil in double-float arithmetic (df_arith.cuh):
-// the potentials, the right-hand side b + rho and the coefficients enter as h + l
-// pairs, the products and sums keep about 48 bits, so r agrees with the FP64
-// residual to a few 2^-48 of the largest term while the FP64 pipe is left to the
-// carrier exponentials.  The output is the high part (T = float, the mixed form's
-// FP32 correction equation) or h + l (T = double); the squared norms accumulate
-// per thread in FP32 (they decide a tolerance, 1e-7 relative is ample) and enter
-// the block sums in FP64.
+// The same residual of planes [k0, k1) of R rows (j0 .. j0 + R - 1) and the 32 cells of a
+// warp: the operations of resid_column in the same order, with each potential loaded
+// once per warp column (z neighbours from the march, x neighbours from the adjacent
+// lanes, inner y neighbours from the thread's other rows) instead of five times.  The
+// FP64 pipe bounds it: seven operations per cell and one for the FP64 norm.  Every lane of
+// the warp has to call it; `in` marks those that hold a cell.
+//   DFC: Boltzmann carriers in double-float on the FP32 pipe, beside the FP64 stencil (the
+//     mixed form), added to the FP64 sum as pairs: FP32 and FP64 pipes overlap, and the
+//     exponentials cost no FP64 instruction.
+//   N: the type of the squared norms (float where they decide a tolerance from an FP32
+//     residual, as in resid_column_df).
+template <typename T, int SC, bool DFC, int R, typename N>
+__device__ __forceinline__ void resid_rows(const ResidArgs& a, int i, int j0, int k0, int k1, bool in, N& acc_r,
+                                           N& acc_b, double& acc_rho) {
+  const int nx = a.nx, ny = a.ny, nz = a.nz;
+  const long long plane = (long long)nx * ny;
+  T* r_out = static_cast<T*>(a.r_out);
+  T* s_out = static_cast<T*>(a.s_out);
+  // electrode lift of static boundary planes (nz >= 2: two planes)
+  double lift_bot = 0.0, lift_top = 0.0;
+  if (k0 == 0) lift_bot = __ldg(&a.planes[0].lift) * a.params->v_bot;
+  if (k1 == nz) lift_top = __ldg(&a.planes[nz - 1].lift) * a.params->v_top;
+  const int lane = threadIdx.x & 31;
+  const int x = in ? i : 0, y = in ? j0 : 0;         // idle lanes read cell 0 of the plane
+  const bool edge_m = lane == 0, edge_p = lane == 31 || i == nx - 1;
+  const long long col = (long long)y * nx + x;
+  const long long dxm = (x == 0) ? nx - 1 : -1, dxp = (x == nx - 1) ? 1 - nx : 1;
+  const long long lo = (long long)((y == 0) ? ny - 1 : y - 1) * nx + x;
+  const long long hi = (long long)((y + R >= ny) ? 0 : y + R) * nx + x;
+  const double* phi = a.phi;
+  float rho2f = 0.0f;   // rho^2 of the double-float carriers (enters only the scale of the test)
+  double pd[R], pc[R];
+#pragma unroll
+  for (int q = 0; q < R; ++q) {
+    pd[q] = k0 > 0 ? phi[(long long)(k0 - 1) * plane + col + (long long)q * nx] : 0.0;
+    pc[q] = phi[(long long)k0 * plane + col + (long long)q * nx];
+  }
+  for (int k = k0; k < k1; ++k) {
+    const long long o = k * plane;
+    const PlaneCoef<double> c = ldg_struct(a.coef0 + k);
+    const PlaneTDGL* pk = a.planes + k;
+    const int b_dyn = __ldg(&pk->b_dyn);
+    const double ylo = phi[o + lo], yhi = phi[o + hi];
+    const bool sc = SC && __ldg(&pk->sc);
+    PlaneTDGL pt;
+    PlaneCarrierDF cd;
+    float diag_f = 0.0f;
+    if (sc) {
+      pt = ldg_struct(pk);
+      if (DFC) {
+        cd = ldg_struct(a.carriers_df + k);
+        diag_f = (float)c.diag;
+      }
+    }
+    double pu[R], bb[R];
+#pragma unroll
+    for (int q = 0; q < R; ++q) {
+      const long long t = o + col + (long long)q * nx;
+      pu[q] = (k < nz - 1) ? phi[t + plane] : 0.0;
+      bb[q] = b_dyn ? a.b[t] : k == 0 ? lift_bot : k == nz - 1 ? lift_top : 0.0;
+    }
+#pragma unroll
+    for (int q = 0; q < R; ++q) {
+      const long long t = o + col + (long long)q * nx;
+      double xm = __shfl_up_sync(0xffffffffu, pc[q], 1), xp = __shfl_down_sync(0xffffffffu, pc[q], 1);
+      if (edge_m) xm = phi[t + dxm];
+      if (edge_p) xp = phi[t + dxp];
+      const double sx = xm + xp;
+      const double sy = (q ? pc[q - 1] : ylo) + (q < R - 1 ? pc[q + 1] : yhi);
+      double b_rho = bb[q];
+      df rho_df{0.0f, 0.0f};
+      bool add_df = false;
+      if (sc) {
+        df u{0.0f, 0.0f};
+        if (DFC) u = df_mul(df_from_double(pc[q]), df{cd.inv_vt_h, cd.inv_vt_l});
+        if (DFC && !(SC == 2 && pt.fd) && fabsf(u.h) <= kExpDFMax) {
+          // rho = kq p0 e^{-u} - kq n0 e^{u} + kq Nnet, u = phi / V_T
+          df ep, em;
+          exp_pm_df(u, ep, em);
+          const df kn = df_mul(df{cd.kqn0_h, cd.kqn0_l}, ep);
+          const df kp = df_mul(df{cd.kqp0_h, cd.kqp0_l}, em);
+          rho_df = df_add(df_add(kp, df_neg(kn)), df{cd.kqN_h, cd.kqN_l});
+          add_df = true;
+          if (in) rho2f = fmaf(rho_df.h, rho_df.h, rho2f);
+          if (s_out && in) {
+            const float sv = (kn.h + kp.h) * cd.inv_vt_h;
+            s_out[t] = (T)sv;
+            if (a.sinv_out) static_cast<T*>(a.sinv_out)[t] = (T)(1.0f / (diag_f + sv));
+          }
+        } else {
+          double s, rho;
+          carrier_charge<SC>(pt, pc[q], rho, s);
+          b_rho = __dadd_rn(b_rho, rho);
+          if (in) {
+            acc_rho = fma(rho, rho, acc_rho);
+            if (s_out) put_shift<T>(a, t, s, (T)c.diag);
+          }
+        }
+      }
+      // r = b + rho - A phi = (b + rho) - diag phi + couplings * neighbours
+      double r = fma(-c.diag, pc[q], b_rho);
+      r = fma(c.czhi, pu[q], r);
+      r = fma(c.czlo, pd[q], r);
+      r = fma(c.cy, sy, r);
+      r = fma(c.cx, sx, r);
+      float rf = 0.0f;
+      if (DFC && add_df) {
+        rf = df_add(df_from_double(r), rho_df).h;
+        if (in) r_out[t] = (T)rf;
+      } else {
+        const T rt = narrow_resid<T>(r);
+        if (in) r_out[t] = rt;
+        rf = (float)rt;
+      }
+      if (in) {
+        if constexpr (sizeof(N) == sizeof(float)) {
+          acc_r = fmaf(rf, rf, acc_r);
+          if (a.first) {
+            const float bf = df_from_double(bb[q]).h;
+            acc_b = fmaf(bf, bf, acc_b);
+          }
+        } else {
+          acc_r = fma(r, r, acc_r);
+          if (a.first) acc_b = fma(bb[q], bb[q], acc_b);
+        }
+      }
+    }
+#pragma unroll
+    for (int q = 0; q < R; ++q) {
+      pd[q] = pc[q];
+      pc[q] = pu[q];
+    }
+  }
+  if (DFC) acc_rho += (double)rho2f;
+}
+
+// The same residual with the stencil in double-float arithmetic too (df_arith.cuh), for
+// the diagnostic entry: the potentials, the right-hand side b + rho and the coefficients
+// enter as h + l pairs, the products and sums keep about 48 bits, so r agrees with the
+// FP64 residual to a few 2^-48 of the largest term.
 template <typename T, int SC>
 __device__ __forceinline__ void resid_column_df(const ResidArgs& a, int i, int j, int k0, int k1,
                                                 float& acc_r, float& acc_b, double& acc_rho) {
@@ -661,21 +804,9 @@ __device__ __forceinline__ void resid_column_df(const ResidArgs& a, int i, int j
         }
       } else {
         double rho;
-        if (SC == 2 && pt.fd) {
-          const double uu = pc_d * pt.inv_vt;
-          double dn, dp;
-          const double n = pt.Nc * fd_half(pt.eta_e0 + uu, dn);
-          const double p = pt.Nv * fd_half(pt.eta_p0 - uu, dp);
-          rho = pt.kq * (p - n + pt.Nnet);
-          if (s_out) put_shift<T>(a, t, pt.kq * fma(pt.Nc, dn, pt.Nv * dp) * pt.inv_vt, diag_of_df<T>(c));
-        } else {
-          double ep, em;
-          exp_pm(pc_d * pt.inv_vt, ep, em);
-          const double n = pt.n0 * ep;
-          const double p = pt.p0 * em;
-          rho = pt.kq * (p - n + pt.Nnet);
-          if (s_out) put_shift<T>(a, t, pt.kq * (n + p) * pt.inv_vt, diag_of_df<T>(c));
-        }
+        double s;
+        carrier_charge<SC>(pt, pc_d, rho, s);
+        if (s_out) put_shift<T>(a, t, s, diag_of_df<T>(c));
         b_df = df_from_double(bb + rho);
         acc_rho = fma(rho, rho, acc_rho);
       }

@@ -21,6 +21,7 @@
 #include <math.h>
 
 #include <algorithm>
+#include <type_traits>
 
 #include "ferrox_internal.cuh"
 #include "mg_device.cuh"
@@ -528,18 +529,39 @@ __global__ void __launch_bounds__(kTailThreads) tail_kernel(MGArgs<T> g, TailArg
   tail_vcycle<T>(g, t, tail_smem);
 }
 
-// grid (x chunk, row chunk, z chunk): block z owns planes [z kchunk, (z+1) kchunk)
-template <typename T, int SC, bool DF = false>
-__global__ void __launch_bounds__(kResidBX* kResidBY) resid_kernel(ResidArgs a) {
+// the double-float residual on its own (ferrox_residual): r only, no norms
+template <typename T, int SC>
+__global__ void __launch_bounds__(kResidBX* kResidBY) resid_df_kernel(ResidArgs a) {
   pdl_enter();
   const int i = blockIdx.x * kResidBX + threadIdx.x;
   const int j = blockIdx.y * kResidBY + threadIdx.y;
   const int k0 = blockIdx.z * a.kchunk;
   const int k1 = min(a.nz, k0 + a.kchunk);
+  float fr = 0.0f, fb = 0.0f;
+  double acc_rho = 0.0;
+  if (i < a.nx && j < a.ny) resid_column_df<T, SC>(a, i, j, k0, k1, fr, fb, acc_rho);
+}
+
+// grid (x chunk, row chunk, z chunk): block z owns planes [z kchunk, (z+1) kchunk)
+// R rows per thread (kResidBY / R thread rows).  256x256x32 without carriers: 49 us with
+// the stencil in double-float (470 FP32 and integer instructions a cell), 64 us in FP64
+// with one column per thread, 33 us here; two rows per thread beat one (35) and four (39),
+// chunks of 4 planes those of 16 (35) and 32 (45).  With double-float carriers 80
+// registers (512x512x128 MFISM 682 us a launch; 104 registers 775, the double-float
+// stencil 1090); Fermi-Dirac planes keep one row per thread (their FP64 exponentials
+// hold 126 registers).
+template <typename T, int SC, bool DFC, int R>
+__global__ void __launch_bounds__(kResidBX* kResidBY / R, DFC && SC == 1 ? 3 * R : 1) resid_kernel(ResidArgs a) {
+  pdl_enter();
+  const int i = blockIdx.x * kResidBX + threadIdx.x;
+  const int j = blockIdx.y * kResidBY + R * threadIdx.y;
+  const int k0 = blockIdx.z * a.kchunk;
+  const int k1 = min(a.nz, k0 + a.kchunk);
   double acc_r = 0.0, acc_b = 0.0, acc_rho = 0.0;
-  if constexpr (DF) {
+  const bool in = i < a.nx && j < a.ny;
+  if constexpr (sizeof(T) == sizeof(float)) {
     float fr = 0.0f, fb = 0.0f;
-    if (i < a.nx && j < a.ny) resid_column_df<T, SC>(a, i, j, k0, k1, fr, fb, acc_rho);
+    resid_rows<T, SC, DFC, R>(a, i, j, k0, k1, in, fr, fb, acc_rho);
     if (a.no_stats) return;
     // the squared norms within the block in FP32 (no FP64 work per cell), across
     // blocks in FP64 below; ||rho||^2 in FP64
@@ -548,7 +570,7 @@ __global__ void __launch_bounds__(kResidBX* kResidBY) resid_kernel(ResidArgs a) 
     acc_r = (double)fr;
     acc_b = (double)fb;
   } else {
-    if (i < a.nx && j < a.ny) resid_column<T, SC>(a, i, j, k0, k1, acc_r, acc_b, acc_rho);
+    resid_rows<T, SC, DFC, R>(a, i, j, k0, k1, in, acc_r, acc_b, acc_rho);
     if (a.no_stats) return;
     // ||b||^2 is summed on the first residual of a solve only, ||rho||^2 with carriers only
     if (SC || a.first)
@@ -571,14 +593,23 @@ __global__ void __launch_bounds__(kResidBX* kResidBY) resid_kernel(ResidArgs a) 
   __syncthreads();
   if (!last) return;
   __threadfence();
-  // fixed-order sum of the partials (deterministic)
+  // fixed-order sum of the partials (deterministic), read at L2, eight in flight
   double sr = 0.0, sb = 0.0, sq = 0.0;
-  const volatile double* P = a.partials;
-  for (int q = tid; q < nblk; q += blockDim.x * blockDim.y) {
-    sr += P[q];
-    sb += P[nblk + q];
-    sq += P[2 * nblk + q];
-  }
+  const int nthr = blockDim.x * blockDim.y;
+  auto sum = [&](const double* P) {
+    double s = 0.0;
+    for (int q = tid; q < nblk; q += 8 * nthr) {
+      double v[8];
+#pragma unroll
+      for (int w = 0; w < 8; ++w) v[w] = q + w * nthr < nblk ? __ldcg(P + q + w * nthr) : 0.0;
+#pragma unroll
+      for (int w = 0; w < 8; ++w) s += v[w];
+    }
+    return s;
+  };
+  sr = sum(a.partials);
+  if (a.first) sb = sum(a.partials + nblk);
+  if (SC) sq = sum(a.partials + 2 * nblk);
   block_sum3(sr, sb, sq);
   if (tid == 0) {
     a.stats->done_ctr = 0;
@@ -852,19 +883,33 @@ template <typename T>
 void launch_resid(const ResidArgs& a_in, cudaStream_t s) {
   ResidArgs a = a_in;
   a.warp_rows = a.nx % 32 == 0;
-  dim3 block(kResidBX, kResidBY);
-  dim3 grid((a.nx + kResidBX - 1) / kResidBX, (a.ny + kResidBY - 1) / kResidBY,
-            (a.nz + a.kchunk - 1) / a.kchunk);
+  const dim3 grid((a.nx + kResidBX - 1) / kResidBX, (a.ny + kResidBY - 1) / kResidBY,
+                  (a.nz + a.kchunk - 1) / a.kchunk);
   // carriers: 0 none, 1 Boltzmann statistics only, 2 with Fermi-Dirac planes
-  if (a.coef_df) {
-    if (a.carriers == 2) launch_k(resid_kernel<T, 2, true>, grid, block, 0, s, a);
-    else if (a.carriers == 1) launch_k(resid_kernel<T, 1, true>, grid, block, 0, s, a);
-    else launch_k(resid_kernel<T, 0, true>, grid, block, 0, s, a);
-  } else {
-    if (a.carriers == 2) launch_k(resid_kernel<T, 2>, grid, block, 0, s, a);
-    else if (a.carriers == 1) launch_k(resid_kernel<T, 1>, grid, block, 0, s, a);
-    else launch_k(resid_kernel<T, 0>, grid, block, 0, s, a);
+  if constexpr (sizeof(T) == sizeof(double)) {
+    if (a.coef_df) {   // the double-float diagnostic
+      const dim3 block(kResidBX, kResidBY);
+      if (a.carriers == 2) launch_k(resid_df_kernel<T, 2>, grid, block, 0, s, a);
+      else if (a.carriers == 1) launch_k(resid_df_kernel<T, 1>, grid, block, 0, s, a);
+      else launch_k(resid_df_kernel<T, 0>, grid, block, 0, s, a);
+      return;
+    }
   }
+  auto go = [&](auto rows) {
+    constexpr int R = decltype(rows)::value;
+    const dim3 block(kResidBX, kResidBY / R);
+    if constexpr (sizeof(T) == sizeof(float)) {
+      if (a.carriers_df) {
+        if (a.carriers == 2) { launch_k(resid_kernel<T, 2, true, R>, grid, block, 0, s, a); return; }
+        if (a.carriers == 1) { launch_k(resid_kernel<T, 1, true, R>, grid, block, 0, s, a); return; }
+      }
+    }
+    if (a.carriers == 2) launch_k(resid_kernel<T, 2, false, R>, grid, block, 0, s, a);
+    else if (a.carriers == 1) launch_k(resid_kernel<T, 1, false, R>, grid, block, 0, s, a);
+    else launch_k(resid_kernel<T, 0, false, R>, grid, block, 0, s, a);
+  };
+  if (a.ny % 2 == 0 && a.carriers != 2) go(std::integral_constant<int, 2>());
+  else go(std::integral_constant<int, 1>());   // Fermi-Dirac planes; one-cell-wide devices
 }
 
 template <typename T>

@@ -169,14 +169,15 @@ __device__ void phase_resid(const Ctx<T>& c, int first, int copy_back) {
   }
 }
 
-// Per-instance convergence decision: one warp per instance, fixed-order sums.
+// Per-instance convergence decision: one warp per instance, fixed-order sums of the
+// residual units [pre[i], pre[i + 1]).
 template <typename T>
-__device__ void phase_decide(const Ctx<T>& c, int first) {
+__device__ void phase_decide(const Ctx<T>& c, int first, const int* pre) {
   const BatchArgs& A = c.A;
   for (int i = c.i_lo + c.gwarp; i < c.i_hi; i += c.nwarps) {
     if (!ld_flag(A.active + i)) continue;
     double sr = 0.0, sb = 0.0, sq = 0.0;
-    for (int u = A.pre[i] + c.lane; u < A.pre[i + 1]; u += 32) {
+    for (int u = pre[i] + c.lane; u < pre[i + 1]; u += 32) {
       sr += A.partials[3 * u];
       sb += A.partials[3 * u + 1];
       sq += A.partials[3 * u + 2];
@@ -376,7 +377,7 @@ __global__ void __launch_bounds__(512, 1) batch_kernel(BatchArgs A) {
     for (int cyc = 0;; ++cyc) {
       phase_resid(c, cyc == 0, A.mode == 0 && cyc == 0);
       FX_BAR();
-      phase_decide(c, cyc == 0);
+      phase_decide(c, cyc == 0, A.pre);
       FX_BAR();
       int any = 0;
       for (int i = c.i_lo; i < c.i_hi; ++i) any |= ld_flag(A.active + i);
@@ -513,10 +514,54 @@ __global__ void __launch_bounds__(kTdglTileX* kTdglTileY* kTdglChunks) ph_tdgl_c
   }
 }
 
-template <typename T>
-__global__ void __launch_bounds__(256) ph_resid_kernel(BatchArgs A, int first, int copy_back) {
+// The outer residual of the graph engine: one block per 32 x kResidBY column tile and z
+// chunk of an instance, R rows per thread (resid_rows), so that short devices fill the
+// SMs too (a warp per row left half of them idle).  The cells' operations are
+// resid_column's; the norms are summed per block instead of per row.  64 instances, per
+// launch: 165 us by rows, 155 in chunks of 4 planes, 136 in chunks of 8 (kept).
+template <typename T, int R>
+__global__ void __launch_bounds__(kResidBX* kResidBY / R) ph_resid_kernel(BatchArgs A, int first, int copy_back) {
   pdl_enter();
-  phase_resid(grid_ctx<T>(A), first, copy_back);
+  const int inst = find_inst(A.rt_pre, A.ninst, (int)blockIdx.x);
+  if (!ld_flag(A.active + inst)) return;
+  const BatchInst I = ldg_struct(A.inst + inst);
+  ResidArgs ra = I.resid;
+  ra.first = first;
+  const int tile = (int)blockIdx.x - A.rt_pre[inst];
+  const int tx = (ra.nx + kResidBX - 1) / kResidBX, ty = (ra.ny + kResidBY - 1) / kResidBY;
+  const int bz = tile / (tx * ty), rest = tile - bz * tx * ty, by = rest / tx, bx = rest - by * tx;
+  const int i = bx * kResidBX + threadIdx.x, j = by * kResidBY + R * threadIdx.y;
+  const int k0 = bz * kResidBatchKZ, k1 = min(ra.nz, k0 + kResidBatchKZ);
+  const bool in = i < ra.nx && j < ra.ny;
+  if (copy_back && in) {
+    for (int k = max(k0, I.fe_lo); k <= min(k1 - 1, I.fe_hi); ++k)
+      for (int q = 0; q < R; ++q) {
+        const long long t = ((long long)k * ra.ny + j + q) * ra.nx + i;
+        I.P[t] = I.Pbuf[t];
+      }
+  }
+  double ar = 0.0, ab = 0.0, aq = 0.0;
+  if (ra.carriers) {
+    resid_rows<T, 2, false, R>(ra, i, j, k0, k1, in, ar, ab, aq);
+    block_sum3(ar, ab, aq);
+  } else {
+    resid_rows<T, 0, false, R>(ra, i, j, k0, k1, in, ar, ab, aq);   // no b + rho add
+    if (first) block_sum3(ar, ab, aq);
+    else block_sum1(ar);
+  }
+  if (threadIdx.x == 0 && threadIdx.y == 0) {
+    double* p = A.partials + 3 * (size_t)blockIdx.x;
+    p[0] = ar;
+    p[1] = ab;
+    p[2] = aq;
+  }
+}
+
+template <typename T>
+cudaError_t launch_ph_resid(const BatchArgs& a, int first, int copy_back, cudaStream_t s) {
+  const dim3 grid(a.rtiles);
+  if (a.rrows == 2) return launch_k(ph_resid_kernel<T, 2>, grid, dim3(kResidBX, kResidBY / 2), 0, s, a, first, copy_back);
+  return launch_k(ph_resid_kernel<T, 1>, grid, dim3(kResidBX, kResidBY), 0, s, a, first, copy_back);
 }
 
 // The per-instance decisions, one single-warp block per instance so that their
@@ -528,7 +573,7 @@ __global__ void __launch_bounds__(32) ph_decide_kernel(BatchArgs A, int first, u
   pdl_enter();
   const Ctx<T> c{A, batch_mg<T>(A), (int)(threadIdx.x & 31), (int)blockIdx.x, (int)gridDim.x,
                  0, A.ninst, 0, 1};
-  phase_decide(c, first);
+  phase_decide(c, first, A.rt_pre);
   __shared__ int last;
   if (threadIdx.x == 0) {
     __threadfence();   // this block's flags before its ticket
@@ -747,7 +792,7 @@ cudaError_t capture_phases(const BatchArgs& a, int unit_blocks, size_t tail_smem
   if ((e = launch_k(ph_tdgl_chunk_kernel, dim3(a.ntiles), dim3(kTdglTileX, kTdglTileY, kTdglChunks), 0, s, a,
                     mode == 1 ? 3 : 0)) != cudaSuccess)
     return e;
-  if ((e = launch_k(ph_resid_kernel<T>, ub, ut, 0, s, a, 1, mode == 0 ? 1 : 0)) != cudaSuccess) return e;
+  if ((e = launch_ph_resid<T>(a, 1, mode == 0 ? 1 : 0, s)) != cudaSuccess) return e;
   cudaStreamCaptureStatus st;
   cudaGraph_t g;
   const cudaGraphNode_t* deps = nullptr;
@@ -792,7 +837,7 @@ cudaError_t capture_phases(const BatchArgs& a, int unit_blocks, size_t tail_smem
     }
   }
   if (a.any_full_tail || a.nu2 == 0) launch_k(ph_update_kernel<T>, ub, ut, 0, s2, a);
-  launch_k(ph_resid_kernel<T>, ub, ut, 0, s2, a, 0, 0);
+  launch_ph_resid<T>(a, 0, 0, s2);
   launch_k(ph_decide_kernel<T>, dim3(a.ninst), dim3(32), 0, s2, a, 0, (unsigned long long)h);
   if ((e = cudaGetLastError()) != cudaSuccess) return e;
   cudaGraph_t body_out;
@@ -839,7 +884,7 @@ cudaError_t profile_phases(const BatchArgs& a0, int unit_blocks, size_t tail_sme
   mark(TDGL);
   note(launch_k(ph_tdgl_chunk_kernel, dim3(a.ntiles), dim3(kTdglTileX, kTdglTileY, kTdglChunks), 0, s, a, 0));
   mark(RESID);
-  note(launch_k(ph_resid_kernel<T>, ub, ut, 0, s, a, 1, 1));
+  note(launch_ph_resid<T>(a, 1, 1, s));
   mark(DECIDE);
   note(launch_k(ph_decide_kernel<T>, dim3(a.ninst), dim3(32), 0, s, a, 1, 0ULL));
   mark(WAIT);
@@ -882,7 +927,7 @@ cudaError_t profile_phases(const BatchArgs& a0, int unit_blocks, size_t tail_sme
       note(launch_k(ph_update_kernel<T>, ub, ut, 0, s, a));
     }
     mark(RESID);
-    note(launch_k(ph_resid_kernel<T>, ub, ut, 0, s, a, 0, 0));
+    note(launch_ph_resid<T>(a, 0, 0, s));
     mark(DECIDE);
     note(launch_k(ph_decide_kernel<T>, dim3(a.ninst), dim3(32), 0, s, a, 0, 0ULL));
     mark(WAIT);
