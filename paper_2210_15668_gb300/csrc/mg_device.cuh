@@ -320,6 +320,86 @@ __device__ FX_TAIL_LINKAGE void tail_smooth(const MGArgs<T>& a, const LevelDesc&
     }
 }
 
+// Many sweeps of one level (a coarsest level that cannot be halved further, relaxed
+// bottom_sweeps times) with two red/black pairs per thread held in registers: their
+// right-hand sides, reciprocal diagonals, couplings, neighbour indices and own
+// corrections are set up once, so a colour phase is five shared-memory loads, six
+// operations and one store per cell, and a barrier.  tail_smooth decodes every pair and
+// loads its level, plane coefficients and shift anew in every phase; it stays the better
+// one for the two sweeps of the other levels, where a tail's time is the first pass over
+// its code (both measured, 256x256x64 MFISM: 28 us a V-cycle either way).  96x80x37
+// MFISM, coarsest level 6x10x37 cells, 64 sweeps: the tail 118 -> 43 us a V-cycle.
+constexpr int kTailHeldSweeps = 8;   // sweeps from which the set-up pays
+template <typename T>
+__device__ __forceinline__ void tail_smooth_held(const MGArgs<T>& a, const LevelDesc& L, int sweeps) {
+  constexpr int ITEMS = 2;
+  const int hx = (L.nx + 1) >> 1, items = hx * L.ny * L.nz;
+  const unsigned long long mx = magic32(hx), my = magic32(L.ny);
+  const int plane = L.nx * L.ny;
+  T* e = a.e + L.off;
+  T v[ITEMS][2], r[ITEMS][2], inv[ITEMS][2], cx[ITEMS], cy[ITEMS], cl[ITEMS], ch[ITEMS];
+  int id[ITEMS], xo[ITEMS][2], ym[ITEMS], yp[ITEMS], zl[ITEMS], zh[ITEMS], par[ITEMS];
+  bool two[ITEMS], div[ITEMS];
+#pragma unroll
+  for (int q = 0; q < ITEMS; ++q) {
+    const int t = (int)threadIdx.x + q * (int)blockDim.x;
+    par[q] = -1;
+    if (t >= items) continue;
+    const int rest = div32(t, mx), k = div32(rest, my);
+    const int ip = t - rest * hx, j = rest - k * L.ny, i = 2 * ip;
+    id[q] = (k * L.ny + j) * L.nx + i;
+    two[q] = i + 1 < L.nx;
+    par[q] = (j + k) & 1;                       // colour of the pair's first cell
+    // the x neighbour outside the pair (of a single cell: itself)
+    xo[q][0] = two[q] ? (i == 0 ? L.nx - 1 : -1) : 0;
+    xo[q][1] = i + 2 >= L.nx ? 1 - L.nx : 1;
+    ym[q] = ((j == 0) ? L.ny - 1 : -1) * L.nx;
+    yp[q] = ((j == L.ny - 1) ? 1 - L.ny : 1) * L.nx;
+    const PlaneCoef<T> c = ldg_struct(a.coef + L.coef_off + k);
+    cx[q] = c.cx; cy[q] = c.cy;
+    cl[q] = k > 0 ? c.czlo : T(0);
+    ch[q] = k < L.nz - 1 ? c.czhi : T(0);
+    zl[q] = k > 0 ? -plane : 0;                 // times a zero coupling at the electrodes
+    zh[q] = k < L.nz - 1 ? plane : 0;
+    // FP64 divides by the shifted diagonal, FP32 multiplies by its reciprocal (over_shifted)
+    div[q] = sizeof(T) == sizeof(double) && c.has_s;
+#pragma unroll
+    for (int w = 0; w < 2; ++w) {
+      const int t2 = id[q] + (w && two[q] ? 1 : 0);
+      r[q][w] = a.r[L.off + t2];
+      if (!c.has_s) inv[q][w] = c.invdiag;
+      else if constexpr (sizeof(T) == sizeof(float)) inv[q][w] = T(1) / (c.diag + a.s[L.off + t2]);
+      else inv[q][w] = c.diag + a.s[L.off + t2];
+      v[q][w] = T(0);
+      e[t2] = T(0);
+    }
+  }
+  __syncthreads();
+  for (int sw = 0; sw < sweeps; ++sw)
+#pragma unroll
+    for (int color = 0; color < 2; ++color) {
+#pragma unroll
+      for (int q = 0; q < ITEMS; ++q) {
+        if (par[q] < 0) continue;
+        const int w = par[q] ^ color;            // which cell of the pair has this colour
+        if (w && !two[q]) continue;
+        const int t = id[q] + w;
+        const T own = two[q] ? (w ? v[q][0] : v[q][1]) : v[q][0];
+        T acc = w ? r[q][1] : r[q][0];
+        acc = fma(cx[q], e[t + (w ? xo[q][1] : xo[q][0])] + own, acc);
+        acc = fma(cy[q], e[t + ym[q]] + e[t + yp[q]], acc);
+        acc = fma(cl[q], e[t + zl[q]], acc);
+        acc = fma(ch[q], e[t + zh[q]], acc);
+        const T d = w ? inv[q][1] : inv[q][0];
+        const T x = div[q] ? acc / d : acc * d;
+        if (w) v[q][1] = x;
+        else v[q][0] = x;
+        e[t] = x;
+      }
+      __syncthreads();
+    }
+}
+
 // e = A^-1 r on a level of n <= kDenseMax cells: the inverse (row-major, computed
 // on the host in FP64) times r, four lanes per row and a fixed-order reduction.
 template <typename T>
@@ -373,7 +453,11 @@ __device__ FX_TAIL_LINKAGE void tail_vcycle(const MGArgs<T>& g, const TailArgs& 
     const LevelDesc B = ldg_struct(lv + bottom);
     tail_dense(static_cast<const T*>(t.dense), (int)B.ncell, sr + B.off, se + B.off);
   } else {
-    tail_smooth(a, lv[bottom], t.bottom_sweeps, 1);
+    const LevelDesc B = ldg_struct(lv + bottom);
+    if (t.bottom_sweeps >= kTailHeldSweeps && ((B.nx + 1) >> 1) * B.ny * B.nz <= 2 * (int)blockDim.x)
+      tail_smooth_held(a, B, t.bottom_sweeps);
+    else
+      tail_smooth(a, B, t.bottom_sweeps, 1);
   }
   for (int l = bottom - 1; l >= 0; --l) {
     const LevelDesc F = ldg_struct(lv + l), C = ldg_struct(lv + l + 1);
