@@ -33,10 +33,6 @@ __device__ __forceinline__ void mma_bf16(float (&d)[4], const unsigned (&a)[4], 
       : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b[0]), "r"(b[1]));
 }
 
-__device__ __forceinline__ unsigned pack2(bf16 lo, bf16 hi) {
-  return (unsigned)__bfloat16_as_ushort(lo) | ((unsigned)__bfloat16_as_ushort(hi) << 16);
-}
-
 // voxel index of the neighbour at tap (dz, dy, dx) = (tap/9, tap/3%3, tap%3) - 1,
 // or -1 outside the z range
 __device__ __forceinline__ int nb_index(int z, int y, int x, int tap, const NNGrid& g) {
@@ -68,7 +64,7 @@ constexpr int kConvTiles = 4;
 template <int COUT>
 __global__ void __launch_bounds__(32 * kConvTiles * 3) conv_fwd_kernel(
     const bf16* __restrict__ in, int cin, const bf16* __restrict__ wk,
-    const float* __restrict__ bias, NNGrid g, int relu, bf16* __restrict__ out_bf,
+    const float* __restrict__ bias, NNGrid g, int relu, const bf16* __restrict__ mask, bf16* __restrict__ out_bf,
     float* __restrict__ out_f, int f_ch0) {
   __shared__ float part[2][kConvTiles][COUT / 8][4][32];
   const int lane = threadIdx.x, tile = threadIdx.y, slab = threadIdx.z;
@@ -136,6 +132,11 @@ __global__ void __launch_bounds__(32 * kConvTiles * 3) conv_fwd_kernel(
       float v0 = acc[j][2 * r], v1 = acc[j][2 * r + 1];
       if (bias) { v0 += bias[co]; v1 += bias[co + 1]; }
       if (relu) { v0 = fmaxf(v0, 0.f); v1 = fmaxf(v1, 0.f); }
+      if (mask) {
+        const float2 am = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(mask + (size_t)m * COUT + co));
+        if (!(am.x > 0.f)) v0 = 0.f;
+        if (!(am.y > 0.f)) v1 = 0.f;
+      }
       if (out_bf)
         *reinterpret_cast<__nv_bfloat162*>(out_bf + (size_t)m * COUT + co) = __floats2bfloat162_rn(v0, v1);
       if (out_f && f_ch0) {
@@ -292,8 +293,8 @@ __device__ __forceinline__ void tc_load_halo(const bf16* __restrict__ in, const 
 
 template <int CIN, int COUT>
 __device__ __forceinline__ void tc_epilogue(unsigned tmem_acc, const NNGrid& g, TcTile t, int zt,
-                                            const float* __restrict__ bias, int relu, bf16* __restrict__ out_bf,
-                                            float* __restrict__ out_f, int f_ch0) {
+                                            const float* __restrict__ bias, int relu, const bf16* __restrict__ mask,
+                                            bf16* __restrict__ out_bf, float* __restrict__ out_f, int f_ch0) {
   const int tid = threadIdx.x, warp = tid >> 5;
   // thread tid holds accumulator row tid = voxel (y0 + tid / 8, x0 + tid % 8)
   const int x = t.x0 + (tid & 7), y = t.y0 + (tid >> 3);
@@ -307,6 +308,17 @@ __device__ __forceinline__ void tc_epilogue(unsigned tmem_acc, const NNGrid& g, 
       for (int i = 0; i < 16; ++i) {
         if (bias) v[i] += __ldg(bias + 16 * j + i);
         if (relu) v[i] = fmaxf(v[i], 0.f);
+      }
+      if (mask) {   // the ReLU's backward: zero where the activation is not positive
+        const uint4* mp = reinterpret_cast<const uint4*>(mask + m * COUT + 16 * j);
+        const uint4 q[2] = {mp[0], mp[1]};
+        const __nv_bfloat162* h = reinterpret_cast<const __nv_bfloat162*>(q);
+#pragma unroll
+        for (int i = 0; i < 8; ++i) {
+          const float2 am = __bfloat1622float2(h[i]);
+          if (!(am.x > 0.f)) v[2 * i] = 0.f;
+          if (!(am.y > 0.f)) v[2 * i + 1] = 0.f;
+        }
       }
       if (out_bf) {
         uint4 q[2];
@@ -331,8 +343,8 @@ __device__ __forceinline__ void tc_epilogue(unsigned tmem_acc, const NNGrid& g, 
 template <int CIN, int COUT, bool UP>
 __global__ void __launch_bounds__(kTcThreads) conv_tc_kernel(
     const bf16* __restrict__ in, const bf16* __restrict__ s1, const bf16* __restrict__ wt,
-    const float* __restrict__ bias, NNGrid g, int zt, int relu, bf16* __restrict__ out_bf,
-    float* __restrict__ out_f, int f_ch0, int* __restrict__ fault) {
+    const float* __restrict__ bias, NNGrid g, int zt, int relu, const bf16* __restrict__ mask,
+    bf16* __restrict__ out_bf, float* __restrict__ out_f, int f_ch0, int* __restrict__ fault) {
   constexpr int NCH = CIN / 8;
   constexpr int WBYTES = 27 * CIN * COUT * 2;
   extern __shared__ __align__(128) unsigned char smem[];
@@ -409,7 +421,7 @@ __global__ void __launch_bounds__(kTcThreads) conv_tc_kernel(
     asm volatile("cp.async.commit_group;\n" ::: "memory");
     if (ok && i > 0)
       tc_epilogue<CIN, COUT>(tmem + (unsigned)((cur ^ 1) * zt * COUT), g, tc_tile(blockIdx.x + (i - 1) * gridDim.x, g, zt),
-                             zt, bias, relu, out_bf, out_f, f_ch0);
+                             zt, bias, relu, mask, out_bf, out_f, f_ch0);
   }
   if (ok && nmine > 0) {
     const int l = nmine - 1;
@@ -417,7 +429,7 @@ __global__ void __launch_bounds__(kTcThreads) conv_tc_kernel(
     asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
     if (ok)
       tc_epilogue<CIN, COUT>(tmem + (unsigned)((l & 1) * zt * COUT), g, tc_tile(blockIdx.x + l * gridDim.x, g, zt), zt,
-                             bias, relu, out_bf, out_f, f_ch0);
+                             bias, relu, mask, out_bf, out_f, f_ch0);
   }
   asm volatile("cp.async.wait_group 0;\n" ::: "memory");
   if (!ok && tid == 0) {
@@ -434,84 +446,141 @@ __global__ void __launch_bounds__(kTcThreads) conv_tc_kernel(
   }
 }
 
-// gw[tap][ci][co] += sum_m in[nb(m, tap)][ci] dout[m][co] over this warp's voxel chunk
-template <int CIN, int COUT>
-__global__ void __launch_bounds__(128) conv_wgrad_kernel(const bf16* __restrict__ in,
-                                                         const bf16* __restrict__ dout, NNGrid g,
-                                                         int chunk, float* __restrict__ gw) {
-  const int warp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-  const int lane = threadIdx.x & 31;
-  const int M = g.D * g.H * g.W;
-  const int nparts = (M + chunk - 1) / chunk;
-  if (warp >= 27 * nparts) return;
-  const int tap = warp % 27, part = warp / 27;
-  const int mb = part * chunk, me = min(M, mb + chunk);
-  const int gq = lane >> 2, tq = lane & 3;
-  float acc[CIN / 16][COUT / 8][4];
-#pragma unroll
-  for (int c = 0; c < CIN / 16; ++c)
-#pragma unroll
-    for (int j = 0; j < COUT / 8; ++j) acc[c][j][0] = acc[c][j][1] = acc[c][j][2] = acc[c][j][3] = 0.f;
-  const bf16 zero = __float2bfloat16(0.f);
-  for (int m0 = mb; m0 < me; m0 += 16) {
-    // the four voxels of this thread's K slots: 2tq, 2tq+1, 2tq+8, 2tq+9
-    int nbv[4];
-    bool okv[4];
-#pragma unroll
-    for (int q = 0; q < 4; ++q) {
-      const int m = m0 + 2 * tq + (q & 1) + 8 * (q >> 1);
-      okv[q] = m < me;
-      int z, y, x;
-      voxel_zyx(okv[q] ? m : 0, g, z, y, x);
-      nbv[q] = okv[q] ? nb_index(z, y, x, tap, g) : -1;
-    }
-    unsigned bfr[COUT / 8][2];
-#pragma unroll
-    for (int j = 0; j < COUT / 8; ++j) {
-      const int co = j * 8 + gq;
-      bf16 d[4];
-#pragma unroll
-      for (int q = 0; q < 4; ++q) {
-        const int m = m0 + 2 * tq + (q & 1) + 8 * (q >> 1);
-        d[q] = okv[q] ? dout[(size_t)m * COUT + co] : zero;
-      }
-      bfr[j][0] = pack2(d[0], d[1]);
-      bfr[j][1] = pack2(d[2], d[3]);
-    }
-#pragma unroll
-    for (int c = 0; c < CIN / 16; ++c) {
-      bf16 lo[4], hi[4];
-#pragma unroll
-      for (int q = 0; q < 4; ++q) {
-        lo[q] = nbv[q] >= 0 ? in[(size_t)nbv[q] * CIN + c * 16 + gq] : zero;
-        hi[q] = nbv[q] >= 0 ? in[(size_t)nbv[q] * CIN + c * 16 + gq + 8] : zero;
-      }
-      const unsigned a[4] = {pack2(lo[0], lo[1]), pack2(hi[0], hi[1]), pack2(lo[2], lo[3]),
-                             pack2(hi[2], hi[3])};
-#pragma unroll
-      for (int j = 0; j < COUT / 8; ++j) mma_bf16(acc[c][j], a, bfr[j]);
-    }
-  }
-#pragma unroll
-  for (int c = 0; c < CIN / 16; ++c)
-#pragma unroll
-    for (int j = 0; j < COUT / 8; ++j) {
-      float* base = gw + (size_t)tap * CIN * COUT;
-      const int co = j * 8 + 2 * tq;
-      atomicAdd(base + (c * 16 + gq) * COUT + co, acc[c][j][0]);
-      atomicAdd(base + (c * 16 + gq) * COUT + co + 1, acc[c][j][1]);
-      atomicAdd(base + (c * 16 + gq + 8) * COUT + co, acc[c][j][2]);
-      atomicAdd(base + (c * 16 + gq + 8) * COUT + co + 1, acc[c][j][3]);
-    }
+// ---- weight gradients -------------------------------------------------------------------
+// gw[tap][ci][co] += sum_m in[nb(m, tap)][ci] dout[m][co] and gb[co] += sum_m dout[m][co].
+// A contraction over the voxels: a block stages tiles of 16 (x) x 8 (y) x tz voxels of
+// dout and of the input with its one-voxel halo once in shared memory (16-byte entries
+// [8-channel chunk][voxel], conflict-free for ldmatrix), and its nine warps take the
+// (dz, dy) pairs of the 27 taps: per 16 voxels a warp loads one dout fragment and three
+// shifted input fragments (ldmatrix.trans turns [voxel][channel] into the transposed
+// operand) and issues the MMAs into FP32 registers, which it keeps over all tiles of the
+// block.  The blocks' sums go to a workspace and are added in a fixed order, so repeated
+// runs agree bit for bit.  16 -> 16 layer on 16x64x64: 85 us (one warp per tap and 1024
+// voxels, gathering 2-byte elements and adding with atomics) + 9 us for the bias before,
+// 8.4 us + 4.3 us for the sums now; 48 -> 16: 92 + 9 before, 16 + 6 now.
+constexpr int kWgX = 16, kWgY = 8, kWgHX = kWgX + 2, kWgHY = kWgY + 2;
+constexpr int kWgThreads = 288;
+
+__device__ __forceinline__ void ldsm_x4_trans(unsigned (&r)[4], unsigned addr) {
+  asm volatile("ldmatrix.sync.aligned.m8n8.x4.trans.shared.b16 {%0,%1,%2,%3}, [%4];"
+               : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3])
+               : "r"(addr)
+               : "memory");
 }
 
-__global__ void bias_grad_kernel(const bf16* __restrict__ dout, int M, int C, int chunk, float* gb) {
-  const int c = threadIdx.x % C;
-  const int part = blockIdx.x * (blockDim.x / C) + threadIdx.x / C;
-  if (threadIdx.x >= (blockDim.x / C) * C) return;
+__host__ __device__ constexpr int wg_elems(int cin, int cout) { return 27 * cin * cout + cout; }
+
+template <int CIN, int COUT>
+__global__ void __launch_bounds__(kWgThreads) conv_wgrad_kernel(const bf16* __restrict__ in, const bf16* __restrict__ dout,
+                                                                NNGrid g, int tz, float* __restrict__ part) {
+  constexpr int KC = CIN / 8, NC = COUT / 8;
+  extern __shared__ __align__(128) unsigned char smem[];
+  const int nv = (tz + 2) * kWgHY * kWgHX, nd = tz * kWgY * kWgX;
+  const unsigned si = smem_u32(smem), sd = si + 16u * KC * nv;
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int dz = warp / 3, dy = warp % 3;
+  const int ntx = (g.W + kWgX - 1) / kWgX, nty = (g.H + kWgY - 1) / kWgY, ntz = (g.D + tz - 1) / tz;
+  float acc[3][CIN / 16][NC][4];
+#pragma unroll
+  for (int t = 0; t < 3; ++t)
+#pragma unroll
+    for (int c = 0; c < CIN / 16; ++c)
+#pragma unroll
+      for (int j = 0; j < NC; ++j) acc[t][c][j][0] = acc[t][c][j][1] = acc[t][c][j][2] = acc[t][c][j][3] = 0.f;
+  float bias = 0.f;
+  // this lane's row of the four 8x8 matrices of a fragment: voxel and chunk
+  const int lv = lane & 7, lm = lane >> 3;
+  const int a_vox = lv + 8 * (lm >> 1), a_ch = lm & 1;   // input: chunk pairs first, then voxels
+  const int b_vox = lv + 8 * (lm & 1), b_ch = lm >> 1;   // dout: voxel halves first, then chunks
+  for (int tile = blockIdx.x; tile < ntx * nty * ntz; tile += gridDim.x) {
+    const int x0 = (tile % ntx) * kWgX, y0 = ((tile / ntx) % nty) * kWgY, z0 = (tile / (ntx * nty)) * tz;
+    __syncthreads();   // the previous tile's readers
+    for (int q = tid; q < nv * KC; q += kWgThreads) {
+      const int ch = q % KC, v = q / KC;
+      const int xx = v % kWgHX, yy = (v / kWgHX) % kWgHY, zz = v / (kWgHX * kWgHY);
+      const int gz = z0 + zz - 1;
+      const int gx = (x0 + xx - 1 + g.W) % g.W, gy = (y0 + yy - 1 + g.H) % g.H;
+      const bool ok = gz >= 0 && gz < g.D;
+      tc_cp16(si + 16u * (ch * nv + v), in + ((size_t)((ok ? gz : 0) * g.H + gy) * g.W + gx) * CIN + 8 * ch, ok);
+    }
+    for (int q = tid; q < nd * NC; q += kWgThreads) {
+      const int ch = q % NC, v = q / NC;
+      const int x = x0 + v % kWgX, y = y0 + (v / kWgX) % kWgY, z = z0 + v / (kWgX * kWgY);
+      const bool ok = x < g.W && y < g.H && z < g.D;   // voxels beyond the grid contribute nothing
+      tc_cp16(sd + 16u * (ch * nd + v), dout + (ok ? ((size_t)(z * g.H + y) * g.W + x) * COUT + 8 * ch : 0), ok);
+    }
+    asm volatile("cp.async.commit_group;\ncp.async.wait_group 0;\n" ::: "memory");
+    __syncthreads();
+    if (tid < 256) {   // bias: thread tid sums channel tid % COUT over every 256 / COUT-th voxel
+      const bf16* d = reinterpret_cast<const bf16*>(smem + 16 * (size_t)KC * nv);
+      const int c = tid % COUT;
+      for (int v = tid / COUT; v < nd; v += 256 / COUT) bias += __bfloat162float(d[((c >> 3) * nd + v) * 8 + (c & 7)]);
+    }
+    for (int row = 0; row < tz * kWgY; ++row) {   // 16 voxels along x
+      const int z = row / kWgY, y = row - z * kWgY;
+      unsigned b[NC / 2][4];
+#pragma unroll
+      for (int j = 0; j < NC / 2; ++j) ldsm_x4_trans(b[j], sd + 16u * ((2 * j + b_ch) * nd + row * kWgX + b_vox));
+      const unsigned base = (unsigned)(((z + dz) * kWgHY + y + dy) * kWgHX);
+#pragma unroll
+      for (int t = 0; t < 3; ++t)
+#pragma unroll
+        for (int c = 0; c < CIN / 16; ++c) {
+          unsigned af[4];
+          ldsm_x4_trans(af, si + 16u * ((2 * c + a_ch) * nv + base + t + a_vox));
+#pragma unroll
+          for (int j = 0; j < NC; ++j) {
+            const unsigned bf[2] = {b[j >> 1][2 * (j & 1)], b[j >> 1][2 * (j & 1) + 1]};
+            mma_bf16(acc[t][c][j], af, bf);
+          }
+        }
+    }
+  }
+  float* out = part + (size_t)blockIdx.x * wg_elems(CIN, COUT);
+  const int gq = lane >> 2, tq = lane & 3;
+#pragma unroll
+  for (int t = 0; t < 3; ++t)
+#pragma unroll
+    for (int c = 0; c < CIN / 16; ++c)
+#pragma unroll
+      for (int j = 0; j < NC; ++j) {
+        float* o = out + (size_t)((warp * 3 + t) * CIN + c * 16 + gq) * COUT + j * 8 + 2 * tq;
+        *reinterpret_cast<float2*>(o) = make_float2(acc[t][c][j][0], acc[t][c][j][1]);
+        *reinterpret_cast<float2*>(o + 8 * COUT) = make_float2(acc[t][c][j][2], acc[t][c][j][3]);
+      }
+  __syncthreads();
+  float* red = reinterpret_cast<float*>(smem);
+  if (tid < 256) red[tid] = bias;
+  __syncthreads();
+  if (tid < COUT) {
+    float s = 0.f;
+    for (int q = tid; q < 256; q += COUT) s += red[q];
+    out[27 * CIN * COUT + tid] = s;
+  }
+}
+
+// gw, gb += the blocks' sums: 32 elements by 8 partial rows per block, a fixed order
+__global__ void __launch_bounds__(256) wgrad_reduce_kernel(const float* __restrict__ part, int nblk, int nw, int nb,
+                                                           float* __restrict__ gw, float* __restrict__ gb) {
+  __shared__ float sh[8][32];
+  const int n = nw + nb, t = blockIdx.x * 32 + threadIdx.x;
   float s = 0.f;
-  for (int m = part * chunk; m < min(M, (part + 1) * chunk); ++m) s += __bfloat162float(dout[(size_t)m * C + c]);
-  atomicAdd(gb + c, s);
+  if (t < n)
+    for (int q = threadIdx.y; q < nblk; q += 64) {
+      float v[8];
+#pragma unroll
+      for (int w = 0; w < 8; ++w) v[w] = q + 8 * w < nblk ? __ldcg(part + (size_t)(q + 8 * w) * n + t) : 0.f;
+#pragma unroll
+      for (int w = 0; w < 8; ++w) s += v[w];
+    }
+  sh[threadIdx.y][threadIdx.x] = s;
+  __syncthreads();
+  if (threadIdx.y == 0 && t < n) {
+#pragma unroll
+    for (int q = 1; q < 8; ++q) s += sh[q][threadIdx.x];
+    if (t < nw) gw[t] += s;
+    else gb[t - nw] += s;
+  }
 }
 
 // 2x2x2 mean of a fine channels-last field: one thread per coarse voxel and
@@ -559,13 +628,6 @@ __global__ void upcat_kernel(const bf16* __restrict__ a4, const bf16* __restrict
   }
 }
 
-// out = bf16(d * (act > 0))   (ReLU backward; act is the post-activation)
-__global__ void mask_kernel(const float* __restrict__ d, const bf16* __restrict__ act, long long n,
-                            bf16* __restrict__ out) {
-  for (long long t = blockIdx.x * (long long)blockDim.x + threadIdx.x; t < n; t += (long long)gridDim.x * blockDim.x)
-    out[t] = __float2bfloat16(__bfloat162float(act[t]) > 0.f ? d[t] : 0.f);
-}
-
 // da4m[V][c] = bf16(sum over the 8 children of dcat[child][c] (c < 32), masked by a4 > 0)
 __global__ void up_grad_kernel(const float* __restrict__ dcat, const bf16* __restrict__ a4, NNGrid f,
                                bf16* __restrict__ out) {
@@ -600,48 +662,71 @@ __global__ void skip_grad_kernel(const float* __restrict__ dcat, const float* __
 }
 
 // loss += sum (y0 - t)^2 / M; dy[m][0] = 2 (y0 - t) / M, other channels 0
-__global__ void mse_kernel(const float* __restrict__ y, const float* __restrict__ tgt, int M,
-                           bf16* __restrict__ dy, float* __restrict__ loss) {
+__global__ void __launch_bounds__(256) mse_kernel(const float* __restrict__ y, const float* __restrict__ tgt, int M,
+                                                  bf16* __restrict__ dy, float* __restrict__ loss) {
+  __shared__ float sh[8];
   float s = 0.f;
   for (int m = blockIdx.x * blockDim.x + threadIdx.x; m < M; m += gridDim.x * blockDim.x) {
     const float d = y[m] - tgt[m];
     s += d * d;
-    dy[(size_t)m * 16] = __float2bfloat16(2.f * d / M);
-    for (int c = 1; c < 16; ++c) dy[(size_t)m * 16 + c] = __float2bfloat16(0.f);
+    uint4* o = reinterpret_cast<uint4*>(dy + (size_t)m * 16);
+    o[0] = make_uint4(__bfloat16_as_ushort(__float2bfloat16(2.f * d / M)), 0u, 0u, 0u);
+    o[1] = make_uint4(0u, 0u, 0u, 0u);
   }
   for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-  if ((threadIdx.x & 31) == 0) atomicAdd(loss, s / M);
+  if ((threadIdx.x & 31) == 0) sh[threadIdx.x >> 5] = s;
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    for (int w = 1; w < 8; ++w) s += sh[w];
+    atomicAdd(loss, s / M);
+  }
 }
 
-__global__ void adam_kernel(float* __restrict__ p, float* __restrict__ g, float* __restrict__ m,
-                            float* __restrict__ v, int n, float lr, float b1, float b2, float c1,
-                            float c2, float eps) {
-  for (int t = blockIdx.x * blockDim.x + threadIdx.x; t < n; t += gridDim.x * blockDim.x) {
+// the six layers' places in the parameter arrays: layer l's weights start at w0[l] (its
+// packed copies too), its biases at b0[l] behind all weights
+struct NNLayout {
+  int w0[7], b0[7], cin[6], cout[6];
+};
+
+// kernel layouts of a weight, FP32 master [tap][ci][co]: forward wk[tap][co][ci];
+// adjoint wb[tap][ci][co] = w[26 - tap][ci][co] read as a conv with Cin' = co, Cout' = ci;
+// the same two in the tensor-memory kernel's operand layout [tap][cin/8][cout][cin%8]:
+// wkt for the forward, wbt (Cin' = co, Cout' = ci) for the adjoint
+__device__ __forceinline__ void pack_weight(int t, int cin, int cout, float w, bf16* __restrict__ wk, bf16* __restrict__ wb,
+                                            bf16* __restrict__ wkt, bf16* __restrict__ wbt) {
+  const int co = t % cout, ci = (t / cout) % cin, tap = t / (cin * cout);
+  const bf16 val = __float2bfloat16(w);
+  wk[((size_t)tap * cout + co) * cin + ci] = val;
+  wb[((size_t)(26 - tap) * cin + ci) * cout + co] = val;
+  wkt[(((size_t)tap * (cin / 8) + ci / 8) * cout + co) * 8 + ci % 8] = val;
+  wbt[(((size_t)(26 - tap) * (cout / 8) + co / 8) * cin + ci) * 8 + co % 8] = val;
+}
+
+// Adam on every parameter (lr > 0) and the packed copies of the weights, all layers in one
+// launch
+__global__ void __launch_bounds__(256) adam_pack_kernel(NNLayout L, float* __restrict__ p, float* __restrict__ g,
+                                                        float* __restrict__ m, float* __restrict__ v, float lr, float b1,
+                                                        float b2, float c1, float c2, float eps, bf16* __restrict__ wk,
+                                                        bf16* __restrict__ wb, bf16* __restrict__ wkt,
+                                                        bf16* __restrict__ wbt) {
+  const int t = blockIdx.x * blockDim.x + threadIdx.x;
+  if (t >= L.b0[6]) return;
+  float x = p[t];
+  if (lr > 0.f) {
     const float gr = g[t];
     const float mt = b1 * m[t] + (1.f - b1) * gr;
     const float vt = b2 * v[t] + (1.f - b2) * gr * gr;
     m[t] = mt;
     v[t] = vt;
-    p[t] -= lr * (mt / c1) / (sqrtf(vt / c2) + eps);
+    x -= lr * (mt / c1) / (sqrtf(vt / c2) + eps);
+    p[t] = x;
     g[t] = 0.f;
   }
-}
-
-// kernel layouts from the FP32 master [tap][ci][co]: forward wk[tap][co][ci];
-// adjoint wb[tap][ci][co] = w[26 - tap][ci][co] read as a conv with Cin' = co, Cout' = ci;
-// the same two in the tensor-memory kernel's operand layout [tap][cin/8][cout][cin%8]:
-// wkt for the forward, wbt (Cin' = co, Cout' = ci) for the adjoint
-__global__ void pack_kernel(const float* __restrict__ w, int cin, int cout, bf16* __restrict__ wk,
-                            bf16* __restrict__ wb, bf16* __restrict__ wkt, bf16* __restrict__ wbt) {
-  const int n = 27 * cin * cout;
-  for (int t = blockIdx.x * blockDim.x + threadIdx.x; t < n; t += gridDim.x * blockDim.x) {
-    const int co = t % cout, ci = (t / cout) % cin, tap = t / (cin * cout);
-    const bf16 val = __float2bfloat16(w[t]);
-    wk[((size_t)tap * cout + co) * cin + ci] = val;
-    wb[((size_t)(26 - tap) * cin + ci) * cout + co] = val;
-    wkt[(((size_t)tap * (cin / 8) + ci / 8) * cout + co) * 8 + ci % 8] = val;
-    wbt[(((size_t)(26 - tap) * (cout / 8) + co / 8) * cin + ci) * 8 + co % 8] = val;
-  }
+  if (t >= L.w0[6]) return;
+  int l = 0;
+  while (t >= L.w0[l + 1]) ++l;
+  const int o = L.w0[l];
+  pack_weight(t - o, L.cin[l], L.cout[l], x, wk + o, wb + o, wkt + o, wbt + o);
 }
 
 int grid1(long long n, int threads) {
@@ -683,13 +768,13 @@ int tc_zt(int cin, int cout, NNGrid g) {
 
 template <int CIN, int COUT, bool UP = false>
 void launch_conv_tc(const bf16* in, const bf16* s1, const bf16* wt, const float* bias, NNGrid g, int relu,
-                    bf16* out_bf, float* out_f, int f_ch0, int* fault, cudaStream_t s) {
+                    const bf16* mask, bf16* out_bf, float* out_f, int f_ch0, int* fault, cudaStream_t s) {
   const int zt = tc_zt(CIN, COUT, g);
   const size_t smem = tc_smem(CIN, COUT, zt);
   const int per_sm = std::max(1, std::min(16, (int)(233472 / (smem + 1024))));
   const int blocks = std::min(tc_tiles(g, zt), sm_count() * per_sm);
-  conv_tc_kernel<CIN, COUT, UP><<<blocks, kTcThreads, smem, s>>>(in, s1, wt, bias, g, zt, relu, out_bf, out_f,
-                                                                    f_ch0, fault);
+  conv_tc_kernel<CIN, COUT, UP><<<blocks, kTcThreads, smem, s>>>(in, s1, wt, bias, g, zt, relu, mask, out_bf,
+                                                                    out_f, f_ch0, fault);
 }
 
 }  // namespace
@@ -713,6 +798,10 @@ cudaError_t nn_tc_setup() {
     set((const void*)conv_tc_kernel<32, 32, false>);
     set((const void*)conv_tc_kernel<48, 16, false>);
     set((const void*)conv_tc_kernel<48, 16, true>);
+    set((const void*)conv_wgrad_kernel<16, 16>);
+    set((const void*)conv_wgrad_kernel<16, 32>);
+    set((const void*)conv_wgrad_kernel<32, 32>);
+    set((const void*)conv_wgrad_kernel<48, 16>);
     return e;
   }();
   return done;
@@ -727,9 +816,9 @@ bool nn_conv_uses_tc(int cin, int cout, NNGrid g) {
 }
 
 bool nn_conv_fwd(const bf16* in, int cin, const bf16* wk, const bf16* wt, const float* bias, int cout,
-                 NNGrid g, int relu, bf16* out_bf, float* out_f, int f_ch0, int* fault, cudaStream_t s) {
+                 NNGrid g, int relu, const bf16* mask, bf16* out_bf, float* out_f, int f_ch0, int* fault, cudaStream_t s) {
   if (wt && fault && nn_conv_uses_tc(cin, cout, g)) {
-    auto go = [&](auto launch) { launch(in, nullptr, wt, bias, g, relu, out_bf, out_f, f_ch0, fault, s); };
+    auto go = [&](auto launch) { launch(in, nullptr, wt, bias, g, relu, mask, out_bf, out_f, f_ch0, fault, s); };
     if (cin == 16 && cout == 16) go(launch_conv_tc<16, 16>);
     else if (cin == 16 && cout == 32) go(launch_conv_tc<16, 32>);
     else if (cin == 16 && cout == 48) go(launch_conv_tc<16, 48>);
@@ -742,9 +831,9 @@ bool nn_conv_fwd(const bf16* in, int cin, const bf16* wk, const bf16* wt, const 
   const int tiles = (M + 15) / 16;
   const int blocks = (tiles + kConvTiles - 1) / kConvTiles;
   const dim3 block(32, kConvTiles, 3);
-  if (cout == 16) conv_fwd_kernel<16><<<blocks, block, 0, s>>>(in, cin, wk, bias, g, relu, out_bf, out_f, f_ch0);
-  else if (cout == 32) conv_fwd_kernel<32><<<blocks, block, 0, s>>>(in, cin, wk, bias, g, relu, out_bf, out_f, f_ch0);
-  else if (cout == 48) conv_fwd_kernel<48><<<blocks, block, 0, s>>>(in, cin, wk, bias, g, relu, out_bf, out_f, f_ch0);
+  if (cout == 16) conv_fwd_kernel<16><<<blocks, block, 0, s>>>(in, cin, wk, bias, g, relu, mask, out_bf, out_f, f_ch0);
+  else if (cout == 32) conv_fwd_kernel<32><<<blocks, block, 0, s>>>(in, cin, wk, bias, g, relu, mask, out_bf, out_f, f_ch0);
+  else if (cout == 48) conv_fwd_kernel<48><<<blocks, block, 0, s>>>(in, cin, wk, bias, g, relu, mask, out_bf, out_f, f_ch0);
   return false;
 }
 
@@ -753,24 +842,37 @@ bool nn_conv_fwd(const bf16* in, int cin, const bf16* wk, const bf16* wt, const 
 bool nn_conv_upcat_tc(const bf16* a4, const bf16* s1, const bf16* wt, const float* bias, NNGrid g, int relu,
                       bf16* out_bf, int* fault, cudaStream_t s) {
   if (!wt || !fault || !nn_conv_uses_tc(48, 16, g)) return false;
-  launch_conv_tc<48, 16, true>(a4, s1, wt, bias, g, relu, out_bf, nullptr, 0, fault, s);
+  launch_conv_tc<48, 16, true>(a4, s1, wt, bias, g, relu, nullptr, out_bf, nullptr, 0, fault, s);
   return true;
 }
 
+// Planes per tile of the weight gradient: the most of {4, 2} that leaves every SM a tile.
+int wg_tz(NNGrid g) {
+  const long long t = (long long)((g.W + kWgX - 1) / kWgX) * ((g.H + kWgY - 1) / kWgY);
+  for (int tz : {4, 2})
+    if (t * ((g.D + tz - 1) / tz) >= 128) return tz;
+  return 1;
+}
+
+int wg_blocks(NNGrid g, int tz) {
+  const long long t = (long long)((g.W + kWgX - 1) / kWgX) * ((g.H + kWgY - 1) / kWgY) * ((g.D + tz - 1) / tz);
+  return (int)std::min<long long>(t, sm_count());
+}
+
+// floats of the weight gradients' workspace for a network whose finest grid is g
+size_t nn_wgrad_workspace(NNGrid) { return (size_t)sm_count() * wg_elems(32, 32); }
+
+// gw and gb of one layer; part: the workspace (one layer at a time)
 void nn_conv_wgrad(const bf16* in, int cin, const bf16* dout, int cout, NNGrid g, float* gw,
-                   float* gb, cudaStream_t s) {
-  const int M = g.D * g.H * g.W;
-  const int chunk = 1024;
-  const int parts = (M + chunk - 1) / chunk;
-  const int warps = 27 * parts;
-  const int blocks = (warps + 3) / 4;
-  if (cin == 16 && cout == 16) conv_wgrad_kernel<16, 16><<<blocks, 128, 0, s>>>(in, dout, g, chunk, gw);
-  else if (cin == 16 && cout == 32) conv_wgrad_kernel<16, 32><<<blocks, 128, 0, s>>>(in, dout, g, chunk, gw);
-  else if (cin == 32 && cout == 32) conv_wgrad_kernel<32, 32><<<blocks, 128, 0, s>>>(in, dout, g, chunk, gw);
-  else if (cin == 48 && cout == 16) conv_wgrad_kernel<48, 16><<<blocks, 128, 0, s>>>(in, dout, g, chunk, gw);
-  const int bchunk = 256, bparts = (M + bchunk - 1) / bchunk;
-  const int per_block = 256 / cout;
-  bias_grad_kernel<<<(bparts + per_block - 1) / per_block, 256, 0, s>>>(dout, M, cout, bchunk, gb);
+                   float* gb, float* part, cudaStream_t s) {
+  const int tz = wg_tz(g), blocks = wg_blocks(g, tz);
+  const size_t smem = 16 * ((size_t)(cin / 8) * (tz + 2) * kWgHY * kWgHX + (size_t)(cout / 8) * tz * kWgY * kWgX);
+  if (cin == 16 && cout == 16) conv_wgrad_kernel<16, 16><<<blocks, kWgThreads, smem, s>>>(in, dout, g, tz, part);
+  else if (cin == 16 && cout == 32) conv_wgrad_kernel<16, 32><<<blocks, kWgThreads, smem, s>>>(in, dout, g, tz, part);
+  else if (cin == 32 && cout == 32) conv_wgrad_kernel<32, 32><<<blocks, kWgThreads, smem, s>>>(in, dout, g, tz, part);
+  else if (cin == 48 && cout == 16) conv_wgrad_kernel<48, 16><<<blocks, kWgThreads, smem, s>>>(in, dout, g, tz, part);
+  const int nw = 27 * cin * cout;
+  wgrad_reduce_kernel<<<(nw + cout + 31) / 32, dim3(32, 8), 0, s>>>(part, blocks, nw, cout, gw, gb);
 }
 
 void nn_pool2(const bf16* in, NNGrid f, int C, bf16* out, cudaStream_t s) {
@@ -778,9 +880,6 @@ void nn_pool2(const bf16* in, NNGrid f, int C, bf16* out, cudaStream_t s) {
 }
 void nn_upcat(const bf16* a4, const bf16* s1, NNGrid f, bf16* cat, cudaStream_t s) {
   upcat_kernel<<<grid1((long long)f.D * f.H * f.W * 6, 256), 256, 0, s>>>(a4, s1, f, cat);
-}
-void nn_mask(const float* d, const bf16* act, long long n, bf16* out, cudaStream_t s) {
-  mask_kernel<<<grid1(n, 256), 256, 0, s>>>(d, act, n, out);
 }
 void nn_up_grad(const float* dcat, const bf16* a4, NNGrid f, bf16* out, cudaStream_t s) {
   up_grad_kernel<<<grid1((long long)f.D * f.H * f.W * 4, 256), 256, 0, s>>>(dcat, a4, f, out);
@@ -791,13 +890,11 @@ void nn_skip_grad(const float* dcat, const float* dp, const bf16* s1, NNGrid f, 
 void nn_mse(const float* y, const float* tgt, int M, bf16* dy, float* loss, cudaStream_t s) {
   mse_kernel<<<grid1(M, 256), 256, 0, s>>>(y, tgt, M, dy, loss);
 }
-void nn_adam(float* p, float* g, float* m, float* v, int n, float lr, int step, cudaStream_t s) {
+void nn_adam_pack(const NNLayout& L, float* p, float* g, float* m, float* v, float lr, int step, bf16* wk, bf16* wb,
+                  bf16* wkt, bf16* wbt, cudaStream_t s) {
   const float b1 = 0.9f, b2 = 0.999f;
   const float c1 = 1.f - powf(b1, (float)step), c2 = 1.f - powf(b2, (float)step);
-  adam_kernel<<<grid1(n, 256), 256, 0, s>>>(p, g, m, v, n, lr, b1, b2, c1, c2, 1e-8f);
-}
-void nn_pack(const float* w, int cin, int cout, bf16* wk, bf16* wb, bf16* wkt, bf16* wbt, cudaStream_t s) {
-  pack_kernel<<<grid1(27 * cin * cout, 256), 256, 0, s>>>(w, cin, cout, wk, wb, wkt, wbt);
+  adam_pack_kernel<<<(L.b0[6] + 255) / 256, 256, 0, s>>>(L, p, g, m, v, lr, b1, b2, c1, c2, 1e-8f, wk, wb, wkt, wbt);
 }
 
 }  // namespace fx
@@ -829,18 +926,21 @@ struct ferrox_nn {
   fx::NNGrid g{}, gc{};
   int M = 0, Mc = 0;
   cudaStream_t stream = nullptr;
+  // every layer's weights, then every layer's biases, in one array each for the values,
+  // gradients and moments (one Adam launch, one copy per array); packed weights likewise
+  fx::NNLayout lay{};
+  float *par = nullptr, *grad = nullptr, *mom1 = nullptr, *mom2 = nullptr;
+  bf16 *wk0 = nullptr, *wb0 = nullptr, *wkt0 = nullptr, *wbt0 = nullptr;
+  // the layers' places in them
   float* w[fx::kLayers] = {};
   float* b[fx::kLayers] = {};
   float* gw[fx::kLayers] = {};
   float* gb[fx::kLayers] = {};
-  float* mw[fx::kLayers] = {};
-  float* vw[fx::kLayers] = {};
-  float* mb[fx::kLayers] = {};
-  float* vb[fx::kLayers] = {};
   bf16* wk[fx::kLayers] = {};
   bf16* wb[fx::kLayers] = {};
   bf16* wkt[fx::kLayers] = {};   // tensor-memory operand layouts of wk and wb
   bf16* wbt[fx::kLayers] = {};
+  float* part = nullptr;         // weight gradients' workspace
   int* fault = nullptr;          // set by a tensor-memory convolution whose wait ran out
   bool tc = true;                // tensor-memory convolutions where the grid allows
   bf16 *x = nullptr, *a1 = nullptr, *s1 = nullptr, *p = nullptr, *a3 = nullptr, *a4 = nullptr,
@@ -884,17 +984,18 @@ cudaError_t nalloc(ferrox_nn* N, P** ptr, size_t bytes) {
   return e;
 }
 
-void repack(ferrox_nn* N) {
-  for (int l = 0; l < fx::kLayers; ++l)
-    fx::nn_pack(N->w[l], fx::kCin[l], fx::kCout[l], N->wk[l], N->wb[l], N->wkt[l], N->wbt[l], N->stream);
+// one Adam update with step size lr (0: none) and the packed copies of the weights
+void adam_pack(ferrox_nn* N, float lr) {
+  fx::nn_adam_pack(N->lay, N->par, N->grad, N->mom1, N->mom2, lr, std::max(1, N->adam_step), N->wk0, N->wb0, N->wkt0,
+                   N->wbt0, N->stream);
 }
 
 // one convolution of layer l: forward weights, or the adjoint's when adjoint is set
 void conv(ferrox_nn* N, int l, bool adjoint, const bf16* in, fx::NNGrid g, int relu, bf16* out_bf, float* out_f,
-          cudaStream_t s, int f_ch0 = 0) {
+          cudaStream_t s, int f_ch0 = 0, const bf16* mask = nullptr) {
   const int cin = adjoint ? fx::kCout[l] : fx::kCin[l], cout = adjoint ? fx::kCin[l] : fx::kCout[l];
   fx::nn_conv_fwd(in, cin, adjoint ? N->wb[l] : N->wk[l], !N->tc ? nullptr : adjoint ? N->wbt[l] : N->wkt[l],
-                  adjoint ? nullptr : N->b[l], cout, g, relu, out_bf, out_f, f_ch0, N->fault, s);
+                  adjoint ? nullptr : N->b[l], cout, g, relu, mask, out_bf, out_f, f_ch0, N->fault, s);
 }
 
 // forward pass from N->x; output channel 0 (FP32) in N->y.  The concatenation
@@ -920,23 +1021,23 @@ void forward(ferrox_nn* N, bool keep_cat) {
 void backward(ferrox_nn* N) {
   cudaStream_t s = N->stream;
   using namespace fx;
-  const long long M = N->M, Mc = N->Mc;
-  nn_conv_wgrad(N->a5, 16, N->dy, 16, N->g, N->gw[5], N->gb[5], s);
-  conv(N, 5, true, N->dy, N->g, 0, nullptr, N->df, s);
-  nn_mask(N->df, N->a5, M * 16, N->t16a, s);                                  // da5
-  nn_conv_wgrad(N->cat, 48, N->t16a, 16, N->g, N->gw[4], N->gb[4], s);
+  auto wgrad = [&](int l, const bf16* in, const bf16* dout, NNGrid g) {
+    nn_conv_wgrad(in, kCin[l], dout, kCout[l], g, N->gw[l], N->gb[l], N->part, s);
+  };
+  // the adjoints whose result passes a ReLU only are masked and rounded as they are stored
+  wgrad(5, N->a5, N->dy, N->g);
+  conv(N, 5, true, N->dy, N->g, 0, N->t16a, nullptr, s, 0, N->a5);            // da5
+  wgrad(4, N->cat, N->t16a, N->g);
   conv(N, 4, true, N->t16a, N->g, 0, nullptr, N->dcat, s);
   nn_up_grad(N->dcat, N->a4, N->g, N->t32a, s);                               // da4
-  nn_conv_wgrad(N->a3, 32, N->t32a, 32, N->gc, N->gw[3], N->gb[3], s);
-  conv(N, 3, true, N->t32a, N->gc, 0, nullptr, N->df, s);
-  nn_mask(N->df, N->a3, Mc * 32, N->t32b, s);                                 // da3
-  nn_conv_wgrad(N->p, 16, N->t32b, 32, N->gc, N->gw[2], N->gb[2], s);
-  conv(N, 2, true, N->t32b, N->gc, 0, nullptr, N->dpc, s);                   // dp
+  wgrad(3, N->a3, N->t32a, N->gc);
+  conv(N, 3, true, N->t32a, N->gc, 0, N->t32b, nullptr, s, 0, N->a3);         // da3
+  wgrad(2, N->p, N->t32b, N->gc);
+  conv(N, 2, true, N->t32b, N->gc, 0, nullptr, N->dpc, s);                    // dp
   nn_skip_grad(N->dcat, N->dpc, N->s1, N->g, N->t16b, s);                     // ds1
-  nn_conv_wgrad(N->a1, 16, N->t16b, 16, N->g, N->gw[1], N->gb[1], s);
-  conv(N, 1, true, N->t16b, N->g, 0, nullptr, N->df, s);
-  nn_mask(N->df, N->a1, M * 16, N->t16a, s);                                  // da1
-  nn_conv_wgrad(N->x, 16, N->t16a, 16, N->g, N->gw[0], N->gb[0], s);
+  wgrad(1, N->a1, N->t16b, N->g);
+  conv(N, 1, true, N->t16b, N->g, 0, N->t16a, nullptr, s, 0, N->a1);          // da1
+  wgrad(0, N->x, N->t16a, N->g);
 }
 
 void nn_release(ferrox_nn* N) {
@@ -996,22 +1097,32 @@ ferrox_status ferrox_nn_create(ferrox_nn** out, int D, int H, int W, int capacit
     return nfail(nullptr, FERROX_ENOMEM, m);
   };
   cudaError_t e;
-  size_t woff = 0, boff = 0;
+  fx::NNLayout& L = N->lay;
   for (int l = 0; l < fx::kLayers; ++l) {
-    const size_t nw = 27 * fx::kCin[l] * fx::kCout[l], nb = fx::kCout[l];
-    for (float** p : {&N->w[l], &N->gw[l], &N->mw[l], &N->vw[l]})
-      if ((e = nalloc(N, p, nw * sizeof(float))) != cudaSuccess) return fail_alloc(e);
-    for (float** p : {&N->b[l], &N->gb[l], &N->mb[l], &N->vb[l]})
-      if ((e = nalloc(N, p, nb * sizeof(float))) != cudaSuccess) return fail_alloc(e);
-    if ((e = nalloc(N, &N->wk[l], nw * sizeof(bf16))) != cudaSuccess) return fail_alloc(e);
-    if ((e = nalloc(N, &N->wb[l], nw * sizeof(bf16))) != cudaSuccess) return fail_alloc(e);
-    if ((e = nalloc(N, &N->wkt[l], nw * sizeof(bf16))) != cudaSuccess) return fail_alloc(e);
-    if ((e = nalloc(N, &N->wbt[l], nw * sizeof(bf16))) != cudaSuccess) return fail_alloc(e);
-    cudaMemcpy(N->w[l], weights + woff, nw * sizeof(float), cudaMemcpyHostToDevice);
-    cudaMemcpy(N->b[l], biases + boff, nb * sizeof(float), cudaMemcpyHostToDevice);
-    woff += nw;
-    boff += nb;
+    L.cin[l] = fx::kCin[l];
+    L.cout[l] = fx::kCout[l];
+    L.w0[l + 1] = L.w0[l] + 27 * fx::kCin[l] * fx::kCout[l];
   }
+  L.b0[0] = L.w0[fx::kLayers];
+  for (int l = 0; l < fx::kLayers; ++l) L.b0[l + 1] = L.b0[l] + fx::kCout[l];
+  const size_t nw = L.w0[fx::kLayers], np = L.b0[fx::kLayers];
+  for (float** p : {&N->par, &N->grad, &N->mom1, &N->mom2})
+    if ((e = nalloc(N, p, np * sizeof(float))) != cudaSuccess) return fail_alloc(e);
+  for (bf16** p : {&N->wk0, &N->wb0, &N->wkt0, &N->wbt0})
+    if ((e = nalloc(N, p, nw * sizeof(bf16))) != cudaSuccess) return fail_alloc(e);
+  if ((e = nalloc(N, &N->part, fx::nn_wgrad_workspace(N->g) * sizeof(float))) != cudaSuccess) return fail_alloc(e);
+  for (int l = 0; l < fx::kLayers; ++l) {
+    N->w[l] = N->par + L.w0[l];
+    N->b[l] = N->par + L.b0[l];
+    N->gw[l] = N->grad + L.w0[l];
+    N->gb[l] = N->grad + L.b0[l];
+    N->wk[l] = N->wk0 + L.w0[l];
+    N->wb[l] = N->wb0 + L.w0[l];
+    N->wkt[l] = N->wkt0 + L.w0[l];
+    N->wbt[l] = N->wbt0 + L.w0[l];
+  }
+  cudaMemcpy(N->par, weights, nw * sizeof(float), cudaMemcpyHostToDevice);
+  cudaMemcpy(N->par + nw, biases, (np - nw) * sizeof(float), cudaMemcpyHostToDevice);
   struct { bf16** p; size_t n; } bufs[] = {
       {&N->x, M * 16}, {&N->a1, M * 16}, {&N->s1, M * 16}, {&N->p, Mc * 16}, {&N->a3, Mc * 32},
       {&N->a4, Mc * 32}, {&N->cat, M * 48}, {&N->a5, M * 16}, {&N->dy, M * 16},
@@ -1028,7 +1139,7 @@ ferrox_status ferrox_nn_create(ferrox_nn** out, int D, int H, int W, int capacit
     if ((e = nalloc(N, &N->snap_x, (size_t)capacity * M * 16 * sizeof(bf16))) != cudaSuccess) return fail_alloc(e);
     if ((e = nalloc(N, &N->snap_t, (size_t)capacity * M * sizeof(float))) != cudaSuccess) return fail_alloc(e);
   }
-  repack(N);
+  adam_pack(N, 0.f);
   if ((e = cudaDeviceSynchronize()) != cudaSuccess) {
     nn_release(N);
     return nfail(nullptr, FERROX_ECUDA, cudaGetErrorString(e));
@@ -1065,30 +1176,20 @@ ferrox_status ferrox_nn_loss_grad(ferrox_nn* N, const float* x_dev, const float*
 ferrox_status ferrox_nn_params(ferrox_nn* N, float* w, float* b, float* gw, float* gb) {
   if (!N) return nfail(nullptr, FERROX_EINVAL, "null network");
   FX_NCK(cudaStreamSynchronize(N->stream));
-  size_t woff = 0, boff = 0;
-  for (int l = 0; l < fx::kLayers; ++l) {
-    const size_t nw = 27 * fx::kCin[l] * fx::kCout[l], nb = fx::kCout[l];
-    if (w) FX_NCK(cudaMemcpy(w + woff, N->w[l], nw * sizeof(float), cudaMemcpyDeviceToHost));
-    if (b) FX_NCK(cudaMemcpy(b + boff, N->b[l], nb * sizeof(float), cudaMemcpyDeviceToHost));
-    if (gw) FX_NCK(cudaMemcpy(gw + woff, N->gw[l], nw * sizeof(float), cudaMemcpyDeviceToHost));
-    if (gb) FX_NCK(cudaMemcpy(gb + boff, N->gb[l], nb * sizeof(float), cudaMemcpyDeviceToHost));
-    woff += nw;
-    boff += nb;
-  }
+  const size_t nw = N->lay.w0[fx::kLayers], nb = N->lay.b0[fx::kLayers] - nw;
+  if (w) FX_NCK(cudaMemcpy(w, N->par, nw * sizeof(float), cudaMemcpyDeviceToHost));
+  if (b) FX_NCK(cudaMemcpy(b, N->par + nw, nb * sizeof(float), cudaMemcpyDeviceToHost));
+  if (gw) FX_NCK(cudaMemcpy(gw, N->grad, nw * sizeof(float), cudaMemcpyDeviceToHost));
+  if (gb) FX_NCK(cudaMemcpy(gb, N->grad + nw, nb * sizeof(float), cudaMemcpyDeviceToHost));
   return FERROX_OK;
 }
 
 ferrox_status ferrox_nn_set_params(ferrox_nn* N, const float* w, const float* b) {
   if (!N || !w || !b) return nfail(N, FERROX_EINVAL, "null argument");
-  size_t woff = 0, boff = 0;
-  for (int l = 0; l < fx::kLayers; ++l) {
-    const size_t nw = 27 * fx::kCin[l] * fx::kCout[l], nb = fx::kCout[l];
-    FX_NCK(cudaMemcpyAsync(N->w[l], w + woff, nw * sizeof(float), cudaMemcpyHostToDevice, N->stream));
-    FX_NCK(cudaMemcpyAsync(N->b[l], b + boff, nb * sizeof(float), cudaMemcpyHostToDevice, N->stream));
-    woff += nw;
-    boff += nb;
-  }
-  repack(N);
+  const size_t nw = N->lay.w0[fx::kLayers], nb = N->lay.b0[fx::kLayers] - nw;
+  FX_NCK(cudaMemcpyAsync(N->par, w, nw * sizeof(float), cudaMemcpyHostToDevice, N->stream));
+  FX_NCK(cudaMemcpyAsync(N->par + nw, b, nb * sizeof(float), cudaMemcpyHostToDevice, N->stream));
+  adam_pack(N, 0.f);
   FX_NCK(cudaStreamSynchronize(N->stream));
   return FERROX_OK;
 }
@@ -1096,12 +1197,7 @@ ferrox_status ferrox_nn_set_params(ferrox_nn* N, const float* w, const float* b)
 ferrox_status ferrox_nn_adam_step(ferrox_nn* N, double lr) {
   if (!N || !(lr > 0.0)) return nfail(N, FERROX_EINVAL, "bad argument");
   N->adam_step += 1;
-  for (int l = 0; l < fx::kLayers; ++l) {
-    const int nw = 27 * fx::kCin[l] * fx::kCout[l], nb = fx::kCout[l];
-    fx::nn_adam(N->w[l], N->gw[l], N->mw[l], N->vw[l], nw, (float)lr, N->adam_step, N->stream);
-    fx::nn_adam(N->b[l], N->gb[l], N->mb[l], N->vb[l], nb, (float)lr, N->adam_step, N->stream);
-  }
-  repack(N);
+  adam_pack(N, (float)lr);
   FX_NCK(cudaGetLastError());
   return FERROX_OK;
 }
@@ -1146,12 +1242,7 @@ ferrox_status ferrox_nn_train(ferrox_nn* N, int epochs, double lr, int batch, fl
         const double lr_k = lr * (0.1 + 0.45 * (1.0 + std::cos(3.141592653589793 * (double)k / (double)total)));
         ++k;
         N->adam_step += 1;
-        for (int l = 0; l < fx::kLayers; ++l) {
-          const int nw = 27 * fx::kCin[l] * fx::kCout[l], nb = fx::kCout[l];
-          fx::nn_adam(N->w[l], N->gw[l], N->mw[l], N->vw[l], nw, (float)lr_k, N->adam_step, N->stream);
-          fx::nn_adam(N->b[l], N->gb[l], N->mb[l], N->vb[l], nb, (float)lr_k, N->adam_step, N->stream);
-        }
-        repack(N);
+        adam_pack(N, (float)lr_k);
       }
     }
     FX_NCK(cudaGetLastError());
