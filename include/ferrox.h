@@ -490,15 +490,17 @@ ferrox_status ferrox_attach_nn(ferrox_ctx* ctx, ferrox_nn* nn, int mode);
  *   the caller's values.
  * It runs the same fused TDGL kernel, with its scratch (plane table, staging
  * copy of the new P, right-hand side) in one file-scope device array of about
- * 8.1 MB that every GPU loading the library holds until the process exits.
+ * 8.6 MB that every GPU loading the library holds until the process exits.
  * Limits: Nx*Ny*Nz <= FERROX_STATIC_MAX_CELLS and Nz <= FERROX_STATIC_MAX_PLANES;
  * larger grids are rejected with FERROX_EINVAL and a message.  No scratch
  * byte is read before the call writes it, so nothing needs clearing between
  * calls.  All calls share the one array: calls whose GPU work overlaps (two
  * streams, or two host threads) race and must be serialised by the caller.
  * The first call on each device looks up the array's device address with
- * that device current.  The plane table is copied from pageable host memory,
- * so the call waits for work already queued on the stream before it returns. */
+ * that device current.  The layers travel in a kernel's arguments, so the call
+ * returns without waiting; with more than 16 layers the plane tables are copied
+ * from pageable host memory, and the call waits for work already queued on the
+ * stream before it returns. */
 ferrox_status ferrox_tdgl_update_static(const ferrox_geometry* geom, double dt, double v_bottom,
                                         double v_top, double* P_dev, const double* phi_dev,
                                         void* cuda_stream);

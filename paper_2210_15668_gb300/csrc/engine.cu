@@ -94,6 +94,7 @@ struct ferrox_ctx {
   PlaneCarrierDF* carriers_df = nullptr;
   bool df_resid = false;              // the mixed form's Boltzmann carriers in double-float
   PlaneTDGL* planes_d = nullptr;
+  PlaneForce* force_d = nullptr;      // the FP64 TDGL update's table
   PlaneF32* planes_f32_d = nullptr;   // FP32 TDGL arithmetic only
   LevelDesc* lv_d = nullptr;
   LevelDesc* lvt_d = nullptr;
@@ -808,6 +809,12 @@ void enqueue_update(ferrox_ctx* c, cudaStream_t s) {
                    adapt_max(c) > 0 ? e : nullptr);
 }
 
+std::vector<PlaneForce> plane_forces(const std::vector<PlaneTDGL>& pl, double h, double dt) {
+  std::vector<PlaneForce> out;
+  for (const PlaneTDGL& p : pl) out.push_back(plane_force(p, 1.0 / (h * h), dt));
+  return out;
+}
+
 // The FP32 TDGL coefficients of each plane (see PlaneF32): the force's
 // coefficients rounded to FP32, d2z rewritten on differences, and the right-hand
 // side b = -(Pf(k + 1/2) - Pf(k - 1/2)) h/eps0 folded into weights of P_{k-1},
@@ -841,6 +848,7 @@ TDGLArgs tdgl_args(ferrox_ctx* c, int mode) {
   a.F_store = c->Fbuf;
   if (mode == 0 || mode == 1 || mode == 3) { a.P_in = c->P; a.P_out = c->Pbuf; a.P_base = nullptr; }
   else { a.P_in = c->Pbuf; a.P_out = c->P; a.P_base = c->P; }
+  a.force = c->force_d;
   a.planes_f32 = c->planes_f32_d;
   a.dtf = (float)a.dt; a.inv_hf = (float)a.inv_h; a.inv_h2f = (float)a.inv_h2;
   return a;
@@ -1248,7 +1256,7 @@ void release(ferrox_ctx* c) {
   for (auto g : ge) if (g) cudaGraphExecDestroy(g);
   for (auto g : gr) if (g) cudaGraphDestroy(g);
   void* ptrs[] = {c->b, c->Pbuf, c->Fbuf, c->phi_prev, c->e_arena, c->eb_arena, c->e_alt, c->r_arena, c->s_arena, c->coef, c->coef0, c->coef0s, c->bs, c->sinv0, c->coef_df, c->carriers_df,
-                  c->planes_d, c->planes_f32_d, c->lv_d, c->lvt_d, c->nn_scale, c->phi_guess, c->nn_pf, c->nn_stats, c->params_d, c->stats_d, c->partials_d, c->charge_d,
+                  c->planes_d, c->force_d, c->planes_f32_d, c->lv_d, c->lvt_d, c->nn_scale, c->phi_guess, c->nn_pf, c->nn_stats, c->params_d, c->stats_d, c->partials_d, c->charge_d,
                   c->charge_part_d, c->dense_d, c->dense_wide_d};
   for (void* p : ptrs) if (p) cudaFree(p);
   if (c->host_pinned) cudaFreeHost(c->host_pinned);
@@ -1487,6 +1495,11 @@ ferrox_status ferrox_init_geometry(ferrox_ctx** out, const ferrox_geometry* geom
   }
   FX_INIT_CK(cudaMemcpy(ctx->planes_d, ctx->planes.data(), ctx->nz * sizeof(PlaneTDGL),
                         cudaMemcpyHostToDevice));
+  {
+    const std::vector<PlaneForce> pf = plane_forces(ctx->planes, ctx->h, ctx->num.dt);
+    FX_INIT_CK(cudaMalloc(&ctx->force_d, pf.size() * sizeof(PlaneForce)));
+    FX_INIT_CK(cudaMemcpy(ctx->force_d, pf.data(), pf.size() * sizeof(PlaneForce), cudaMemcpyHostToDevice));
+  }
   if (ctx->num.tdgl_arith == FERROX_TDGL_FP32) {
     const std::vector<PlaneF32> pf = planes_f32(ctx->planes, ctx->h / kEps0);
     FX_INIT_CK(cudaMalloc(&ctx->planes_f32_d, pf.size() * sizeof(PlaneF32)));
@@ -1873,6 +1886,7 @@ struct ferrox_batch {
   void* dense = nullptr;              // T: inverses of the instances' dense tail levels
   PlaneCoef<double>* coef0 = nullptr;
   PlaneTDGL* planes = nullptr;
+  PlaneForce* force = nullptr;
   LevelDesc* lv = nullptr;
   LevelDesc* lvt = nullptr;
   int* pre = nullptr;
@@ -2237,7 +2251,7 @@ void batch_release(ferrox_batch* B) {
   if (B->ge_solve) cudaGraphExecDestroy(B->ge_solve);
   if (B->gr_step) cudaGraphDestroy(B->gr_step);
   if (B->gr_solve) cudaGraphDestroy(B->gr_solve);
-  void* ptrs[] = {B->b, B->Pbuf, B->backup, B->e, B->r, B->s, B->eb, B->sinv, B->leg_pre, B->coef, B->dense, B->coef0, B->planes, B->lv,
+  void* ptrs[] = {B->b, B->Pbuf, B->backup, B->e, B->r, B->s, B->eb, B->sinv, B->leg_pre, B->coef, B->dense, B->coef0, B->planes, B->force, B->lv,
                   B->lvt, B->pre, B->partials, B->active, B->bar, B->grp_d, B->status, B->ticket, B->tile_pre, B->rt_pre, B->any_d, B->nsteps_d, B->dbg, B->params,
                   B->stats, B->inst, B->charge_part, B->charge_out};
   for (void* p : ptrs) if (p) cudaFree(p);
@@ -2351,6 +2365,7 @@ ferrox_status ferrox_init_batch(ferrox_batch** out, int n, const ferrox_geometry
   FX_BINIT(cudaMalloc(&B->coef, (size_t)ncoef * (B->mixed ? sizeof(PlaneCoef<float>) : sizeof(PlaneCoef<double>))));
   FX_BINIT(cudaMalloc(&B->coef0, (size_t)nplanes * sizeof(PlaneCoef<double>)));
   FX_BINIT(cudaMalloc(&B->planes, (size_t)nplanes * sizeof(PlaneTDGL)));
+  FX_BINIT(cudaMalloc(&B->force, (size_t)nplanes * sizeof(PlaneForce)));
   FX_BINIT(cudaMalloc(&B->lv, (size_t)nlv * sizeof(LevelDesc)));
   FX_BINIT(cudaMalloc(&B->lvt, (size_t)nlvt * sizeof(LevelDesc)));
   FX_BINIT(cudaMalloc(&B->pre, (size_t)(1 + 2 * B->Ldown) * (n + 1) * sizeof(int)));
@@ -2436,6 +2451,7 @@ ferrox_status ferrox_init_batch(ferrox_batch** out, int n, const ferrox_geometry
   std::vector<unsigned char> coefT, denseT;
   std::vector<PlaneCoef<double>> coef0;
   std::vector<PlaneTDGL> planes;
+  std::vector<PlaneForce> force;
   std::vector<LevelDesc> lv, lvt;
   std::vector<BatchInst> inst(n);
   for (int i = 0; i < n; ++i) {
@@ -2465,6 +2481,8 @@ ferrox_status ferrox_init_batch(ferrox_batch** out, int n, const ferrox_geometry
       }
     }
     planes.insert(planes.end(), c.planes.begin(), c.planes.end());
+    const std::vector<PlaneForce> pf = plane_forces(c.planes, c.h, num->dt);
+    force.insert(force.end(), pf.begin(), pf.end());
     for (auto L : c.lv) { L.off += p.arena_off; L.coef_off += p.coef_off; lv.push_back(L); }
     for (auto L : c.lv_tail) { L.coef_off += p.coef_off; lvt.push_back(L); }
     BatchInst& I = inst[i];
@@ -2480,7 +2498,7 @@ ferrox_status ferrox_init_batch(ferrox_batch** out, int n, const ferrox_geometry
     I.tail_base = c.lv[c.tail_first].off + p.arena_off;
     TDGLArgs& t = I.tdgl;
     t.P_in = I.P; t.P_out = I.Pbuf; t.P_base = nullptr; t.F_store = nullptr;
-    t.phi = I.phi; t.b = B->b + p.cell_off; t.planes = B->planes + p.plane_off; t.params = B->params + i;
+    t.phi = I.phi; t.b = B->b + p.cell_off; t.planes = B->planes + p.plane_off; t.force = B->force + p.plane_off; t.params = B->params + i;
     t.nx = c.nx; t.ny = c.ny; t.nz = c.nz; t.ncomp = 1; t.kd_lo = c.kd_lo; t.kd_hi = c.kd_hi;
     t.dt = num->dt; t.inv_h = 1.0 / c.h; t.inv_h2 = 1.0 / (c.h * c.h); t.b_scale = c.h / kEps0; t.mode = 0;
     ResidArgs& ra = I.resid;
@@ -2507,6 +2525,7 @@ ferrox_status ferrox_init_batch(ferrox_batch** out, int n, const ferrox_geometry
   }
   FX_BINIT(cudaMemcpy(B->coef0, coef0.data(), coef0.size() * sizeof(PlaneCoef<double>), cudaMemcpyHostToDevice));
   FX_BINIT(cudaMemcpy(B->planes, planes.data(), planes.size() * sizeof(PlaneTDGL), cudaMemcpyHostToDevice));
+  FX_BINIT(cudaMemcpy(B->force, force.data(), force.size() * sizeof(PlaneForce), cudaMemcpyHostToDevice));
   FX_BINIT(cudaMemcpy(B->lv, lv.data(), lv.size() * sizeof(LevelDesc), cudaMemcpyHostToDevice));
   FX_BINIT(cudaMemcpy(B->lvt, lvt.data(), lvt.size() * sizeof(LevelDesc), cudaMemcpyHostToDevice));
   FX_BINIT(cudaMemcpy(B->inst, inst.data(), n * sizeof(BatchInst), cudaMemcpyHostToDevice));
@@ -2793,71 +2812,75 @@ constexpr int kStaticMaxPlanes = FERROX_STATIC_MAX_PLANES;
 constexpr size_t kStaticPlaneBytes = ((size_t)kStaticMaxPlanes * sizeof(PlaneTDGL) + 255) / 256 * 256;
 constexpr size_t kStaticParamBytes = 256;
 constexpr size_t kStaticStateBytes = (size_t)kStaticMaxCells * 4 * sizeof(double);  // 3 comps + b
-constexpr size_t kStaticBytes = kStaticParamBytes + kStaticPlaneBytes + kStaticStateBytes;
+constexpr size_t kStaticForceBytes = ((size_t)kStaticMaxPlanes * sizeof(PlaneForce) + 255) / 256 * 256;
+constexpr size_t kStaticBytes = kStaticParamBytes + kStaticPlaneBytes + kStaticForceBytes + kStaticStateBytes;
 
 static __device__ __align__(256) unsigned char g_static_scratch[kStaticBytes];
 
 std::mutex g_static_mu;
 unsigned char* g_static_ptr[64] = {};   // device address of g_static_scratch, per device
 
-// Plane table of the static path, written into a caller-side array without any
-// heap use; the same per-plane quantities as the context path.
-ferrox_status static_planes(const ferrox_geometry* g, PlaneTDGL* out, int* nz_out, int* fe_lo,
-                            int* fe_hi) {
-  int nz = 0;
-  for (int q = 0; q < g->nlayers; ++q) nz += g->layers[q].ncells;
-  if (nz > kStaticMaxPlanes) return FERROX_EINVAL;
-  const double h = g->h;
-  double kappa;
-  if (g->pbc == FERROX_PBC_FREE) kappa = 1.0 / 8.0;
-  else if (g->pbc == FERROX_PBC_ZERO) kappa = 0.0;
-  else kappa = g->lambda / (3.0 * h + 8.0 * g->lambda);
-  int z = 0;
-  *fe_lo = nz;
-  *fe_hi = -1;
-  for (int q = 0; q < g->nlayers; ++q) {
-    const ferrox_layer& L = g->layers[q];
-    for (int c = 0; c < L.ncells; ++c, ++z) {
-      PlaneTDGL p{};
-      p.eps_r = L.eps_r;
-      p.fe = L.kind == FERROX_FE;
-      if (p.fe) {
-        p.alpha = L.alpha; p.beta = L.beta; p.gamma = L.gamma;
-        p.alpha_xy = L.alpha_xy; p.beta_xy = L.beta_xy; p.gamma_xy = L.gamma_xy;
-        p.g11 = L.g11; p.g44 = L.g44; p.Gamma = L.Gamma;
-        *fe_lo = std::min(*fe_lo, z);
-        *fe_hi = std::max(*fe_hi, z);
-      }
-      out[z] = p;
+// What the static path's tables are made of.  Stacks of up to kStaticLayers layers pass it
+// to a kernel that writes the tables; with more layers the host writes them and copies.
+constexpr int kStaticLayers = 16;
+struct StaticStack {
+  int nlayers, nz;
+  double h, kappa, dt, v_bot, v_top;
+  ferrox_layer layer[kStaticLayers];
+};
+
+double static_kappa(const ferrox_geometry* g) {
+  if (g->pbc == FERROX_PBC_FREE) return 1.0 / 8.0;
+  if (g->pbc == FERROX_PBC_ZERO) return 0.0;
+  return g->lambda / (3.0 * g->h + 8.0 * g->lambda);
+}
+
+// the TDGL entries of plane z, which layer q holds, from the layers of its neighbours (dn,
+// up; null beyond the stack); the same per-plane quantities as the context path
+__host__ __device__ inline PlaneTDGL static_plane(const ferrox_layer& L, const ferrox_layer* dn, const ferrox_layer* up,
+                                                  double h, double kappa) {
+  PlaneTDGL p{};
+  const bool fe_dn = dn && dn->kind == FERROX_FE, fe_up = up && up->kind == FERROX_FE;
+  p.eps_r = L.eps_r;
+  p.fe = L.kind == FERROX_FE;
+  p.b_dyn = p.fe || fe_dn || fe_up;
+  if (p.fe) {
+    p.alpha = L.alpha; p.beta = L.beta; p.gamma = L.gamma;
+    p.alpha_xy = L.alpha_xy; p.beta_xy = L.beta_xy; p.gamma_xy = L.gamma_xy;
+    p.g11 = L.g11; p.g44 = L.g44; p.Gamma = L.Gamma;
+    const double ih2 = 1.0 / (h * h);
+    if (fe_dn && fe_up) {
+      p.wz_dn = ih2; p.wz_c = -2.0 * ih2; p.wz_up = ih2;
+    } else {
+      const double wn = 4.0 * (1.0 - 2.0 * kappa) / 3.0 * ih2;
+      p.wz_c = 4.0 * (18.0 * kappa - 3.0) / 3.0 * ih2;
+      p.wz_up = fe_up ? wn : 0.0;
+      p.wz_dn = fe_dn ? wn : 0.0;
     }
   }
-  for (z = 0; z < nz; ++z) {
-    PlaneTDGL& p = out[z];
-    const bool dn = z > 0 && out[z - 1].fe, up = z < nz - 1 && out[z + 1].fe;
-    p.b_dyn = p.fe || dn || up;
-    if (p.fe) {
-      const double ih2 = 1.0 / (h * h);
-      if (dn && up) {
-        p.wz_dn = ih2; p.wz_c = -2.0 * ih2; p.wz_up = ih2;
-      } else if (up || dn) {
-        const double wn = 4.0 * (1.0 - 2.0 * kappa) / 3.0 * ih2;
-        p.wz_c = 4.0 * (18.0 * kappa - 3.0) / 3.0 * ih2;
-        p.wz_up = up ? wn : 0.0;
-        p.wz_dn = dn ? wn : 0.0;
-      } else {
-        return FERROX_EINVAL;
-      }
-    }
-    if (z > 0) {
-      const double eL = out[z - 1].eps_r, eR = p.eps_r;
-      p.fw_L = eL / (eL + eR);
-      p.fw_R = eR / (eL + eR);
-      p.fpc = h / (2.0 * kEps0 * (eL + eR));
-    }
-    p.lift = (z == 0 || z == nz - 1) ? 2.0 * p.eps_r : 0.0;
+  if (dn) {
+    const double eL = dn->eps_r, eR = p.eps_r;
+    p.fw_L = eL / (eL + eR);
+    p.fw_R = eR / (eL + eR);
+    p.fpc = h / (2.0 * kEps0 * (eL + eR));
   }
-  *nz_out = nz;
-  return FERROX_OK;
+  p.lift = !dn || !up ? 2.0 * p.eps_r : 0.0;
+  return p;
+}
+
+__global__ void __launch_bounds__(64) static_table_kernel(const __grid_constant__ StaticStack S, DevParams* params,
+                                                          PlaneTDGL* planes, PlaneForce* force) {
+  const int z = blockIdx.x * blockDim.x + threadIdx.x;
+  if (z == 0) *params = DevParams{S.v_bot, S.v_top};
+  if (z >= S.nz) return;
+  int q = 0, first = 0;
+  while (z >= first + S.layer[q].ncells) first += S.layer[q++].ncells;
+  const ferrox_layer& L = S.layer[q];
+  const ferrox_layer* dn = z > first ? &L : q > 0 ? &S.layer[q - 1] : nullptr;
+  const ferrox_layer* up = z + 1 < first + L.ncells ? &L : q + 1 < S.nlayers ? &S.layer[q + 1] : nullptr;
+  const PlaneTDGL p = static_plane(L, dn, up, S.h, S.kappa);
+  planes[z] = p;
+  force[z] = plane_force(p, 1.0 / (S.h * S.h), S.dt);
 }
 
 }  // namespace
@@ -2883,10 +2906,19 @@ extern "C" ferrox_status ferrox_tdgl_update_static(const ferrox_geometry* geom, 
   if (N > kStaticMaxCells || nzl > kStaticMaxPlanes)
     return bad("ferrox_tdgl_update_static: grid larger than its static scratch "
                "(at most FERROX_STATIC_MAX_CELLS cells and FERROX_STATIC_MAX_PLANES planes)");
-  PlaneTDGL planes[kStaticMaxPlanes];
-  int nz = 0, fe_lo = 0, fe_hi = -1;
-  if (static_planes(geom, planes, &nz, &fe_lo, &fe_hi) != FERROX_OK || fe_hi < 0)
-    return bad("the stack needs a ferroelectric layer at least 2 cells thick");
+  // runs of ferroelectric planes (adjacent ferroelectric layers form one)
+  const int nz = (int)nzl, nl = geom->nlayers;
+  int fe_lo = nz, fe_hi = -1;
+  for (int q = 0, z = 0; q < nl; z += geom->layers[q++].ncells) {
+    if (geom->layers[q].kind != FERROX_FE) continue;
+    const bool joined = (q > 0 && geom->layers[q - 1].kind == FERROX_FE) ||
+                        (q + 1 < nl && geom->layers[q + 1].kind == FERROX_FE);
+    if (geom->layers[q].ncells < 2 && !joined)
+      return bad("the stack needs a ferroelectric layer at least 2 cells thick");
+    fe_lo = std::min(fe_lo, z);
+    fe_hi = z + geom->layers[q].ncells - 1;
+  }
+  if (fe_hi < 0) return bad("the stack needs a ferroelectric layer at least 2 cells thick");
   int dev = 0;
   cudaError_t e = cudaGetDevice(&dev);
   if (e != cudaSuccess || dev < 0 || dev >= 64) return fail(nullptr, FERROX_ECUDA, "cudaGetDevice failed");
@@ -2907,15 +2939,37 @@ extern "C" ferrox_status ferrox_tdgl_update_static(const ferrox_geometry* geom, 
   cudaStream_t s = static_cast<cudaStream_t>(cuda_stream);
   DevParams* params = reinterpret_cast<DevParams*>(base);
   PlaneTDGL* planes_d = reinterpret_cast<PlaneTDGL*>(base + kStaticParamBytes);
-  double* Pout = reinterpret_cast<double*>(base + kStaticParamBytes + kStaticPlaneBytes);
+  PlaneForce* force_d = reinterpret_cast<PlaneForce*>(base + kStaticParamBytes + kStaticPlaneBytes);
+  double* Pout = reinterpret_cast<double*>(base + kStaticParamBytes + kStaticPlaneBytes + kStaticForceBytes);
   double* b = Pout + (size_t)geom->ncomp * N;
-  // pageable source: the copy is staged before the call returns
-  e = cudaMemcpyAsync(planes_d, planes, nz * sizeof(PlaneTDGL), cudaMemcpyHostToDevice, s);
-  if (e != cudaSuccess) return fail(nullptr, FERROX_ECUDA, std::string("cudaMemcpyAsync: ") + cudaGetErrorString(e));
-  launch_set_params(params, v_bottom, v_top, s);
+  const double kappa = static_kappa(geom);
+  if (nl <= kStaticLayers) {
+    StaticStack S;
+    S.nlayers = nl; S.nz = nz;
+    S.h = geom->h; S.kappa = kappa; S.dt = dt; S.v_bot = v_bottom; S.v_top = v_top;
+    for (int q = 0; q < nl; ++q) S.layer[q] = geom->layers[q];
+    static_table_kernel<<<(nz + 63) / 64, 64, 0, s>>>(S, params, planes_d, force_d);
+  } else {
+    PlaneTDGL planes[kStaticMaxPlanes];
+    PlaneForce force[kStaticMaxPlanes];
+    for (int q = 0, z = 0; q < nl; ++q) {
+      const ferrox_layer& L = geom->layers[q];
+      for (int c = 0; c < L.ncells; ++c, ++z) {
+        const ferrox_layer* dn = c > 0 ? &L : q > 0 ? &geom->layers[q - 1] : nullptr;
+        const ferrox_layer* up = c + 1 < L.ncells ? &L : q + 1 < nl ? &geom->layers[q + 1] : nullptr;
+        planes[z] = static_plane(L, dn, up, geom->h, kappa);
+        force[z] = plane_force(planes[z], 1.0 / (geom->h * geom->h), dt);
+      }
+    }
+    // pageable sources: the copies are staged before the call returns
+    e = cudaMemcpyAsync(planes_d, planes, nz * sizeof(PlaneTDGL), cudaMemcpyHostToDevice, s);
+    if (e == cudaSuccess) e = cudaMemcpyAsync(force_d, force, nz * sizeof(PlaneForce), cudaMemcpyHostToDevice, s);
+    if (e != cudaSuccess) return fail(nullptr, FERROX_ECUDA, std::string("cudaMemcpyAsync: ") + cudaGetErrorString(e));
+    launch_set_params(params, v_bottom, v_top, s);
+  }
   TDGLArgs a{};
   a.P_in = P_dev; a.P_out = Pout; a.P_base = nullptr; a.F_store = nullptr;
-  a.phi = phi_dev; a.b = b; a.planes = planes_d; a.params = params;
+  a.phi = phi_dev; a.b = b; a.planes = planes_d; a.force = force_d; a.params = params;
   a.nx = geom->nx; a.ny = geom->ny; a.nz = nz; a.ncomp = geom->ncomp;
   a.kd_lo = std::max(0, fe_lo - 1);
   a.kd_hi = std::min(nz - 1, fe_hi + 1);
@@ -2928,18 +2982,21 @@ extern "C" ferrox_status ferrox_tdgl_update_static(const ferrox_geometry* geom, 
   // an earlier call left on the other planes, and the caller's planes between two
   // ferroelectric layers must not receive it.
   const long long plane = (long long)geom->nx * geom->ny;
-  for (int z0 = fe_lo; z0 <= fe_hi;) {
-    if (!planes[z0].fe) { ++z0; continue; }
-    int z1 = z0;
-    while (z1 + 1 <= fe_hi && planes[z1 + 1].fe) ++z1;
-    const size_t off = (size_t)z0 * plane, cnt = (size_t)(z1 - z0 + 1) * plane;
-    for (int q = 0; q < geom->ncomp; ++q) {
-      e = cudaMemcpyAsync(P_dev + q * N + off, Pout + q * N + off, cnt * sizeof(double),
-                          cudaMemcpyDeviceToDevice, s);
-      if (e != cudaSuccess)
-        return fail(nullptr, FERROX_ECUDA, std::string("cudaMemcpyAsync: ") + cudaGetErrorString(e));
+  for (int q = 0, z0 = 0; q < nl;) {
+    int z1 = z0;   // one past the run
+    const bool fe = geom->layers[q].kind == FERROX_FE;
+    do z1 += geom->layers[q++].ncells;
+    while (q < nl && fe && geom->layers[q].kind == FERROX_FE);
+    if (fe) {
+      const size_t off = (size_t)z0 * plane, cnt = (size_t)(z1 - z0) * plane;
+      for (int c = 0; c < geom->ncomp; ++c) {
+        e = cudaMemcpyAsync(P_dev + c * N + off, Pout + c * N + off, cnt * sizeof(double),
+                            cudaMemcpyDeviceToDevice, s);
+        if (e != cudaSuccess)
+          return fail(nullptr, FERROX_ECUDA, std::string("cudaMemcpyAsync: ") + cudaGetErrorString(e));
+      }
     }
-    z0 = z1 + 1;
+    z0 = z1;
   }
   e = cudaGetLastError();
   if (e != cudaSuccess) return fail(nullptr, FERROX_ECUDA, std::string("launch: ") + cudaGetErrorString(e));

@@ -106,6 +106,29 @@ struct PlaneTDGL {
   double kqn0, kqp0, kqN;
 };
 
+// What the FP64 update of P_z reads of a plane, with everything that is constant over a
+// run folded on the host (the update is bound by the FP64 pipe):
+//   dF = P (lin + beta P^2 + gamma P^4) + w_dn P_dn + w_up P_up + glat (sum of the four
+//        lateral neighbours) + (upper - lower face potential) / h,   f = -Gamma dF,
+// lin = alpha + 4 g44/h^2 - g11 wz_c; the face weights are those of the plane's lower face.
+struct PlaneForce {
+  int fe, pad;
+  double lin, beta, gamma, w_dn, w_up, glat;
+  double gam, gdt;                    // -Gamma, -Gamma dt
+  double fw_L, fw_R, fpc;
+};
+__host__ __device__ inline PlaneForce plane_force(const PlaneTDGL& p, double inv_h2, double dt) {
+  PlaneForce f;
+  f.fe = p.fe; f.pad = 0;
+  f.lin = p.alpha + 4.0 * p.g44 * inv_h2 - p.g11 * p.wz_c;
+  f.beta = p.beta; f.gamma = p.gamma;
+  f.w_dn = -p.g11 * p.wz_dn; f.w_up = -p.g11 * p.wz_up;
+  f.glat = -p.g44 * inv_h2;
+  f.gam = -p.Gamma; f.gdt = -p.Gamma * dt;
+  f.fw_L = p.fw_L; f.fw_R = p.fw_R; f.fpc = p.fpc;
+  return f;
+}
+
 // a semiconductor plane's 1/VT, kq n0, kq p0 and kq Nnet as double-float pairs (nearest
 // floats of the value and of the rest), a table of its own: PlaneTDGL's stride is the
 // TDGL kernel's (256 bytes instead of 224 cost it 8%)
@@ -346,6 +369,7 @@ struct TDGLArgs {
   const double* phi;
   double* b;              // scaled RHS, dynamic planes written
   const PlaneTDGL* planes;
+  const PlaneForce* force;
   const DevParams* params;
   int nx, ny, nz, ncomp;
   int kd_lo, kd_hi;       // dynamic plane range

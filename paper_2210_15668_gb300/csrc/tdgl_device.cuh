@@ -14,40 +14,140 @@ __device__ __forceinline__ double landau(double a, double b, double g, double P)
   return P * fma(P2, fma(g, P2, b), a);
 }
 
-// z component of the force at plane k of column (i, j)
-__device__ __forceinline__ double force_z(const TDGLArgs& a, const PlaneTDGL& pt,
-                                          const PlaneTDGL* planes, const double* Pz,
-                                          const double* phi, long long t, int k, int i, int j,
-                                          int im, int ip, int jm, int jp, double v_bot,
-                                          double v_top) {
+// The FP64 update of P_z along a column, plane by plane upwards.  The face potential,
+// polarization and potential that a plane shares with the next one are kept, so each is
+// computed and loaded once: 17 FP64 operations for the force and update of a cell and 4
+// for its right-hand side (38 executed per cell before, with both faces of every cell
+// evaluated on their own).  Every rounding is spelled out: all kernels that march, from
+// whatever plane they start, agree bit for bit.
+struct PzMarch {
+  double P, Pdn, ph, face;   // of the plane updated next: P, P below, potential, lower face potential
+  bool ready = false;        // they are its own (the plane below was ferroelectric)
+};
+
+// potential of the face between planes k - 1 and k (f: plane k's table entry)
+__device__ __forceinline__ double face_potential(const PlaneForce& f, double ph_lo, double ph_hi, double P_lo,
+                                                 double P_hi) {
+  return fma(-f.fpc, __dadd_rn(P_hi, -P_lo), fma(f.fw_L, ph_lo, __dmul_rn(f.fw_R, ph_hi)));
+}
+
+// new P of ferroelectric plane k (cell t) of column (i, j)
+__device__ __forceinline__ double advance_z(const TDGLArgs& a, PzMarch& m, const double* Pz, long long t, long long ti,
+                                            int k, int i, int j, int im, int ip, int jm, int jp, double v_bot,
+                                            double v_top) {
   const long long plane = (long long)a.nx * a.ny;
-  const double P = Pz[t];
-  const double lat = (Pz[t - i + im] + Pz[t - i + ip]) +
-                     (Pz[t + (long long)(jm - j) * a.nx] + Pz[t + (long long)(jp - j) * a.nx]);
-  const bool fe_dn = k > 0 && __ldg(&planes[k - 1].fe);
-  const bool fe_up = k < a.nz - 1 && __ldg(&planes[k + 1].fe);
-  const double Pdn = fe_dn ? Pz[t - plane] : 0.0;
-  const double Pup = fe_up ? Pz[t + plane] : 0.0;
-  const double ph = phi[t];
-  double phif_dn, phif_up;
-  if (k == 0) {
-    phif_dn = v_bot;
-  } else {
-    phif_dn = fma(pt.fw_L, phi[t - plane], pt.fw_R * ph) - pt.fpc * (P - Pdn);
+  const PlaneForce f = ldg_struct(a.force + k);
+  if (!m.ready) {
+    m.P = Pz[t];
+    m.ph = a.phi[t];
+    m.Pdn = k > 0 && __ldg(&a.force[k - 1].fe) ? Pz[t - plane] : 0.0;
+    m.face = k == 0 ? v_bot : face_potential(f, a.phi[t - plane], m.ph, m.Pdn, m.P);
   }
-  if (k == a.nz - 1) {
-    phif_up = v_top;
-  } else {
-    const PlaneTDGL pu = ldg_struct(planes + k + 1);
-    phif_up = fma(pu.fw_L, ph, pu.fw_R * phi[t + plane]) - pu.fpc * (Pup - P);
+  const double lat = __dadd_rn(__dadd_rn(Pz[t - i + im], Pz[t - i + ip]),
+                               __dadd_rn(Pz[t + (long long)(jm - j) * a.nx], Pz[t + (long long)(jp - j) * a.nx]));
+  double Pup = 0.0, ph_up = 0.0, face_up = v_top;
+  bool fe_up = false;
+  if (k < a.nz - 1) {
+    const PlaneForce* u = a.force + k + 1;
+    fe_up = __ldg(&u->fe);
+    if (fe_up) Pup = Pz[t + plane];
+    ph_up = a.phi[t + plane];
+    PlaneForce fu;
+    fu.fw_L = __ldg(&u->fw_L); fu.fw_R = __ldg(&u->fw_R); fu.fpc = __ldg(&u->fpc);
+    face_up = face_potential(fu, m.ph, ph_up, m.P, Pup);
   }
-  const double lap = fma(-4.0, P, lat) * a.inv_h2;
-  const double d2z = fma(pt.wz_dn, Pdn, fma(pt.wz_c, P, pt.wz_up * Pup));
-  double dF = landau(pt.alpha, pt.beta, pt.gamma, P);
-  dF = fma(-pt.g44, lap, dF);
-  dF = fma(-pt.g11, d2z, dF);
-  dF = fma(phif_up - phif_dn, a.inv_h, dF);
-  return -pt.Gamma * dF;
+  const double P2 = __dmul_rn(m.P, m.P);
+  double dF = __dmul_rn(m.P, fma(P2, fma(f.gamma, P2, f.beta), f.lin));
+  dF = fma(f.w_dn, m.Pdn, dF);
+  dF = fma(f.w_up, Pup, dF);
+  dF = fma(f.glat, lat, dF);
+  dF = fma(__dadd_rn(face_up, -m.face), a.inv_h, dF);
+  double pn;
+  if (a.mode == 0) {
+    pn = fma(f.gdt, dF, m.P);
+  } else {
+    const double fz = __dmul_rn(f.gam, dF);
+    if (a.mode == 1) {
+      a.F_store[ti] = fz;
+      pn = fma(a.dt, fz, m.P);
+    } else {
+      pn = fma(0.5 * a.dt, __dadd_rn(a.F_store[ti], fz), a.P_base[ti]);
+    }
+  }
+  m.Pdn = m.P;
+  m.P = Pup;
+  m.ph = ph_up;
+  m.face = face_up;
+  m.ready = fe_up;
+  return pn;
+}
+
+// polarization of the face below plane k from the new P of planes k - 1 and k (the cell's
+// own on electrode faces)
+__device__ __forceinline__ double face_polarization(const TDGLArgs& a, int k, double lo, double hi) {
+  if (k == 0) return hi;
+  if (k == a.nz) return lo;
+  return fma(__ldg(&a.force[k].fw_R), lo, __dmul_rn(__ldg(&a.force[k].fw_L), hi));
+}
+
+// right-hand side of plane k from its two face polarizations
+__device__ __forceinline__ double rhs_faces(const TDGLArgs& a, int k, double pf_dn, double pf_up, double v_bot,
+                                            double v_top) {
+  double b = __dmul_rn(__dadd_rn(pf_dn, -pf_up), a.b_scale);
+  if (k == 0) b = fma(__ldg(&a.planes[0].lift), v_bot, b);
+  if (k == a.nz - 1) b = fma(__ldg(&a.planes[a.nz - 1].lift), v_top, b);
+  return b;
+}
+
+// One of CZ chunks of a column's dynamic planes (one component): the new P of its planes,
+// and their right-hand sides; those of the chunk's first and last planes take the
+// neighbouring chunks' edge values from shared memory (first_s, last_s: [CZ] of this
+// column, STRIDE apart).  Every thread of the block has to call it.
+template <int CZ>
+__device__ __forceinline__ void tdgl_chunk(const TDGLArgs& a, int mode, int i, int j, bool col, int c, double* first_s,
+                                           double* last_s, int stride) {
+  const int per = (a.kd_hi - a.kd_lo + 1 + CZ - 1) / CZ;
+  const int k0 = a.kd_lo + c * per, k1 = min(a.kd_hi, k0 + per - 1);   // empty when k0 > k1
+  const long long plane = (long long)a.nx * a.ny, cix = (long long)j * a.nx + i;
+  const double v_bot = a.params->v_bot, v_top = a.params->v_top;
+  double p_first = 0.0, pm1 = 0.0, pf_second = 0.0, pf = 0.0;
+  if (col && k0 <= k1) {
+    const int im = (i == 0) ? a.nx - 1 : i - 1, ip = (i == a.nx - 1) ? 0 : i + 1;
+    const int jm = (j == 0) ? a.ny - 1 : j - 1, jp = (j == a.ny - 1) ? 0 : j + 1;
+    PzMarch m;
+    for (int k = k0; k <= k1; ++k) {
+      const long long t = k * plane + cix;
+      double pn = 0.0;
+      if (__ldg(&a.force[k].fe)) {
+        if (mode == 3) {
+          pn = a.P_in[t];
+        } else {
+          pn = advance_z(a, m, a.P_in, t, t, k, i, j, im, ip, jm, jp, v_bot, v_top);
+          a.P_out[t] = pn;
+        }
+      } else {
+        m.ready = false;
+      }
+      if (k == k0) {
+        p_first = pn;
+      } else {
+        const double up = face_polarization(a, k, pm1, pn);
+        if (k == k0 + 1) pf_second = up;
+        else a.b[(k - 1) * plane + cix] = rhs_faces(a, k - 1, pf, up, v_bot, v_top);
+        pf = up;
+      }
+      pm1 = pn;
+    }
+    first_s[c * stride] = p_first;
+    last_s[c * stride] = pm1;
+  }
+  __syncthreads();
+  if (!col || k0 > k1) return;
+  const double below = k0 - 1 >= a.kd_lo ? last_s[(c - 1) * stride] : 0.0;
+  const double above = k1 + 1 <= a.kd_hi ? first_s[(c + 1) * stride] : 0.0;
+  const double pf_lo = face_polarization(a, k0, below, p_first), pf_hi = face_polarization(a, k1 + 1, pm1, above);
+  a.b[k0 * plane + cix] = rhs_faces(a, k0, pf_lo, k1 == k0 ? pf_hi : pf_second, v_bot, v_top);
+  if (k1 > k0) a.b[k1 * plane + cix] = rhs_faces(a, k1, pf, pf_hi, v_bot, v_top);
 }
 
 // in-plane component (3-component model): own Landau polynomial and dPhi/dx
@@ -113,17 +213,17 @@ __device__ __forceinline__ void tdgl_column(const TDGLArgs& a, int i, int j) {
   const double v_bot = a.params->v_bot, v_top = a.params->v_top;
   const PlaneTDGL* planes = a.planes;
   const double* Pz_in = a.P_in + (long long)(a.ncomp - 1) * N;
-  // ring of new P_z values at planes k-1, k (b of plane k-1 is emitted once P(k) is known)
-  double pn_m2 = 0.0, pn_m1 = 0.0;
+  PzMarch m;
+  double pm1 = 0.0, pf = 0.0;   // new P of the plane below, polarization of its lower face
   for (int k = a.kd_lo; k <= a.kd_hi + 1; ++k) {
     double pn = 0.0;
-    if (k <= a.kd_hi) {
-      const PlaneTDGL pt = ldg_struct(planes + k);
-      if (pt.fe && a.mode == 3) {
-        pn = Pz_in[k * plane + col];          // right-hand side of the current P only
-      } else if (pt.fe) {
-        const long long t = k * plane + col;
+    if (k <= a.kd_hi && __ldg(&a.force[k].fe)) {
+      const long long t = k * plane + col;
+      if (a.mode == 3) {
+        pn = Pz_in[t];                        // right-hand side of the current P only
+      } else {
         if (a.ncomp == 3) {
+          const PlaneTDGL pt = ldg_struct(planes + k);
           const double inv_eps_abs = 1.0 / (8.8541878128e-12 * pt.eps_r);
           for (int c = 0; c < 2; ++c) {
             const double* Pc = a.P_in + (long long)c * N;
@@ -132,17 +232,19 @@ __device__ __forceinline__ void tdgl_column(const TDGLArgs& a, int i, int j) {
             a.P_out[c * N + t] = advance(a, c * N + t, f);
           }
         }
-        const double f = force_z(a, pt, planes, Pz_in, a.phi, t, k, i, j, im, ip, jm, jp, v_bot, v_top);
         const long long zi = (long long)(a.ncomp - 1) * N + t;
-        pn = advance(a, zi, f);
+        pn = advance_z(a, m, Pz_in, t, zi, k, i, j, im, ip, jm, jp, v_bot, v_top);
         a.P_out[zi] = pn;
       }
+    } else {
+      m.ready = false;
     }
-    if (a.ncomp == 1 && k - 1 >= a.kd_lo) {
-      a.b[(k - 1) * plane + col] = rhs_value(a, planes, k - 1, pn_m2, pn_m1, pn, v_bot, v_top);
+    if (a.ncomp == 1) {   // b of plane k - 1 once P(k) is known
+      const double up = face_polarization(a, k, pm1, pn);
+      if (k > a.kd_lo) a.b[(k - 1) * plane + col] = rhs_faces(a, k - 1, pf, up, v_bot, v_top);
+      pf = up;
     }
-    pn_m2 = pn_m1;
-    pn_m1 = pn;
+    pm1 = pn;
   }
 }
 
