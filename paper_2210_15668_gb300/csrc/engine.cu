@@ -80,6 +80,8 @@ struct ferrox_ctx {
   double* phi_prev = nullptr;         // previous step's potential (guess = 1)
   void* e_arena = nullptr;
   float* eb_arena = nullptr;          // black corrections between the legs of a V-cycle
+  MidPlan mid;                        // FP64: middle levels and tail in one cluster launch (mid.first > 0)
+  LevelDesc* lvm_d = nullptr;         // ... its tail's levels
   bool legs = false;                  // FP32 levels run one launch per leg (leg_device.cuh)
   void* e_alt = nullptr;              // second error array of the fused sweeps (largest such level)
   void* r_arena = nullptr;
@@ -208,6 +210,69 @@ void plan_tail(ferrox_ctx* c, size_t elem_size, bool wide = false) {
     // one cell: a single update is the exact solve (more sweeps repeat it)
     c->num.bottom_sweeps = B.ncell == 1 ? 1 : std::min(64, 2 * (B.nx + B.ny + B.nz));
   }
+}
+
+// The levels of an FP64 V-cycle that run with the tail in one cluster launch (mid.cu):
+// from the first level of at most kMidCells cells down to the tail (with a shift, where
+// the tail's first level is relaxed and not solved by its inverse, to a smaller one: one
+// SM's FP64 rate bounds the tail).  Fills everything but the device pointers; first = 0
+// where the levels do not fit the kernel.
+void plan_mid(const ferrox_ctx* c, MidPlan& m, std::vector<LevelDesc>& tail) {
+  m.first = 0;
+  if (c->num.nu1 < 1 || c->num.nu2 < 1) return;
+  auto fits = [&](int l) { return leg_level(c->lv[l]) && c->lv[l].nx > 1 && c->lv[l].ny > 1; };
+  int first = 1, end = c->tail_first;
+  while (first < end && c->lv[first].ncell > kMidCells) ++first;
+  if (c->shift)
+    while (end + 1 < (int)c->lv.size() && end - first < kMidMax && fits(end)) ++end;
+  for (int l = first; l < end; ++l)
+    if (!fits(l)) return;
+  if (end <= first || end - first > kMidMax || c->tail_first <= first) return;
+  MidArgs& a = m.args;
+  a = MidArgs{};
+  const int narr = c->shift ? 3 : 2;
+  a.n = end - first;
+  a.nu1 = c->num.nu1;
+  a.nu2 = c->num.nu2;
+  int off = 16, per0 = 0;   // two zeros first
+  for (int q = 0; q < a.n; ++q) {
+    MidLevel& L = a.lv[q];
+    L.d = c->lv[first + q];
+    L.seq = first + q >= c->tail_first;
+    const long long pairs = L.d.ncell / 2;
+    L.sh = 0;
+    // two neighbouring pairs lie in one CTA
+    do ++L.sh;
+    while ((long long)kMidCtas << L.sh < pairs);
+    auto magic = [](int d) { return d == 1 ? 0u : 0xFFFFFFFFu / (unsigned)d + 1u; };
+    L.mx = magic(L.d.nx / 2);
+    L.my = magic(L.d.ny);
+    a.planes += L.d.nz;
+    const int bytes = 16 << L.sh;
+    L.e_off = off;
+    L.r_off = off + bytes;
+    L.s_off = off + 2 * bytes;
+    off += narr * bytes;
+    per0 = std::max(per0, 1 << L.sh);
+  }
+  a.coef_off = off;
+  off += a.planes * (int)sizeof(PlaneCoef<double>);
+  a.q_off = (off + 15) / 16 * 16;
+  off = a.q_off + 8 * per0;
+  a.tail_off = (off + 15) / 16 * 16;
+  a.coarse = c->lv[end];
+  const long long base = a.coarse.off;
+  tail.assign(c->lv.begin() + end, c->lv.end());
+  for (auto& t : tail) t.off -= base;
+  a.tail.nlev = (int)tail.size();
+  a.tail.elems = c->arena - base;
+  a.tail.base = base;
+  a.tail.nu1 = a.nu1; a.tail.nu2 = a.nu2; a.tail.bottom_sweeps = c->num.bottom_sweeps;
+  a.tail.constant = 0;
+  m.smem = a.tail_off + (int)(a.tail.elems * (long long)sizeof(double) * narr);
+  m.threads = std::max(256, per0);
+  if (per0 > kMidThreadsMax || m.smem > kMidMaxSmem) return;
+  m.first = first;
 }
 
 // The first tail level of at most kDenseMax cells (and more than one) is solved
@@ -523,6 +588,9 @@ bool rb_sweeps(const ferrox_ctx* c, int l, int nu) {
 // Levels whose smoothing and transfers run as one launch per V-cycle leg
 bool leg_at(const ferrox_ctx* c, int l) { return c->legs && l < c->tail_first && leg_level(c->lv[l]); }
 
+// the first level that the V-cycle's bottom launch takes
+int mid_or_tail(const ferrox_ctx* c) { return c->mid.first > 0 ? c->mid.first : c->tail_first; }
+
 // kernels of one smoothing of level l with nu sweeps
 int smoothing_launches(const ferrox_ctx* c, int l, int nu) {
   const bool rb = c->num.precision == FERROX_MIXED ? rb_sweeps<float>(c, l, nu)
@@ -553,7 +621,7 @@ void enqueue_levels(ferrox_ctx* c, cudaStream_t s, W wrap, int l0, bool first, b
   auto sw_args = [&](int l) -> const MGArgs<T>& { return l == 0 ? a0 : a; };
   const int nu1 = c->num.nu1, nu2 = c->num.nu2;
   const int constant = 0;
-  const int lt = c->tail_first, L = (int)c->lv.size() - 1;
+  const int lt = mid_or_tail(c), L = (int)c->lv.size() - 1;
   T* alt = static_cast<T*>(c->e_alt);
   const UpdateArgs upd{c->phi, c->stats_d, update_clamp(c)};
   // the fine level's e is wanted whole where phi is not updated by its last sweep
@@ -606,7 +674,12 @@ void enqueue_levels(ferrox_ctx* c, cudaStream_t s, W wrap, int l0, bool first, b
     wrap(FERROX_K_RESTRICT, restrict_bytes<T>(c->lv[l], c->lv[l + 1]),
          [&] { launch_restrict<T>(a, c->lv[l], c->lv[l + 1], nu1, s); });
   }
-  if (c->dense_wide_d) {
+  if (lt < c->tail_first) {
+    // the arrays of the levels above the tail in and out, and the tail's
+    double mb = 0.0;
+    for (int l = lt; l <= L; ++l) mb += 2.0 * (double)c->lv[l].ncell * sizeof(T);
+    if constexpr (sizeof(T) == sizeof(double)) wrap(FERROX_K_TAIL, mb, [&] { launch_mid(a, c->mid, s); });
+  } else if (c->dense_wide_d) {
     // the whole tail as one exact solve of its first level, spread over the SMs
     const LevelDesc& B = c->lv[lt];
     // the inverse (n^2 elements) and the level's r in, e out
@@ -759,7 +832,7 @@ bool separate_update(const ferrox_ctx* c) {
 // kernels launched by one outer iteration: V-cycle, (update), residual
 int vcycle_launches(const ferrox_ctx* c) {
   int n = 1;   // the tail or the dense bottom solve
-  for (int l = 0; l < c->tail_first; ++l)
+  for (int l = 0; l < mid_or_tail(c); ++l)
     n += leg_at(c, l) ? 2 : smoothing_launches(c, l, c->num.nu1) + 1 + 1 + smoothing_launches(c, l, c->num.nu2);
   return n;
 }
@@ -1256,7 +1329,7 @@ void release(ferrox_ctx* c) {
   for (auto g : ge) if (g) cudaGraphExecDestroy(g);
   for (auto g : gr) if (g) cudaGraphDestroy(g);
   void* ptrs[] = {c->b, c->Pbuf, c->Fbuf, c->phi_prev, c->e_arena, c->eb_arena, c->e_alt, c->r_arena, c->s_arena, c->coef, c->coef0, c->coef0s, c->bs, c->sinv0, c->coef_df, c->carriers_df,
-                  c->planes_d, c->force_d, c->planes_f32_d, c->lv_d, c->lvt_d, c->nn_scale, c->phi_guess, c->nn_pf, c->nn_stats, c->params_d, c->stats_d, c->partials_d, c->charge_d,
+                  c->planes_d, c->force_d, c->planes_f32_d, c->lv_d, c->lvt_d, c->lvm_d, c->nn_scale, c->phi_guess, c->nn_pf, c->nn_stats, c->params_d, c->stats_d, c->partials_d, c->charge_d,
                   c->charge_part_d, c->dense_d, c->dense_wide_d};
   for (void* p : ptrs) if (p) cudaFree(p);
   if (c->host_pinned) cudaFreeHost(c->host_pinned);
@@ -1495,6 +1568,20 @@ ferrox_status ferrox_init_geometry(ferrox_ctx** out, const ferrox_geometry* geom
   }
   FX_INIT_CK(cudaMemcpy(ctx->planes_d, ctx->planes.data(), ctx->nz * sizeof(PlaneTDGL),
                         cudaMemcpyHostToDevice));
+  if (!mixed && !(rb_env && rb_env[0] == '0')) {
+    std::vector<LevelDesc> tail;
+    plan_mid(ctx, ctx->mid, tail);
+    if (ctx->mid.first > 0 && !mid_prepare(ctx->mid, ctx->shift)) ctx->mid.first = 0;
+    if (ctx->mid.first > 0) {
+      FX_INIT_CK(cudaMalloc(&ctx->lvm_d, tail.size() * sizeof(LevelDesc)));
+      FX_INIT_CK(cudaMemcpy(ctx->lvm_d, tail.data(), tail.size() * sizeof(LevelDesc), cudaMemcpyHostToDevice));
+      MidArgs& a = ctx->mid.args;
+      a.dense = static_cast<const double*>(ctx->dense_wide_d);
+      a.tail.lv = ctx->lvm_d;
+      a.tail.dense = ctx->dense_d;
+      a.tail.dense_lev = ctx->dense_lev;
+    }
+  }
   {
     const std::vector<PlaneForce> pf = plane_forces(ctx->planes, ctx->h, ctx->num.dt);
     FX_INIT_CK(cudaMalloc(&ctx->force_d, pf.size() * sizeof(PlaneForce)));

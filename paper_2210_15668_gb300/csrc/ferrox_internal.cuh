@@ -255,6 +255,36 @@ struct TailArgs {
   int pad;
 };
 
+// The middle levels of an FP64 V-cycle and the tail in one launch of one cluster (mid.cu)
+constexpr int kMidCtas = 16;             // CTAs of the cluster
+constexpr int kMidThreadsMax = 512;      // pairs of a level a CTA may hold, one per thread
+constexpr long long kMidCells = 16384;   // the first middle level's cells at most
+constexpr int kMidMax = 6;               // levels at most
+constexpr int kMidMaxSmem = 200 * 1024;
+struct MidLevel {
+  LevelDesc d;
+  int sh;                                // log2 of the pairs per CTA
+  unsigned mx, my;                       // ceil(2^32 / d) of nx / 2 and ny (0: 1)
+  int seq;                               // restricted in the tail's order of the children
+  int e_off, r_off, s_off;               // the CTA's corrections, right-hand sides and shifts in shared memory
+};
+struct MidArgs {
+  MidLevel lv[kMidMax];
+  LevelDesc coarse;                      // the tail's first level
+  int n, nu1, nu2;
+  int coef_off, planes;                  // shared memory: the levels' plane coefficients, and their count
+  int q_off, tail_off;                   // ... red residuals, tail arrays
+  const double* dense;                   // the first tail level's inverse (null: the tail's V-cycle)
+  TailArgs tail;
+};
+struct MidPlan {
+  MidArgs args;
+  int first = 0;                         // the first middle level (0: none)
+  int threads = 0;
+  int smem = 0;
+};
+bool mid_prepare(const MidPlan& p, bool sc);   // false where the cluster cannot be launched
+
 // Direct FP64 form (V-cycle on phi itself): the fused fine-level residual +
 // restriction + norm that takes the convergence decision
 struct CheckArgs {
@@ -321,6 +351,7 @@ struct LegPlan {
 LegPlan leg_plan(long long cells, int nx, int ny, int nz, bool wide);
 cudaError_t leg_prepare();
 void launch_leg_down(const LegArgs& a, cudaStream_t s);
+void launch_mid(const MGArgs<double>& g, const MidPlan& p, cudaStream_t s);
 void launch_leg_up(const LegArgs& a, const UpdateArgs* upd, cudaStream_t s);
 dim3 check_grid(const LevelDesc& C);
 void launch_restrict_check(const MGArgs<double>& fa, double* rc, const LevelDesc& F,
