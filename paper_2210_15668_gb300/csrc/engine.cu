@@ -705,7 +705,7 @@ void enqueue_levels(ferrox_ctx* c, cudaStream_t s, W wrap, int l0, bool first, b
     // the tiled form where FP64 arithmetic bounds the launch: the fine level
     const bool tiled = sizeof(T) == sizeof(double) && l == 0;
     wrap(FERROX_K_PROLONG, prolong_bytes<T>(c->lv[l], c->lv[l + 1]),
-         [&] { launch_prolong<T>(a, c->lv[l], c->lv[l + 1], constant, s, tiled); });
+         [&] { launch_prolong<T>(a, c->lv[l], c->lv[l + 1], constant, s, tiled, nullptr, nu2); });
     const double sb = sweep_bytes<T>(c, c->lv[l]);
     const bool rb = rb_sweeps<T>(c, l, nu2);
     T* own = a.e + c->lv[l].off;
@@ -790,7 +790,7 @@ void enqueue_check(ferrox_ctx* c, cudaStream_t s, W wrap, int first, int set_con
   double* rc = static_cast<double*>(c->r_arena);
   // phi and b of the fine level read, the coarse residual written
   const double rb = (double)c->lv[0].ncell * 16.0 + (double)c->lv[1].ncell * 8.0;
-  wrap(FERROX_K_RESID, rb, [&] { launch_restrict_check(fa, rc, c->lv[0], c->lv[1], c->num.nu1, ck, s); });
+  wrap(FERROX_K_RESID, rb, [&] { launch_restrict_check(fa, rc, c->lv[0], c->lv[1], ck, s); });
 }
 
 // prologue of a solve: pre-smoothing and the first check
@@ -811,7 +811,7 @@ void enqueue_direct_cycle(ferrox_ctx* c, cudaStream_t s, W wrap, int set_cond,
   enqueue_levels<double>(c, s, wrap, 1, true, false);
   MGArgs<double> a = mg_args<double>(c);
   wrap(FERROX_K_PROLONG, prolong_bytes<double>(c->lv[0], c->lv[1]),
-       [&] { launch_prolong<double>(a, c->lv[0], c->lv[1], 0, s, true, c->phi); });
+       [&] { launch_prolong<double>(a, c->lv[0], c->lv[1], 0, s, true, c->phi, c->num.nu2 + c->num.nu1); });
   enqueue_fine_sweeps(c, s, wrap, c->num.nu2, c->stats_d);
   enqueue_fine_sweeps(c, s, wrap, c->num.nu1, c->stats_d);
   enqueue_check(c, s, wrap, 0, set_cond, handle);

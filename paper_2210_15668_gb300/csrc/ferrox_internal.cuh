@@ -355,13 +355,14 @@ void launch_mid(const MGArgs<double>& g, const MidPlan& p, cudaStream_t s);
 void launch_leg_up(const LegArgs& a, const UpdateArgs* upd, cudaStream_t s);
 dim3 check_grid(const LevelDesc& C);
 void launch_restrict_check(const MGArgs<double>& fa, double* rc, const LevelDesc& F,
-                           const LevelDesc& C, int nu1, const CheckArgs& ck, cudaStream_t s);
+                           const LevelDesc& C, const CheckArgs& ck, cudaStream_t s);
 template <typename T>
 void launch_restrict(const MGArgs<T>& a, const LevelDesc& F, const LevelDesc& C, int nu1,
                      cudaStream_t s);
+// sweeps: red-black sweeps of F that follow (none: the red cells are wanted too)
 template <typename T>
 void launch_prolong(const MGArgs<T>& a, const LevelDesc& F, const LevelDesc& C, int constant,
-                    cudaStream_t s, bool tiled = false, T* fine = nullptr);
+                    cudaStream_t s, bool tiled = false, T* fine = nullptr, int sweeps = 0);
 template <typename T>
 size_t tail_smem_bytes(long long elems, bool has_s);
 template <typename T>

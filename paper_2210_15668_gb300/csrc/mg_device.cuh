@@ -122,21 +122,12 @@ __host__ __device__ __forceinline__ int black_residual_zero(const LevelDesc& F, 
   return nu1 > 0 && (F.nx == 1 || !(F.nx & 1)) && (F.ny == 1 || !(F.ny & 1));
 }
 
-// Residual of the children of coarse cell (I, J, K) on level F (arrays of `fa`),
-// their mean written to the coarse right-hand side rc (and the mean Newton shift
-// to sc).  NORM also accumulates the squared residuals of the children it
-// computes into rr and, with want_b, the squared right-hand sides of all
-// children into bb (the direct FP64 form's stopping test).
-//
-// With a float accumulator (the direct FP64 form's check) the squares are summed
-// in FP32 from FP32 approximations taken with integer operations (the FP64 ->
-// FP32 conversion instruction runs on the FP64 pipe): the norms only scale the
-// stopping test, where a relative error of ~1e-6 in ||r|| is immaterial.
-template <typename T, bool NORM = false, typename A = double>
-__device__ __forceinline__ void restrict_children(const MGArgs<T>& fa, T* rc, T* sc,
-                                                  const LevelDesc& F, const LevelDesc& C, int I,
-                                                  int J, int K, int skip_black, A& rr,
-                                                  A& bb, int want_b) {
+// Residual of the children of coarse cell (I, J, K) on level F, their mean written to the
+// coarse right-hand side (and the mean Newton shift).
+template <typename T>
+__device__ __forceinline__ void restrict_cell(const MGArgs<T>& a, const LevelDesc& F,
+                                              const LevelDesc& C, int I, int J, int K,
+                                              int skip_black = 0) {
   const int nxc = F.crx ? 2 : 1, nyc = F.cry ? 2 : 1, nzc = F.crz ? 2 : 1;
   const int i0 = F.crx ? 2 * I : I, j0 = F.cry ? 2 * J : J, k0 = F.crz ? 2 * K : K;
   T sum = T(0), ssum = T(0);
@@ -144,39 +135,25 @@ __device__ __forceinline__ void restrict_children(const MGArgs<T>& fa, T* rc, T*
     for (int dj = 0; dj < nyc; ++dj)
       for (int di = 0; di < nxc; ++di) {
         const int i = i0 + di, j = j0 + dj, k = k0 + dk;
-        if (!(skip_black && ((i + j + k) & 1))) {
-          const T r = cell_residual(fa, F, i, j, k);
-          sum += r;
-          if constexpr (NORM && sizeof(A) == sizeof(float)) {
-            const float rf = dev::df_from_double((double)r).h;
-            rr = fmaf(rf, rf, rr);
-          } else if constexpr (NORM) {
-            rr = fma((double)r, (double)r, rr);
-          }
-        }
-        if (NORM && want_b) {
-          const double b = fa.r[lidx(F, i, j, k)];
-          if constexpr (sizeof(A) == sizeof(float)) {
-            const float bf = dev::df_from_double(b).h;
-            bb = fmaf(bf, bf, bb);
-          } else {
-            bb = fma(b, b, bb);
-          }
-        }
-        if (sc) ssum += fa.s[lidx(F, i, j, k)];
+        if (!(skip_black && ((i + j + k) & 1))) sum += cell_residual(a, F, i, j, k);
+        if (a.s) ssum += a.s[lidx(F, i, j, k)];
       }
   const T inv = T(1) / T(nxc * nyc * nzc);
   const int idc = lidx(C, I, J, K);
-  rc[idc] = sum * inv;
-  if (sc) sc[idc] = ssum * inv;
+  a.r[idc] = sum * inv;
+  if (a.s) a.s[idc] = ssum * inv;
 }
 
+// x / 4.  In FP64 by the exponent where x and the result are normal numbers: the same value
+// as the multiplication, which would take 19 clocks of an SM's FP64 pipe per warp (7 of
+// prolong_fine's 15 FP64 operations and 10 of prolong_tiled_kernel's 24 are these).
 template <typename T>
-__device__ __forceinline__ void restrict_cell(const MGArgs<T>& a, const LevelDesc& F,
-                                              const LevelDesc& C, int I, int J, int K,
-                                              int skip_black = 0) {
-  double rr = 0.0, bb = 0.0;
-  restrict_children<T, false>(a, a.r, a.s, F, C, I, J, K, skip_black, rr, bb, 0);
+__device__ __forceinline__ T quarter(T x) {
+  if constexpr (sizeof(T) == sizeof(double)) {
+    const int hi = __double2hiint(x);
+    if (((unsigned)(hi >> 20) & 0x7ffu) - 3u < 0x7fcu) return __hiloint2double(hi - (2 << 20), __double2loint(x));
+  }
+  return T(0.25) * x;   // zero, subnormal numbers, infinities, NaN
 }
 
 // Prolongation + correction for the children of coarse cell (I, J, K).
@@ -261,16 +238,16 @@ __device__ __forceinline__ void prolong_fine(const MGArgs<T>& a, const LevelDesc
   auto zcol = [&](int x, int y) -> T {
     const T c0 = e[lidx(C, x, y, K)];
     if (!F.crz) return c0;
-    return (K2 >= 0 && K2 < C.nz) ? fma(T(0.75), c0, T(0.25) * e[lidx(C, x, y, K2)])
+    return (K2 >= 0 && K2 < C.nz) ? fma(T(0.75), c0, quarter(e[lidx(C, x, y, K2)]))
                                   : T(0.5) * c0;
   };
   const T z11 = zcol(I, J);
   T y1 = z11, y2 = T(0);
-  if (F.cry) y1 = fma(T(0.75), z11, T(0.25) * zcol(I, J2));
+  if (F.cry) y1 = fma(T(0.75), z11, quarter(zcol(I, J2)));
   if (F.crx) {
     const T z21 = zcol(I2, J);
-    y2 = F.cry ? fma(T(0.75), z21, T(0.25) * zcol(I2, J2)) : z21;
-    e[lidx(F, i, j, k)] += fma(T(0.75), y1, T(0.25) * y2);
+    y2 = F.cry ? fma(T(0.75), z21, quarter(zcol(I2, J2))) : z21;
+    e[lidx(F, i, j, k)] += fma(T(0.75), y1, quarter(y2));
   } else {
     e[lidx(F, i, j, k)] += y1;
   }

@@ -211,11 +211,11 @@ __device__ __forceinline__ double mid_prolong(E e, int i, int j, int k, int crz,
   auto zcol = [&](int x, int y) -> double {
     const double c0 = e(x, y, K);
     if (!crz) return c0;
-    return in ? fma(0.75, c0, 0.25 * e(x, y, K2)) : 0.5 * c0;
+    return in ? fma(0.75, c0, quarter(e(x, y, K2))) : 0.5 * c0;
   };
   const double z11 = zcol(I, J), z12 = zcol(I, J2), z21 = zcol(I2, J), z22 = zcol(I2, J2);
-  const double y1 = fma(0.75, z11, 0.25 * z12), y2 = fma(0.75, z21, 0.25 * z22);
-  return fma(0.75, y1, 0.25 * y2);
+  const double y1 = fma(0.75, z11, quarter(z12)), y2 = fma(0.75, z21, quarter(z22));
+  return fma(0.75, y1, quarter(y2));
 }
 
 template <bool SC>

@@ -325,23 +325,90 @@ __global__ void __launch_bounds__(256) restrict_kernel(MGArgs<T> a, LevelDesc F,
   restrict_cell(a, F, C, I, J, (int)blockIdx.z, skip_black);
 }
 
+// a thread's part of the blocks' sums: a fixed order (deterministic), read at L2, eight in flight
+__device__ __forceinline__ double sum_partials(const double* P, int nblk, int tid, int nthr) {
+  double s = 0.0;
+  for (int q = tid; q < nblk; q += 8 * nthr) {
+    double v[8];
+#pragma unroll
+    for (int w = 0; w < 8; ++w) v[w] = q + w * nthr < nblk ? __ldcg(P + q + w * nthr) : 0.0;
+#pragma unroll
+    for (int w = 0; w < 8; ++w) s += v[w];
+  }
+  return s;
+}
+
 // Direct FP64 form: the fine level's residual b - A phi after the pre-smoothing,
-// restricted to the first coarse level (8-child mean, red children only when the
-// black residuals vanish) and its squared norm summed on the way; the last block
-// sums the per-block partials in a fixed order, takes the convergence decision
-// (||r|| <= tol ||b||, ||b||^2 summed on the first check of a solve) and sets the
-// loop condition.  phi after the pre-smoothing is the iterate the test accepts.
-template <typename T>
-__global__ void __launch_bounds__(256) restrict_check_kernel(MGArgs<T> fa, T* rc, LevelDesc F,
-                                                             LevelDesc C, int skip_black,
-                                                             CheckArgs ck) {
+// restricted to the first coarse level (8-child mean; the black residuals vanish, see
+// black_residual_zero) and its squared norm summed on the way; the last block sums the
+// per-block partials in a fixed order, takes the convergence decision (||r|| <= tol ||b||,
+// ||b||^2 summed on the first check of a solve) and sets the loop condition.  phi after
+// the pre-smoothing is the iterate the test accepts.
+//
+// The squares are summed in FP32 from FP32 approximations taken with integer operations
+// (the FP64 -> FP32 conversion instruction runs on the FP64 pipe): the norms only scale
+// the stopping test, where a relative error of ~1e-6 in ||r|| is immaterial.
+//
+// A thread holds the 2 x 2 x 2 children of its coarse cell: 24 loads in flight at once and
+// 33 FP64 operations (a loop over the children serialised four loads-to-sum chains).
+// 256x256x32: 34.8 -> 28.6 us, 64x64x16: 16.3 -> 12.3 us (launches timed one by one, which
+// adds about 3.5 us; the reduction's last block about as much).
+__global__ void __launch_bounds__(256) restrict_check_kernel(MGArgs<double> fa, double* rc, LevelDesc F,
+                                                             LevelDesc C, CheckArgs ck) {
   pdl_enter();
   const int I = blockIdx.x * blockDim.x + threadIdx.x;
   const int J = blockIdx.y * blockDim.y + threadIdx.y;
-  float rr = 0.0f, bb = 0.0f;   // FP32 sums of the squares (see restrict_children)
-  if (I < C.nx && J < C.ny)
-    restrict_children<T, true, float>(fa, rc, nullptr, F, C, I, J, (int)blockIdx.z, skip_black, rr,
-                                      bb, ck.first);
+  const int K = blockIdx.z;
+  float rr = 0.0f, bb = 0.0f;
+  if (I < C.nx && J < C.ny) {
+    const double *e = fa.e + F.off, *r = fa.r + F.off;
+    const int nx = F.nx, plane = F.nx * F.ny;
+    // rows 2 J and 2 J + 1 of planes 2 K and 2 K + 1; red cells at x = 2 I + p, p = (dj + dk) & 1
+    const int base = (2 * K * F.ny + 2 * J) * nx + 2 * I;
+    const int xl = I == 0 ? nx - 1 : -1, xr = I + 1 == C.nx ? 2 - nx : 2;
+    const int ym = J == 0 ? (F.ny - 1) * nx : -nx, yp = J + 1 == C.ny ? (2 - F.ny) * nx : 2 * nx;
+    double g[2][2][2], out_x[2][2], out_y[2][2], out_z[2][2], b[2][2], bk[2][2];
+#pragma unroll
+    for (int dk = 0; dk < 2; ++dk)
+#pragma unroll
+      for (int dj = 0; dj < 2; ++dj) {
+        const int p = (dj + dk) & 1, row = base + dk * plane + dj * nx;
+        g[dk][dj][0] = e[row];
+        g[dk][dj][1] = e[row + 1];
+        b[dk][dj] = r[row + p];
+        bk[dk][dj] = ck.first ? r[row + 1 - p] : 0.0;
+        out_x[dk][dj] = e[row + (p ? xr : xl)];
+        out_y[dk][dj] = e[base + dk * plane + p + (dj ? yp : ym)];
+        const bool in = dk ? K + 1 < C.nz : K > 0;
+        out_z[dk][dj] = in ? e[row + p + (dk ? plane : -plane)] : 0.0;
+      }
+    double sum = 0.0;
+#pragma unroll
+    for (int dk = 0; dk < 2; ++dk) {
+      const PlaneCoef<double> c = ldg_struct(fa.coef + F.coef_off + 2 * K + dk);
+#pragma unroll
+      for (int dj = 0; dj < 2; ++dj) {
+        const int p = (dj + dk) & 1;
+        const double x = out_x[dk][dj] + g[dk][dj][1 - p];
+        const double y = out_y[dk][dj] + g[dk][1 - dj][p];
+        const double z = g[1 - dk][dj][p], o = out_z[dk][dj];
+        double acc = fma(c.cx, x, b[dk][dj]);
+        acc = fma(c.cy, y, acc);
+        acc = fma(c.czlo, dk ? z : o, acc);
+        acc = fma(c.czhi, dk ? o : z, acc);
+        const double q = fma(-c.diag, g[dk][dj][p], acc);
+        sum += q;
+        const float qf = df_from_double(q).h;
+        rr = fmaf(qf, qf, rr);
+        if (ck.first) {   // in the order of the cells
+          const float b0 = df_from_double(p ? bk[dk][dj] : b[dk][dj]).h, b1 = df_from_double(p ? b[dk][dj] : bk[dk][dj]).h;
+          bb = fmaf(b0, b0, bb);
+          bb = fmaf(b1, b1, bb);
+        }
+      }
+    }
+    rc[lidx(C, I, J, K)] = sum * 0.125;
+  }
   block_sum2f(rr, bb);
   double zz = 0.0;
   __shared__ bool last;
@@ -358,12 +425,8 @@ __global__ void __launch_bounds__(256) restrict_check_kernel(MGArgs<T> fa, T* rc
   __syncthreads();
   if (!last) return;
   __threadfence();
-  double sr = 0.0, sb = 0.0;
-  const volatile double* P = ck.partials;
-  for (int q = tid; q < nblk; q += blockDim.x * blockDim.y) {
-    sr += P[q];
-    sb += P[nblk + q];
-  }
+  double sr = sum_partials(ck.partials, nblk, tid, blockDim.x * blockDim.y);
+  double sb = ck.first ? sum_partials(ck.partials + nblk, nblk, tid, blockDim.x * blockDim.y) : 0.0;
   block_sum3(sr, sb, zz);
   if (tid == 0) {
     ck.stats->done_ctr = 0;
@@ -420,15 +483,18 @@ __global__ void __launch_bounds__(256) restrict4_kernel(MGArgs<T> a, LevelDesc F
   }
 }
 
-// Prolongation + correction with one thread per fine cell (prolong_fine).
-template <typename T>
+// Prolongation + correction with one thread per fine cell (prolong_fine).  BLACK: of the
+// black cells only, one per pair of an even row; the sweep that follows relaxes the red
+// cells before anything reads them.
+template <typename T, bool BLACK>
 __global__ void __launch_bounds__(256) prolong_fine_kernel(MGArgs<T> a, LevelDesc F, LevelDesc C,
                                                            int constant) {
   pdl_enter();
-  const int i = blockIdx.x * blockDim.x + threadIdx.x;
-  const int j = blockIdx.y * blockDim.y + threadIdx.y;
+  const int ix = blockIdx.x * blockDim.x + threadIdx.x;
+  const int j = blockIdx.y * blockDim.y + threadIdx.y, k = blockIdx.z;
+  const int i = BLACK ? 2 * ix + ((j + k + 1) & 1) : ix;
   if (i >= F.nx || j >= F.ny) return;
-  prolong_fine(a, F, C, i, j, (int)blockIdx.z, constant);
+  prolong_fine(a, F, C, i, j, k, constant);
 }
 
 template <typename T>
@@ -441,84 +507,85 @@ __global__ void __launch_bounds__(256) prolong_kernel(MGArgs<T> a, LevelDesc F, 
   prolong_cell(a, F, C, I, J, (int)blockIdx.z, constant);
 }
 
-// Prolongation + correction onto the fine level in the FP64 form, tiled: the
-// separable trilinear interpolation (3/4 own, 1/4 neighbour per direction) is
-// done in y and then x once per coarse plane through shared memory, and then
-// in z while the block marches up its coarse planes with the interpolated
-// planes K-1, K, K+1 in registers.  An electrode beyond the coarse grid is a
-// ghost plane holding -e (zero correction on the electrode face).  About 40
-// FP64 operations per coarse cell against about 84 for the per-cell form
-// (prolong_cell), which recomputes its neighbours' interpolations; used only
-// where that arithmetic, not latency, bounds the launch.
-// coarse columns (x, y) and planes per block; measured on the 256x256x32 stack
-// (FP64, 500 steps): (32, 4, 4) 1227, (32, 8, 4) 1224, (32, 8, 2) 1216,
-// (32, 4, 8) 1213, (32, 16, 4) 1207 Mcell-steps/s
-constexpr int kPX = 32, kPY = 4, kPZ = 4;
+// Prolongation + correction onto the fine level in the FP64 form, tiled: the separable
+// trilinear interpolation (3/4 own, 1/4 neighbour per direction) in y by each thread for
+// its coarse column, in x with the neighbours' values from shared memory, and in z while
+// the block marches up its coarse planes with the last plane's four values in registers.
+// An electrode beyond the coarse grid is a ghost plane holding -e (zero correction on the
+// electrode face).
+// BLACK: the black cells only (see prolong_fine_kernel): 14 FP64 operations per coarse
+// cell and one barrier per plane instead of 37 and three for all cells with both
+// interpolations through shared memory.  256x256x32: 40 -> 27 us,
+// 64x64x16: 19 -> 8.8 us (launches timed one by one, which adds about 3.5 us).
+constexpr int kPX = 32, kPY = 2;   // coarse columns (x, y) per block
 
-template <typename T>
-__global__ void __launch_bounds__(kPX* kPY) prolong_tiled_kernel(MGArgs<T> a, LevelDesc F,
-                                                                LevelDesc C, T* fine) {
+template <bool BLACK>
+__global__ void __launch_bounds__(kPX* kPY) prolong_tiled_kernel(const double* __restrict__ e, LevelDesc F, LevelDesc C,
+                                                                double* fine, int kz) {
   pdl_enter();
-  __shared__ T sE[kPY + 2][kPX + 2];     // coarse e of one plane: tile + periodic halo
-  __shared__ T sY[2 * kPY][kPX + 2];     // interpolated in y: fine rows x coarse columns
+  __shared__ double sY[2][2 * kPY][kPX + 2];   // interpolated in y: fine rows x coarse columns
   const int tx = threadIdx.x, ty = threadIdx.y, tid = ty * kPX + tx;
-  const int I0 = blockIdx.x * kPX, J0 = blockIdx.y * kPY;
-  const int I = I0 + tx, J = J0 + ty;
+  const int I0 = blockIdx.x * kPX, J0 = blockIdx.y * kPY, I = I0 + tx, J = J0 + ty;
   const bool own = I < C.nx && J < C.ny;
-  const int K0 = blockIdx.z * kPZ, K1 = min(C.nz, K0 + kPZ);
-  T* e = a.e;
-  T* ef = fine ? fine : e + F.off;       // the level's corrections, or phi (direct form)
-  auto plane_xy = [&](int K, T out[4]) {
-    __syncthreads();                     // the previous plane's readers are done with sE, sY
-    for (int q = tid; q < (kPY + 2) * (kPX + 2); q += kPX * kPY) {
-      const int r = q / (kPX + 2), col = q - r * (kPX + 2);
-      int gy = (J0 - 1 + r) % C.ny, gx = (I0 - 1 + col) % C.nx;
-      if (gy < 0) gy += C.ny;
-      if (gx < 0) gx += C.nx;
-      sE[r][col] = e[C.off + ((long long)K * C.ny + gy) * C.nx + gx];
-    }
-    __syncthreads();
-    for (int q = tid; q < 2 * kPY * (kPX + 2); q += kPX * kPY) {
-      const int fr = q / (kPX + 2), col = q - fr * (kPX + 2);
-      const int ry = fr >> 1, b = fr & 1;
-      sY[fr][col] = fma(T(0.75), sE[ry + 1][col], T(0.25) * sE[ry + 2 * b][col]);
-    }
-    __syncthreads();
-#pragma unroll
-    for (int b = 0; b < 2; ++b) {
-      const T yc = sY[2 * ty + b][tx + 1];
-      out[2 * b] = fma(T(0.75), yc, T(0.25) * sY[2 * ty + b][tx]);
-      out[2 * b + 1] = fma(T(0.75), yc, T(0.25) * sY[2 * ty + b][tx + 2]);
-    }
+  const int K0 = blockIdx.z * kz, K1 = min(C.nz, K0 + kz);
+  const int ks = max(K0 - 1, 0), ke = min(K1, C.nz - 1);
+  const int cplane = C.nx * C.ny, plane = F.nx * F.ny;
+  // own column: coarse rows J - 1, J, J + 1 (periodic images beyond the grid)
+  const int gx = I % C.nx, gy = J % C.ny;
+  const int o0 = gy * C.nx + gx, om = (gy == 0 ? C.ny - 1 : gy - 1) * C.nx + gx, op = (gy + 1 == C.ny ? 0 : gy + 1) * C.nx + gx;
+  // the columns left and right of the tile: thread tid < 4 kPY one fine row of one of them
+  const bool halo = tid < 4 * kPY;
+  const int hr = tid % (2 * kPY), right = tid / (2 * kPY);
+  const int hx = right ? (I0 + kPX) % C.nx : (I0 + C.nx - 1) % C.nx;
+  const int hy = (J0 + (hr >> 1)) % C.ny;
+  const int h0 = hy * C.nx + hx, h1 = ((hr & 1) ? (hy + 1 == C.ny ? 0 : hy + 1) : (hy == 0 ? C.ny - 1 : hy - 1)) * C.nx + hx;
+  double e0, em, ep, q0 = 0.0, q1 = 0.0;
+  auto load = [&](int K) {
+    const double* c = e + (long long)K * cplane;
+    e0 = c[o0]; em = c[om]; ep = c[op];
+    if (halo) { q0 = c[h0]; q1 = c[h1]; }
   };
-  T xm[4], xc[4], xp[4];
-  plane_xy(K0, xc);
-  if (K0 > 0) {
-    plane_xy(K0 - 1, xm);
-  } else {
+  load(ks);
+  double xm[4], v[4];
+  double* const col = fine + (long long)(2 * J) * F.nx + 2 * I;
+  for (int K = ks; K <= ke; ++K) {
+    const bool lo = K >= K0 && K < K1, hi = K > K0;    // fine planes 2 K and 2 K - 1 are the block's
+    double fl[4], fh[4];
 #pragma unroll
-    for (int q = 0; q < 4; ++q) xm[q] = -xc[q];
-  }
-  for (int K = K0; K < K1; ++K) {
-    if (K + 1 < C.nz) {
-      plane_xy(K + 1, xp);
-    } else {
+    for (int q = 0; q < 4; ++q) {   // column (di, b) = (q & 1, q >> 1)
+      const int o = (q >> 1) * F.nx + (q & 1);
+      const bool odd = (q ^ (q >> 1)) & 1;
+      if ((!BLACK || odd) && own && lo) fl[q] = col[(long long)(2 * K) * plane + o];
+      if ((!BLACK || !odd) && own && hi) fh[q] = col[(long long)(2 * K - 1) * plane + o];
+    }
+    double (*Y)[kPX + 2] = sY[K & 1];
+    Y[2 * ty][tx + 1] = fma(0.75, e0, quarter(em));
+    Y[2 * ty + 1][tx + 1] = fma(0.75, e0, quarter(ep));
+    if (halo) Y[hr][right ? kPX + 1 : 0] = fma(0.75, q0, quarter(q1));
+    if (K < ke) load(K + 1);
+    __syncthreads();
 #pragma unroll
-      for (int q = 0; q < 4; ++q) xp[q] = -xc[q];
+    for (int q = 0; q < 4; ++q) {
+      const double* y = Y[2 * ty + (q >> 1)] + tx;
+      v[q] = fma(0.75, y[1], quarter(y[(q & 1) ? 2 : 0]));
+    }
+    if (K == 0) {
+#pragma unroll
+      for (int q = 0; q < 4; ++q) xm[q] = -v[q];
     }
     if (own) {
 #pragma unroll
-      for (int b = 0; b < 2; ++b) {
-        T* lo = ef + ((long long)(2 * K) * F.ny + 2 * J + b) * F.nx + 2 * I;
-        T* hi = lo + (long long)F.ny * F.nx;
-        lo[0] += fma(T(0.75), xc[2 * b], T(0.25) * xm[2 * b]);
-        lo[1] += fma(T(0.75), xc[2 * b + 1], T(0.25) * xm[2 * b + 1]);
-        hi[0] += fma(T(0.75), xc[2 * b], T(0.25) * xp[2 * b]);
-        hi[1] += fma(T(0.75), xc[2 * b + 1], T(0.25) * xp[2 * b + 1]);
+      for (int q = 0; q < 4; ++q) {
+        const int o = (q >> 1) * F.nx + (q & 1);
+        const bool odd = (q ^ (q >> 1)) & 1;
+        if ((!BLACK || odd) && lo) col[(long long)(2 * K) * plane + o] = fl[q] + fma(0.75, v[q], quarter(xm[q]));
+        if ((!BLACK || !odd) && hi) col[(long long)(2 * K - 1) * plane + o] = fh[q] + fma(0.75, xm[q], quarter(v[q]));
+        if ((!BLACK || !odd) && lo && K == C.nz - 1)
+          col[(long long)(2 * K + 1) * plane + o] += fma(0.75, v[q], quarter(-v[q]));
       }
     }
 #pragma unroll
-    for (int q = 0; q < 4; ++q) { xm[q] = xc[q]; xc[q] = xp[q]; }
+    for (int q = 0; q < 4; ++q) xm[q] = v[q];
   }
 }
 
@@ -593,23 +660,11 @@ __global__ void __launch_bounds__(kResidBX* kResidBY / R, DFC && SC == 1 ? 3 * R
   __syncthreads();
   if (!last) return;
   __threadfence();
-  // fixed-order sum of the partials (deterministic), read at L2, eight in flight
   double sr = 0.0, sb = 0.0, sq = 0.0;
   const int nthr = blockDim.x * blockDim.y;
-  auto sum = [&](const double* P) {
-    double s = 0.0;
-    for (int q = tid; q < nblk; q += 8 * nthr) {
-      double v[8];
-#pragma unroll
-      for (int w = 0; w < 8; ++w) v[w] = q + w * nthr < nblk ? __ldcg(P + q + w * nthr) : 0.0;
-#pragma unroll
-      for (int w = 0; w < 8; ++w) s += v[w];
-    }
-    return s;
-  };
-  sr = sum(a.partials);
-  if (a.first) sb = sum(a.partials + nblk);
-  if (SC) sq = sum(a.partials + 2 * nblk);
+  sr = sum_partials(a.partials, nblk, tid, nthr);
+  if (a.first) sb = sum_partials(a.partials + nblk, nblk, tid, nthr);
+  if (SC) sq = sum_partials(a.partials + 2 * nblk, nblk, tid, nthr);
   block_sum3(sr, sb, sq);
   if (tid == 0) {
     a.stats->done_ctr = 0;
@@ -807,18 +862,24 @@ void launch_smooth_rb(const MGArgs<T>& a, const LevelDesc& L, const T* e_in, T* 
   }
 }
 
+// the check's blocks: one warp each where the level leaves SMs idle otherwise
+static void check_shape(const LevelDesc& C, dim3& block, dim3& grid) {
+  int t = 128;
+  while (t > 32 && C.ncell < 2LL * 152 * t) t >>= 1;
+  block_shape(C.nx, C.ny, block, grid, C.nz, t);
+}
+
 dim3 check_grid(const LevelDesc& C) {
   dim3 block, grid;
-  block_shape(C.nx, C.ny, block, grid, C.nz);
+  check_shape(C, block, grid);
   return grid;
 }
 
 void launch_restrict_check(const MGArgs<double>& fa, double* rc, const LevelDesc& F,
-                           const LevelDesc& C, int nu1, const CheckArgs& ck, cudaStream_t s) {
+                           const LevelDesc& C, const CheckArgs& ck, cudaStream_t s) {
   dim3 block, grid;
-  block_shape(C.nx, C.ny, block, grid, C.nz);
-  launch_k(restrict_check_kernel<double>, grid, block, 0, s, fa, rc, F, C,
-           black_residual_zero(F, nu1), ck);
+  check_shape(C, block, grid);
+  launch_k(restrict_check_kernel, grid, block, 0, s, fa, rc, F, C, ck);
 }
 
 template <typename T>
@@ -839,19 +900,29 @@ void launch_restrict(const MGArgs<T>& a, const LevelDesc& F, const LevelDesc& C,
 
 template <typename T>
 void launch_prolong(const MGArgs<T>& a, const LevelDesc& F, const LevelDesc& C, int constant,
-                    cudaStream_t s, bool tiled, T* fine) {
-  if (fine || (tiled && F.crx && F.cry && F.crz && !constant)) {
-    const dim3 grid((C.nx + kPX - 1) / kPX, (C.ny + kPY - 1) / kPY, (C.nz + kPZ - 1) / kPZ);
-    launch_k(prolong_tiled_kernel<T>, grid, dim3(kPX, kPY), 0, s, a, F, C, fine);
-    return;
+                    cudaStream_t s, bool tiled, T* fine, int sweeps) {
+  const bool black = black_residual_zero(F, sweeps) && !(F.nx & 1);
+  if constexpr (sizeof(T) == sizeof(double)) {
+    if (fine || (tiled && F.crx && F.cry && F.crz && !constant)) {
+      // planes per block: four, fewer where that leaves SMs idle (a block computes one
+      // more plane than it holds)
+      dim3 grid((C.nx + kPX - 1) / kPX, (C.ny + kPY - 1) / kPY, 1);
+      int kz = 4;
+      while (kz > 1 && (long long)grid.x * grid.y * ((C.nz + kz - 1) / kz) < 304) kz >>= 1;
+      grid.z = (C.nz + kz - 1) / kz;
+      launch_k(black ? prolong_tiled_kernel<true> : prolong_tiled_kernel<false>, grid, dim3(kPX, kPY), 0, s, a.e + C.off,
+               F, C, fine ? fine : a.e + F.off, kz);
+      return;
+    }
   }
   if (sizeof(T) == sizeof(double) || F.ncell <= kSmallTransfer) {
     // one thread per fine cell, a 15-operation chain instead of 84 per coarse
     // cell, where latency bounds the prolongation: FP64 levels, and FP32 levels
     // up to kSmallTransfer fine cells
     dim3 block, grid;
-    block_shape(F.nx, F.ny, block, grid, F.nz, spread_threads(F.ncell));
-    launch_k(prolong_fine_kernel<T>, grid, block, 0, s, a, F, C, constant);
+    const int w = black ? F.nx >> 1 : F.nx;
+    block_shape(w, F.ny, block, grid, F.nz, spread_threads((long long)w * F.ny * F.nz));
+    launch_k(black ? prolong_fine_kernel<T, true> : prolong_fine_kernel<T, false>, grid, block, 0, s, a, F, C, constant);
     return;
   }
   dim3 block, grid;
@@ -983,7 +1054,7 @@ cudaError_t launch_carrier_exp_df(const float* u_hl, double* ep, double* em, lon
   template void launch_restrict<T>(const MGArgs<T>&, const LevelDesc&, const LevelDesc&, int,   \
                                    cudaStream_t);                                               \
   template void launch_prolong<T>(const MGArgs<T>&, const LevelDesc&, const LevelDesc&, int,    \
-                                  cudaStream_t, bool, T*);                                      \
+                                  cudaStream_t, bool, T*, int);                                 \
   template size_t tail_smem_bytes<T>(long long, bool);                                          \
   template cudaError_t tail_prepare<T>(size_t);                                                 \
   template void launch_tail<T>(const MGArgs<T>&, const TailArgs&, size_t, cudaStream_t);        \
