@@ -48,6 +48,20 @@ __device__ __forceinline__ void exp_pm(double u, double& ep, double& em) {
   em = fma(sm, E - O, sm);
 }
 
+// e^{-x} alone for 0 <= x < 700 (the same reduction and table)
+__device__ __forceinline__ double exp_minus(double x) {
+  const double shift = 0x1.8p52;
+  const double t = fma(-x, kExpInvL, shift);
+  const double kd = __dadd_rn(t, -shift);
+  const int k = __double2loint(t);
+  double r = fma(-kd, kExpLhi, -x);
+  r = fma(-kd, kExpLlo, r);
+  const double r2 = __dmul_rn(r, r);
+  const double p = fma(r2, fma(r, fma(r, 1.0 / 120.0, 1.0 / 24.0), 1.0 / 6.0), __dmul_rn(r, 0.5));
+  const double s = scale_pow2(__ldg(&kExpTab[k & ((1 << kExpTabBits) - 1)].x), k >> kExpTabBits);
+  return fma(s, fma(r, p, r), s);
+}
+
 // The same pair in double-float arithmetic on the FP32 pipe, for |u.h| <= kExpDFMax
 // (callers take exp_pm beyond).  The reduction r = u - k ln2/64 uses ln2/64 =
 // C1 + C2 + C3 + C4 with C1..C3 of 11 significant bits, so k C1, k C2, k C3 are

@@ -86,5 +86,18 @@ __device__ __forceinline__ df df_from_double(double x) {
   return {h, __uint_as_float(sign | ((unsigned)(nb + e - 949) << 23) | (m & 0x7fffffu))};
 }
 
+// a float as an FP64 value (exact for normal floats; FP32 subnormals, below
+// 2^-126, become signed zero)
+__device__ __forceinline__ double f64_of_float(float f) {
+  const unsigned u = __float_as_uint(f);
+  const unsigned sign = u & 0x80000000u, e = (u >> 23) & 0xffu, m = u & 0x7fffffu;
+  unsigned hi;
+  if (e == 0u) hi = sign;
+  else if (e == 255u) hi = sign | 0x7ff00000u | (m >> 3);
+  else hi = sign | ((e + 896u) << 20) | (m >> 3);
+  const unsigned lo = e == 0u ? 0u : (m & 7u) << 29;
+  return __longlong_as_double((long long)(((unsigned long long)hi << 32) | lo));
+}
+
 }  // namespace dev
 }  // namespace fx

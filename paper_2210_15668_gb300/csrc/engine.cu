@@ -446,6 +446,8 @@ ferrox_status build_planes(ferrox_ctx* c) {
         p.Nc = effective_dos(L.m_e, L.T);
         p.Nv = effective_dos(L.m_p, L.T);
         fd_reference(p.Nc, p.Nv, L.E_g, L.T, L.N_A, L.N_D, &p.eta_e0, &p.eta_p0);
+        p.em_e0 = std::exp(-p.eta_e0);
+        p.em_p0 = std::exp(-p.eta_p0);
       }
       c->has_sc = true;
     }
@@ -1424,11 +1426,15 @@ ferrox_status ferrox_init_geometry(ferrox_ctx** out, const ferrox_geometry* geom
   const size_t tsz = mixed ? sizeof(float) : sizeof(double);
   plan_tail(ctx, tsz, true);
   {
-    // residual grid: split the columns into z chunks (halving, at least 4 planes
-    // each) until there are about four waves of blocks on 152 SMs
+    // residual grid: split the columns into z chunks (halving, at least 4 planes each)
+    // until there are about four waves of blocks on 152 SMs; down to two planes where
+    // carriers in FP64 make the semiconductor's planes several times dearer than the
+    // others (64^3 cube with Fermi-Dirac carriers on 16 planes, launches timed one by one:
+    // 49 us with 4 planes, 43 with 2, 55 with 1)
+    const int least = carrier_kind(ctx) == 2 || (ctx->has_sc && !mixed) ? 2 : 4;
     const int bxy = ((ctx->nx + kResidBX - 1) / kResidBX) * ((ctx->ny + kResidBY - 1) / kResidBY);
     int zc = 1;
-    while ((long long)bxy * zc < 4LL * 152 * 3 && ctx->nz / (2 * zc) >= 4) zc *= 2;
+    while ((long long)bxy * zc < 4LL * 152 * 3 && ctx->nz / (2 * zc) >= least) zc *= 2;
     ctx->resid_kchunk = (ctx->nz + zc - 1) / zc;
     ctx->resid_blocks = bxy * ((ctx->nz + ctx->resid_kchunk - 1) / ctx->resid_kchunk);
     // the double-float form: at least 8 planes per thread (its block reduction and

@@ -102,6 +102,7 @@ struct PlaneTDGL {
   double kq, n0, p0, Nnet, inv_vt;
   // Fermi-Dirac: n = Nc F(eta_e0 + phi/VT), p = Nv F(eta_p0 - phi/VT)
   double Nc, Nv, eta_e0, eta_p0;
+  double em_e0, em_p0;                // e^-eta_e0, e^-eta_p0
   // kq n0, kq p0, kq Nnet (the double-float residual forms rho from these)
   double kqn0, kqp0, kqN;
 };

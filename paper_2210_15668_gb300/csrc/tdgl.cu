@@ -56,18 +56,6 @@ constexpr int kCX = 32, kCY = 2, kCZ = 4;
 
 __device__ __forceinline__ float df_diff(df a, df b) { return (a.h - b.h) + (a.l - b.l); }
 
-// a float as an FP64 value (exact for normal floats; FP32 subnormals, below
-// 2^-126, become signed zero)
-__device__ __forceinline__ double f64_of_float(float f) {
-  const unsigned u = __float_as_uint(f);
-  const unsigned sign = u & 0x80000000u, e = (u >> 23) & 0xffu, m = u & 0x7fffffu;
-  unsigned hi;
-  if (e == 0u) hi = sign;
-  else if (e == 255u) hi = sign | 0x7ff00000u | (m >> 3);
-  else hi = sign | ((e + 896u) << 20) | (m >> 3);
-  const unsigned lo = e == 0u ? 0u : (m & 7u) << 29;
-  return __longlong_as_double((long long)(((unsigned long long)hi << 32) | lo));
-}
 
 // z-component force of plane k (FP32 arithmetic on double-float differences)
 __device__ __forceinline__ float force_z_f32(const TDGLArgs& a, const PlaneF32& q, const PlaneF32* qs,
