@@ -80,7 +80,7 @@ struct ferrox_ctx {
   double* phi_prev = nullptr;         // previous step's potential (guess = 1)
   void* e_arena = nullptr;
   float* eb_arena = nullptr;          // black corrections between the legs of a V-cycle
-  MidPlan mid;                        // FP64: middle levels and tail in one cluster launch (mid.first > 0)
+  MidPlan mid;                        // middle levels and tail in one cluster launch (mid.first > 0)
   LevelDesc* lvm_d = nullptr;         // ... its tail's levels
   bool legs = false;                  // FP32 levels run one launch per leg (leg_device.cuh)
   void* e_alt = nullptr;              // second error array of the fused sweeps (largest such level)
@@ -212,28 +212,39 @@ void plan_tail(ferrox_ctx* c, size_t elem_size, bool wide = false) {
   }
 }
 
-// The levels of an FP64 V-cycle that run with the tail in one cluster launch (mid.cu):
-// from the first level of at most kMidCells cells down to the tail (with a shift, where
-// the tail's first level is relaxed and not solved by its inverse, to a smaller one: one
-// SM's FP64 rate bounds the tail).  Fills everything but the device pointers; first = 0
-// where the levels do not fit the kernel.
+// The levels of a V-cycle that run with the tail in one cluster launch (mid.cu): from the
+// first level whose pairs fit the CTAs down to the tail; to the coarsest level where the
+// tail is relaxed and not solved by an inverse (a Newton shift, or a coarsest level too
+// large for one), because a phase of the cluster is shorter than one of the tail's CTA.
+// FP32 stacks whose tail is solved by its inverse keep the legs (256x256x32: 5.48 ms for
+// five solves, 5.47 with the levels below 64x64x8 in the cluster).  Fills everything but
+// the device pointers; first = 0 where the levels do not fit the kernel.
+template <typename T>
 void plan_mid(const ferrox_ctx* c, MidPlan& m, std::vector<LevelDesc>& tail) {
   m.first = 0;
-  if (c->num.nu1 < 1 || c->num.nu2 < 1) return;
-  auto fits = [&](int l) { return leg_level(c->lv[l]) && c->lv[l].nx > 1 && c->lv[l].ny > 1; };
+  const int coarsest = (int)c->lv.size() - 1, most = mid_threads_max<T>();
+  if (c->num.nu1 < 1 || c->num.nu2 < 1 || c->tail_first < 1) return;
+  const bool relaxed = c->shift || (c->tail_first == coarsest && c->lv[coarsest].ncell > kDenseWide);
+  if (sizeof(T) == sizeof(float) && !relaxed) return;
+  auto fits = [&](int l) {   // a proper colouring by pairs
+    const LevelDesc& L = c->lv[l];
+    return !(L.nx & 1) && !(L.ny & 1) && (l == coarsest || L.crx || L.cry || L.crz);
+  };
   int first = 1, end = c->tail_first;
-  while (first < end && c->lv[first].ncell > kMidCells) ++first;
-  if (c->shift)
-    while (end + 1 < (int)c->lv.size() && end - first < kMidMax && fits(end)) ++end;
+  while (first < end && c->lv[first].ncell > 2LL * kMidCtas * kMidPairs) ++first;
+  if (relaxed)
+    while (end <= coarsest && end - first < kMidMax && fits(end)) ++end;
   for (int l = first; l < end; ++l)
     if (!fits(l)) return;
-  if (end <= first || end - first > kMidMax || c->tail_first <= first) return;
+  const bool bottom = end > coarsest;
+  if (end - first < (bottom ? 2 : 1) || end - first > kMidMax) return;
   MidArgs& a = m.args;
   a = MidArgs{};
   const int narr = c->shift ? 3 : 2;
   a.n = end - first;
   a.nu1 = c->num.nu1;
   a.nu2 = c->num.nu2;
+  a.bottom = bottom ? c->num.bottom_sweeps : 0;
   int off = 16, per0 = 0;   // two zeros first
   for (int q = 0; q < a.n; ++q) {
     MidLevel& L = a.lv[q];
@@ -248,7 +259,7 @@ void plan_mid(const ferrox_ctx* c, MidPlan& m, std::vector<LevelDesc>& tail) {
     L.mx = magic(L.d.nx / 2);
     L.my = magic(L.d.ny);
     a.planes += L.d.nz;
-    const int bytes = 16 << L.sh;
+    const int bytes = std::max(16, (int)(2 * sizeof(T)) << L.sh);
     L.e_off = off;
     L.r_off = off + bytes;
     L.s_off = off + 2 * bytes;
@@ -256,22 +267,33 @@ void plan_mid(const ferrox_ctx* c, MidPlan& m, std::vector<LevelDesc>& tail) {
     per0 = std::max(per0, 1 << L.sh);
   }
   a.coef_off = off;
-  off += a.planes * (int)sizeof(PlaneCoef<double>);
+  off += a.planes * (int)sizeof(PlaneCoef<T>);
   a.q_off = (off + 15) / 16 * 16;
-  off = a.q_off + 8 * per0;
+  off = a.q_off + (int)sizeof(T) * per0;
   a.tail_off = (off + 15) / 16 * 16;
-  a.coarse = c->lv[end];
-  const long long base = a.coarse.off;
-  tail.assign(c->lv.begin() + end, c->lv.end());
-  for (auto& t : tail) t.off -= base;
-  a.tail.nlev = (int)tail.size();
-  a.tail.elems = c->arena - base;
-  a.tail.base = base;
-  a.tail.nu1 = a.nu1; a.tail.nu2 = a.nu2; a.tail.bottom_sweeps = c->num.bottom_sweeps;
-  a.tail.constant = 0;
-  m.smem = a.tail_off + (int)(a.tail.elems * (long long)sizeof(double) * narr);
-  m.threads = std::max(256, per0);
-  if (per0 > kMidThreadsMax || m.smem > kMidMaxSmem) return;
+  long long smem = a.tail_off, want = std::max(256, per0);
+  if (per0 > kMidPairs) return;   // odd sizes round up
+  if (!bottom) {
+    a.coarse = c->lv[end];
+    a.single = a.coarse.ncell == 1 && c->num.bottom_sweeps == 1;
+    const long long base = a.coarse.off;
+    tail.assign(c->lv.begin() + end, c->lv.end());
+    for (auto& t : tail) t.off -= base;
+    a.tail.nlev = (int)tail.size();
+    a.tail.elems = c->arena - base;
+    a.tail.base = base;
+    a.tail.nu1 = a.nu1; a.tail.nu2 = a.nu2; a.tail.bottom_sweeps = c->num.bottom_sweeps;
+    a.tail.constant = 0;
+    smem += a.tail.elems * (long long)sizeof(T) * narr;
+    // the tail on CTA 0: a pair of its first level per thread, two of a coarsest level with
+    // many sweeps (tail_smooth_held)
+    const LevelDesc &T0 = tail.front(), &B = tail.back();
+    want = std::max(want, std::min<long long>(most, (T0.ncell / 2 + 31) / 32 * 32));
+    if (c->num.bottom_sweeps >= 8) want = std::max(want, ((B.nx + 1) / 2 * (long long)B.ny * B.nz / 2 + 32) / 32 * 32);
+  }
+  if (want > most || smem > kMidMaxSmem) return;
+  m.smem = (int)smem;
+  m.threads = (int)want;
   m.first = first;
 }
 
@@ -587,11 +609,11 @@ bool rb_sweeps(const ferrox_ctx* c, int l, int nu) {
   return c->e_alt && nu % 2 == 0 && smooth_rb_tile<T>(c->lv[l], c->shift) > 0;
 }
 
-// Levels whose smoothing and transfers run as one launch per V-cycle leg
-bool leg_at(const ferrox_ctx* c, int l) { return c->legs && l < c->tail_first && leg_level(c->lv[l]); }
-
 // the first level that the V-cycle's bottom launch takes
 int mid_or_tail(const ferrox_ctx* c) { return c->mid.first > 0 ? c->mid.first : c->tail_first; }
+
+// Levels whose smoothing and transfers run as one launch per V-cycle leg
+bool leg_at(const ferrox_ctx* c, int l) { return c->legs && l < mid_or_tail(c) && leg_level(c->lv[l]); }
 
 // kernels of one smoothing of level l with nu sweeps
 int smoothing_launches(const ferrox_ctx* c, int l, int nu) {
@@ -676,11 +698,11 @@ void enqueue_levels(ferrox_ctx* c, cudaStream_t s, W wrap, int l0, bool first, b
     wrap(FERROX_K_RESTRICT, restrict_bytes<T>(c->lv[l], c->lv[l + 1]),
          [&] { launch_restrict<T>(a, c->lv[l], c->lv[l + 1], nu1, s); });
   }
-  if (lt < c->tail_first) {
+  if (c->mid.first > 0) {
     // the arrays of the levels above the tail in and out, and the tail's
     double mb = 0.0;
     for (int l = lt; l <= L; ++l) mb += 2.0 * (double)c->lv[l].ncell * sizeof(T);
-    if constexpr (sizeof(T) == sizeof(double)) wrap(FERROX_K_TAIL, mb, [&] { launch_mid(a, c->mid, s); });
+    wrap(FERROX_K_TAIL, mb, [&] { launch_mid<T>(a, c->mid, s); });
   } else if (c->dense_wide_d) {
     // the whole tail as one exact solve of its first level, spread over the SMs
     const LevelDesc& B = c->lv[lt];
@@ -1574,15 +1596,20 @@ ferrox_status ferrox_init_geometry(ferrox_ctx** out, const ferrox_geometry* geom
   }
   FX_INIT_CK(cudaMemcpy(ctx->planes_d, ctx->planes.data(), ctx->nz * sizeof(PlaneTDGL),
                         cudaMemcpyHostToDevice));
-  if (!mixed && !(rb_env && rb_env[0] == '0')) {
+  if (!(rb_env && rb_env[0] == '0')) {
     std::vector<LevelDesc> tail;
-    plan_mid(ctx, ctx->mid, tail);
-    if (ctx->mid.first > 0 && !mid_prepare(ctx->mid, ctx->shift)) ctx->mid.first = 0;
+    if (mixed) plan_mid<float>(ctx, ctx->mid, tail);
+    else plan_mid<double>(ctx, ctx->mid, tail);
+    if (ctx->mid.first > 0 &&
+        !(mixed ? mid_prepare<float>(ctx->mid, ctx->shift) : mid_prepare<double>(ctx->mid, ctx->shift)))
+      ctx->mid.first = 0;
     if (ctx->mid.first > 0) {
-      FX_INIT_CK(cudaMalloc(&ctx->lvm_d, tail.size() * sizeof(LevelDesc)));
-      FX_INIT_CK(cudaMemcpy(ctx->lvm_d, tail.data(), tail.size() * sizeof(LevelDesc), cudaMemcpyHostToDevice));
+      if (!tail.empty()) {
+        FX_INIT_CK(cudaMalloc(&ctx->lvm_d, tail.size() * sizeof(LevelDesc)));
+        FX_INIT_CK(cudaMemcpy(ctx->lvm_d, tail.data(), tail.size() * sizeof(LevelDesc), cudaMemcpyHostToDevice));
+      }
       MidArgs& a = ctx->mid.args;
-      a.dense = static_cast<const double*>(ctx->dense_wide_d);
+      a.dense = ctx->dense_wide_d;
       a.tail.lv = ctx->lvm_d;
       a.tail.dense = ctx->dense_d;
       a.tail.dense_lev = ctx->dense_lev;

@@ -256,10 +256,12 @@ struct TailArgs {
   int pad;
 };
 
-// The middle levels of an FP64 V-cycle and the tail in one launch of one cluster (mid.cu)
+// The middle levels of a V-cycle and the tail in one launch of one cluster (mid.cu)
 constexpr int kMidCtas = 16;             // CTAs of the cluster
-constexpr int kMidThreadsMax = 512;      // pairs of a level a CTA may hold, one per thread
-constexpr long long kMidCells = 16384;   // the first middle level's cells at most
+constexpr int kMidPairs = 512;           // pairs of a level a CTA may hold, one per thread
+// threads of a CTA: more than its pairs where the tail's coarsest level is large
+template <typename T>
+__host__ __device__ constexpr int mid_threads_max() { return sizeof(T) == sizeof(double) ? 512 : 768; }
 constexpr int kMidMax = 6;               // levels at most
 constexpr int kMidMaxSmem = 200 * 1024;
 struct MidLevel {
@@ -273,9 +275,11 @@ struct MidArgs {
   MidLevel lv[kMidMax];
   LevelDesc coarse;                      // the tail's first level
   int n, nu1, nu2;
+  int bottom;                            // sweeps of the last level where it is the coarsest (0: the tail follows)
+  int single;                            // the tail is one cell, relaxed once
   int coef_off, planes;                  // shared memory: the levels' plane coefficients, and their count
   int q_off, tail_off;                   // ... red residuals, tail arrays
-  const double* dense;                   // the first tail level's inverse (null: the tail's V-cycle)
+  const void* dense;                     // T[n * n]: the first tail level's inverse (null: the tail's V-cycle)
   TailArgs tail;
 };
 struct MidPlan {
@@ -284,6 +288,7 @@ struct MidPlan {
   int threads = 0;
   int smem = 0;
 };
+template <typename T>
 bool mid_prepare(const MidPlan& p, bool sc);   // false where the cluster cannot be launched
 
 // Direct FP64 form (V-cycle on phi itself): the fused fine-level residual +
@@ -352,7 +357,8 @@ struct LegPlan {
 LegPlan leg_plan(long long cells, int nx, int ny, int nz, bool wide);
 cudaError_t leg_prepare();
 void launch_leg_down(const LegArgs& a, cudaStream_t s);
-void launch_mid(const MGArgs<double>& g, const MidPlan& p, cudaStream_t s);
+template <typename T>
+void launch_mid(const MGArgs<T>& g, const MidPlan& p, cudaStream_t s);
 void launch_leg_up(const LegArgs& a, const UpdateArgs* upd, cudaStream_t s);
 dim3 check_grid(const LevelDesc& C);
 void launch_restrict_check(const MGArgs<double>& fa, double* rc, const LevelDesc& F,
