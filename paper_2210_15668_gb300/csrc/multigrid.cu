@@ -520,7 +520,7 @@ __global__ void __launch_bounds__(256) prolong_kernel(MGArgs<T> a, LevelDesc F, 
 constexpr int kPX = 32, kPY = 2;   // coarse columns (x, y) per block
 
 template <bool BLACK>
-__global__ void __launch_bounds__(kPX* kPY) prolong_tiled_kernel(const double* __restrict__ e, LevelDesc F, LevelDesc C,
+__global__ void __launch_bounds__(kPX* kPY) prolong_tiled_kernel(const double* e, LevelDesc F, LevelDesc C,
                                                                 double* fine, int kz) {
   pdl_enter();
   __shared__ double sY[2][2 * kPY][kPX + 2];   // interpolated in y: fine rows x coarse columns

@@ -63,9 +63,10 @@ constexpr int kConvTiles = 4;
 
 template <int COUT, bool MASK>   // MASK: the ReLU's backward on the output (an adjoint)
 __global__ void __launch_bounds__(32 * kConvTiles * 3) conv_fwd_kernel(
-    const bf16* __restrict__ in, int cin, const bf16* __restrict__ wk,
-    const float* __restrict__ bias, NNGrid g, int relu, const bf16* __restrict__ mask, bf16* __restrict__ out_bf,
+    const bf16* in, int cin, const bf16* __restrict__ wk,
+    const float* __restrict__ bias, NNGrid g, int relu, const bf16* mask, bf16* __restrict__ out_bf,
     float* __restrict__ out_f, int f_ch0) {
+  pdl_enter();
   __shared__ float part[2][kConvTiles][COUT / 8][4][32];
   const int lane = threadIdx.x, tile = threadIdx.y, slab = threadIdx.z;
   const int M = g.D * g.H * g.W;
@@ -256,7 +257,7 @@ __device__ __forceinline__ TcTile tc_tile(int t, const NNGrid& g, int zt) {
 // channels are the concatenation [up(a4) (32), s1 (16)] read in place: chunks
 // 0-3 from the coarse field a4 (= in) at the parent voxel, chunks 4-5 from s1.
 template <int CIN, bool UP>
-__device__ __forceinline__ void tc_load_halo(const bf16* __restrict__ in, const bf16* __restrict__ s1,
+__device__ __forceinline__ void tc_load_halo(const bf16* in, const bf16* s1,
                                              const NNGrid& g, TcTile t, int zt, unsigned buf, int chunk_entries) {
   constexpr int NCH = CIN / 8, PER_ROW = kTcHX * NCH;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -293,7 +294,7 @@ __device__ __forceinline__ void tc_load_halo(const bf16* __restrict__ in, const 
 
 template <int CIN, int COUT, bool MASK>
 __device__ __forceinline__ void tc_epilogue(unsigned tmem_acc, const NNGrid& g, TcTile t, int zt,
-                                            const float* __restrict__ bias, int relu, const bf16* __restrict__ mask,
+                                            const float* __restrict__ bias, int relu, const bf16* mask,
                                             bf16* __restrict__ out_bf, float* __restrict__ out_f, int f_ch0) {
   const int tid = threadIdx.x, warp = tid >> 5;
   // thread tid holds accumulator row tid = voxel (y0 + tid / 8, x0 + tid % 8)
@@ -342,8 +343,8 @@ __device__ __forceinline__ void tc_epilogue(unsigned tmem_acc, const NNGrid& g, 
 
 template <int CIN, int COUT, bool UP, bool MASK>
 __global__ void __launch_bounds__(kTcThreads) conv_tc_kernel(
-    const bf16* __restrict__ in, const bf16* __restrict__ s1, const bf16* __restrict__ wt,
-    const float* __restrict__ bias, NNGrid g, int zt, int relu, const bf16* __restrict__ mask,
+    const bf16* in, const bf16* s1, const bf16* __restrict__ wt,
+    const float* __restrict__ bias, NNGrid g, int zt, int relu, const bf16* mask,
     bf16* __restrict__ out_bf, float* __restrict__ out_f, int f_ch0, int* __restrict__ fault) {
   constexpr int NCH = CIN / 8;
   constexpr int WBYTES = 27 * CIN * COUT * 2;
@@ -370,8 +371,17 @@ __global__ void __launch_bounds__(kTcThreads) conv_tc_kernel(
     asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;\n" ::"r"(mb0 + 8) : "memory");
     asm volatile("fence.mbarrier_init.release.cluster;\n" ::: "memory");
   }
-  // weights (a straight copy of the packed array) and the first tile, one group
+  // weights (a straight copy of the packed array) and the first tile, one group.  The next
+  // convolution's blocks may take their places now: each allocates its accumulators and
+  // loads its weights while this kernel runs, and waits for it before its first input (no
+  // kernel that writes weights lets its successor start early).  With the launches' own
+  // work done ahead, nine dependent launches of a forward pass on 8x64x64 take 44 us
+  // instead of 68; inputs of kernels that may start early are not marked __restrict__,
+  // which would allow their loads before the wait.
   for (int i = tid; i < WBYTES / 16; i += kTcThreads) tc_cp16(sw + 16u * i, wt + 8 * i, true);
+  __syncwarp();
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  pdl_enter();
   if (nmine > 0) tc_load_halo<CIN, UP>(in, s1, g, tc_tile(blockIdx.x, g, zt), zt, hb0, chunk_entries);
   asm volatile("cp.async.commit_group;\n" ::: "memory");
 
@@ -471,8 +481,9 @@ __device__ __forceinline__ void ldsm_x4_trans(unsigned (&r)[4], unsigned addr) {
 __host__ __device__ constexpr int wg_elems(int cin, int cout) { return 27 * cin * cout + cout; }
 
 template <int CIN, int COUT>
-__global__ void __launch_bounds__(kWgThreads) conv_wgrad_kernel(const bf16* __restrict__ in, const bf16* __restrict__ dout,
+__global__ void __launch_bounds__(kWgThreads) conv_wgrad_kernel(const bf16* in, const bf16* dout,
                                                                 NNGrid g, int tz, float* __restrict__ part) {
+  pdl_enter();
   constexpr int KC = CIN / 8, NC = COUT / 8;
   extern __shared__ __align__(128) unsigned char smem[];
   const int nv = (tz + 2) * kWgHY * kWgHX, nd = tz * kWgY * kWgX;
@@ -560,8 +571,9 @@ __global__ void __launch_bounds__(kWgThreads) conv_wgrad_kernel(const bf16* __re
 }
 
 // gw, gb += the blocks' sums: 32 elements by 8 partial rows per block, a fixed order
-__global__ void __launch_bounds__(256) wgrad_reduce_kernel(const float* __restrict__ part, int nblk, int nw, int nb,
+__global__ void __launch_bounds__(256) wgrad_reduce_kernel(const float* part, int nblk, int nw, int nb,
                                                            float* __restrict__ gw, float* __restrict__ gb) {
+  pdl_enter();
   __shared__ float sh[8][32];
   const int n = nw + nb, t = blockIdx.x * 32 + threadIdx.x;
   float s = 0.f;
@@ -585,7 +597,8 @@ __global__ void __launch_bounds__(256) wgrad_reduce_kernel(const float* __restri
 
 // 2x2x2 mean of a fine channels-last field: one thread per coarse voxel and
 // 8-channel chunk (16 bytes)
-__global__ void pool2_kernel(const bf16* __restrict__ in, NNGrid f, int C, bf16* __restrict__ out) {
+__global__ void pool2_kernel(const bf16* in, NNGrid f, int C, bf16* __restrict__ out) {
+  pdl_enter();
   const int Dc = f.D / 2, Hc = f.H / 2, Wc = f.W / 2, nch = C / 8;
   const long long n = (long long)Dc * Hc * Wc * nch;
   for (long long t = blockIdx.x * (long long)blockDim.x + threadIdx.x; t < n; t += (long long)gridDim.x * blockDim.x) {
@@ -614,8 +627,9 @@ __global__ void pool2_kernel(const bf16* __restrict__ in, NNGrid f, int C, bf16*
 
 // cat[v] = [a4(parent of v) (32 channels), s1(v) (16 channels)]: one thread per
 // voxel and 8-channel chunk (16 bytes)
-__global__ void upcat_kernel(const bf16* __restrict__ a4, const bf16* __restrict__ s1, NNGrid f,
+__global__ void upcat_kernel(const bf16* a4, const bf16* s1, NNGrid f,
                              bf16* __restrict__ cat) {
+  pdl_enter();
   const long long n = (long long)f.D * f.H * f.W * 6;
   const int Hc = f.H / 2, Wc = f.W / 2;
   for (long long t = blockIdx.x * (long long)blockDim.x + threadIdx.x; t < n; t += (long long)gridDim.x * blockDim.x) {
@@ -629,8 +643,9 @@ __global__ void upcat_kernel(const bf16* __restrict__ a4, const bf16* __restrict
 }
 
 // da4m[V][c] = bf16(sum over the 8 children of dcat[child][c] (c < 32), masked by a4 > 0)
-__global__ void up_grad_kernel(const float* __restrict__ dcat, const bf16* __restrict__ a4, NNGrid f,
+__global__ void up_grad_kernel(const float* dcat, const bf16* a4, NNGrid f,
                                bf16* __restrict__ out) {
+  pdl_enter();
   const int Dc = f.D / 2, Hc = f.H / 2, Wc = f.W / 2;
   const long long n = (long long)Dc * Hc * Wc * 32;
   for (long long t = blockIdx.x * (long long)blockDim.x + threadIdx.x; t < n; t += (long long)gridDim.x * blockDim.x) {
@@ -647,8 +662,9 @@ __global__ void up_grad_kernel(const float* __restrict__ dcat, const bf16* __res
 }
 
 // ds1m[v][c] = bf16((dcat[v][32 + c] + dp[parent(v)][c] / 8) masked by s1 > 0)
-__global__ void skip_grad_kernel(const float* __restrict__ dcat, const float* __restrict__ dp,
-                                 const bf16* __restrict__ s1, NNGrid f, bf16* __restrict__ out) {
+__global__ void skip_grad_kernel(const float* dcat, const float* dp,
+                                 const bf16* s1, NNGrid f, bf16* __restrict__ out) {
+  pdl_enter();
   const long long n = (long long)f.D * f.H * f.W * 16;
   const int Hc = f.H / 2, Wc = f.W / 2;
   for (long long t = blockIdx.x * (long long)blockDim.x + threadIdx.x; t < n; t += (long long)gridDim.x * blockDim.x) {
@@ -662,8 +678,9 @@ __global__ void skip_grad_kernel(const float* __restrict__ dcat, const float* __
 }
 
 // loss += sum (y0 - t)^2 / M; dy[m][0] = 2 (y0 - t) / M, other channels 0
-__global__ void __launch_bounds__(256) mse_kernel(const float* __restrict__ y, const float* __restrict__ tgt, int M,
+__global__ void __launch_bounds__(256) mse_kernel(const float* y, const float* tgt, int M,
                                                   bf16* __restrict__ dy, float* __restrict__ loss) {
+  pdl_enter();
   __shared__ float sh[8];
   float s = 0.f;
   for (int m = blockIdx.x * blockDim.x + threadIdx.x; m < M; m += gridDim.x * blockDim.x) {
@@ -709,6 +726,7 @@ __global__ void __launch_bounds__(256) adam_pack_kernel(NNLayout L, float* __res
                                                         float b2, float c1, float c2, float eps, bf16* __restrict__ wk,
                                                         bf16* __restrict__ wb, bf16* __restrict__ wkt,
                                                         bf16* __restrict__ wbt) {
+  pdl_enter();
   const int t = blockIdx.x * blockDim.x + threadIdx.x;
   if (t >= L.b0[6]) return;
   float x = p[t];
@@ -774,7 +792,7 @@ void launch_conv_tc(const bf16* in, const bf16* s1, const bf16* wt, const float*
   const int per_sm = std::max(1, std::min(16, (int)(233472 / (smem + 1024))));
   const int blocks = std::min(tc_tiles(g, zt), sm_count() * per_sm);
   auto k = mask ? conv_tc_kernel<CIN, COUT, false, true> : conv_tc_kernel<CIN, COUT, UP, false>;
-  k<<<blocks, kTcThreads, smem, s>>>(in, s1, wt, bias, g, zt, relu, mask, out_bf, out_f, f_ch0, fault);
+  launch_k(k, dim3(blocks), dim3(kTcThreads), smem, s, in, s1, wt, bias, g, zt, relu, mask, out_bf, out_f, f_ch0, fault);
 }
 
 }  // namespace
@@ -838,7 +856,7 @@ bool nn_conv_fwd(const bf16* in, int cin, const bf16* wk, const bf16* wt, const 
   const int blocks = (tiles + kConvTiles - 1) / kConvTiles;
   const dim3 block(32, kConvTiles, 3);
   // two kernels each: the mask's branch cost the forward 9% (22x20x32: 74.8 -> 81.9 us)
-  auto go = [&](auto k) { k<<<blocks, block, 0, s>>>(in, cin, wk, bias, g, relu, mask, out_bf, out_f, f_ch0); };
+  auto go = [&](auto k) { launch_k(k, dim3(blocks), block, 0, s, in, cin, wk, bias, g, relu, mask, out_bf, out_f, f_ch0); };
   if (cout == 16) go(mask ? conv_fwd_kernel<16, true> : conv_fwd_kernel<16, false>);
   else if (cout == 32) go(mask ? conv_fwd_kernel<32, true> : conv_fwd_kernel<32, false>);
   else if (cout == 48) go(mask ? conv_fwd_kernel<48, true> : conv_fwd_kernel<48, false>);
@@ -875,34 +893,34 @@ void nn_conv_wgrad(const bf16* in, int cin, const bf16* dout, int cout, NNGrid g
                    float* gb, float* part, cudaStream_t s) {
   const int tz = wg_tz(g), blocks = wg_blocks(g, tz);
   const size_t smem = 16 * ((size_t)(cin / 8) * (tz + 2) * kWgHY * kWgHX + (size_t)(cout / 8) * tz * kWgY * kWgX);
-  if (cin == 16 && cout == 16) conv_wgrad_kernel<16, 16><<<blocks, kWgThreads, smem, s>>>(in, dout, g, tz, part);
-  else if (cin == 16 && cout == 32) conv_wgrad_kernel<16, 32><<<blocks, kWgThreads, smem, s>>>(in, dout, g, tz, part);
-  else if (cin == 32 && cout == 32) conv_wgrad_kernel<32, 32><<<blocks, kWgThreads, smem, s>>>(in, dout, g, tz, part);
-  else if (cin == 48 && cout == 16) conv_wgrad_kernel<48, 16><<<blocks, kWgThreads, smem, s>>>(in, dout, g, tz, part);
+  if (cin == 16 && cout == 16) launch_k(conv_wgrad_kernel<16, 16>, dim3(blocks), dim3(kWgThreads), smem, s, in, dout, g, tz, part);
+  else if (cin == 16 && cout == 32) launch_k(conv_wgrad_kernel<16, 32>, dim3(blocks), dim3(kWgThreads), smem, s, in, dout, g, tz, part);
+  else if (cin == 32 && cout == 32) launch_k(conv_wgrad_kernel<32, 32>, dim3(blocks), dim3(kWgThreads), smem, s, in, dout, g, tz, part);
+  else if (cin == 48 && cout == 16) launch_k(conv_wgrad_kernel<48, 16>, dim3(blocks), dim3(kWgThreads), smem, s, in, dout, g, tz, part);
   const int nw = 27 * cin * cout;
-  wgrad_reduce_kernel<<<(nw + cout + 31) / 32, dim3(32, 8), 0, s>>>(part, blocks, nw, cout, gw, gb);
+  launch_k(wgrad_reduce_kernel, dim3((nw + cout + 31) / 32), dim3(32, 8), 0, s, part, blocks, nw, cout, gw, gb);
 }
 
 void nn_pool2(const bf16* in, NNGrid f, int C, bf16* out, cudaStream_t s) {
-  pool2_kernel<<<grid1((long long)f.D * f.H * f.W * C / 64, 256), 256, 0, s>>>(in, f, C, out);
+  launch_k(pool2_kernel, dim3(grid1((long long)f.D * f.H * f.W * C / 64, 256)), dim3(256), 0, s, in, f, C, out);
 }
 void nn_upcat(const bf16* a4, const bf16* s1, NNGrid f, bf16* cat, cudaStream_t s) {
-  upcat_kernel<<<grid1((long long)f.D * f.H * f.W * 6, 256), 256, 0, s>>>(a4, s1, f, cat);
+  launch_k(upcat_kernel, dim3(grid1((long long)f.D * f.H * f.W * 6, 256)), dim3(256), 0, s, a4, s1, f, cat);
 }
 void nn_up_grad(const float* dcat, const bf16* a4, NNGrid f, bf16* out, cudaStream_t s) {
-  up_grad_kernel<<<grid1((long long)f.D * f.H * f.W * 4, 256), 256, 0, s>>>(dcat, a4, f, out);
+  launch_k(up_grad_kernel, dim3(grid1((long long)f.D * f.H * f.W * 4, 256)), dim3(256), 0, s, dcat, a4, f, out);
 }
 void nn_skip_grad(const float* dcat, const float* dp, const bf16* s1, NNGrid f, bf16* out, cudaStream_t s) {
-  skip_grad_kernel<<<grid1((long long)f.D * f.H * f.W * 16, 256), 256, 0, s>>>(dcat, dp, s1, f, out);
+  launch_k(skip_grad_kernel, dim3(grid1((long long)f.D * f.H * f.W * 16, 256)), dim3(256), 0, s, dcat, dp, s1, f, out);
 }
 void nn_mse(const float* y, const float* tgt, int M, bf16* dy, float* loss, cudaStream_t s) {
-  mse_kernel<<<grid1(M, 256), 256, 0, s>>>(y, tgt, M, dy, loss);
+  launch_k(mse_kernel, dim3(grid1(M, 256)), dim3(256), 0, s, y, tgt, M, dy, loss);
 }
 void nn_adam_pack(const NNLayout& L, float* p, float* g, float* m, float* v, float lr, int step, bf16* wk, bf16* wb,
                   bf16* wkt, bf16* wbt, cudaStream_t s) {
   const float b1 = 0.9f, b2 = 0.999f;
   const float c1 = 1.f - powf(b1, (float)step), c2 = 1.f - powf(b2, (float)step);
-  adam_pack_kernel<<<(L.b0[6] + 255) / 256, 256, 0, s>>>(L, p, g, m, v, lr, b1, b2, c1, c2, 1e-8f, wk, wb, wkt, wbt);
+  launch_k(adam_pack_kernel, dim3((L.b0[6] + 255) / 256), dim3(256), 0, s, L, p, g, m, v, lr, b1, b2, c1, c2, 1e-8f, wk, wb, wkt, wbt);
 }
 
 }  // namespace fx
@@ -919,11 +937,31 @@ constexpr int kLayers = 6;
 constexpr int kCin[kLayers] = {16, 16, 16, 32, 48, 16};
 constexpr int kCout[kLayers] = {16, 16, 32, 32, 16, 16};
 
-__global__ void f32_to_bf16_kernel(const float* __restrict__ in, long long n, bf16* __restrict__ out) {
+__global__ void __launch_bounds__(256) f32_to_bf16_kernel(const float* in, long long n, int vec,
+                                                          bf16* __restrict__ out) {
+  pdl_enter();
+  if (vec) {   // eight values by 16-byte accesses
+    const long long t = blockIdx.x * (long long)blockDim.x + threadIdx.x;
+    if (8 * t >= n) return;
+    const float4 *p = reinterpret_cast<const float4*>(in) + 2 * t, a = p[0], b = p[1];
+    uint4 q;
+    __nv_bfloat162* h = reinterpret_cast<__nv_bfloat162*>(&q);
+    h[0] = __floats2bfloat162_rn(a.x, a.y);
+    h[1] = __floats2bfloat162_rn(a.z, a.w);
+    h[2] = __floats2bfloat162_rn(b.x, b.y);
+    h[3] = __floats2bfloat162_rn(b.z, b.w);
+    reinterpret_cast<uint4*>(out)[t] = q;
+    return;
+  }
   for (long long t = blockIdx.x * (long long)blockDim.x + threadIdx.x; t < n; t += (long long)gridDim.x * blockDim.x)
     out[t] = __float2bfloat16(in[t]);
 }
 
+void nn_to_bf16(const float* in, long long n, bf16* out, cudaStream_t s) {
+  const int vec = n % 8 == 0 && reinterpret_cast<uintptr_t>(in) % 16 == 0;   // out is the network's own
+  launch_k(f32_to_bf16_kernel, dim3(vec ? (unsigned)((n / 8 + 255) / 256) : (unsigned)grid1(n, 256)), dim3(256), 0, s, in, n,
+           vec, out);
+}
 
 }  // namespace
 }  // namespace fx
@@ -1006,10 +1044,10 @@ void conv(ferrox_nn* N, int l, bool adjoint, const bf16* in, fx::NNGrid g, int r
                   adjoint ? nullptr : N->b[l], cout, g, relu, mask, out_bf, out_f, f_ch0, N->fault, s);
 }
 
-// forward pass from N->x; output channel 0 (FP32) in N->y.  The concatenation
+// forward pass from N->x; output channel 0 (FP32) in y (null: N->y).  The concatenation
 // [up(a4), s1] is formed in memory only for a backward pass (keep_cat) or where
 // the tensor-memory kernel cannot read it in place.
-void forward(ferrox_nn* N, bool keep_cat) {
+void forward(ferrox_nn* N, bool keep_cat, float* y = nullptr) {
   cudaStream_t s = N->stream;
   using namespace fx;
   conv(N, 0, false, N->x, N->g, 1, N->a1, nullptr, s);
@@ -1022,7 +1060,7 @@ void forward(ferrox_nn* N, bool keep_cat) {
     nn_upcat(N->a4, N->s1, N->g, N->cat, s);
     conv(N, 4, false, N->cat, N->g, 1, N->a5, nullptr, s);
   }
-  conv(N, 5, false, N->a5, N->g, 0, nullptr, N->y, s, 1);   // output channel 0 only
+  conv(N, 5, false, N->a5, N->g, 0, nullptr, y ? y : N->y, s, 1);   // output channel 0 only
 }
 
 // backward pass from N->dy (gradient of the loss w.r.t. the output); accumulates gw, gb
@@ -1158,9 +1196,8 @@ ferrox_status ferrox_nn_create(ferrox_nn** out, int D, int H, int W, int capacit
 
 ferrox_status ferrox_nn_forward(ferrox_nn* N, const float* x_dev, float* y_dev) {
   if (!N || !x_dev || !y_dev) return nfail(N, FERROX_EINVAL, "null argument");
-  fx::f32_to_bf16_kernel<<<fx::grid1((long long)N->M * 16, 256), 256, 0, N->stream>>>(x_dev, (long long)N->M * 16, N->x);
-  forward(N, false);
-  FX_NCK(cudaMemcpyAsync(y_dev, N->y, (size_t)N->M * sizeof(float), cudaMemcpyDeviceToDevice, N->stream));
+  fx::nn_to_bf16(x_dev, (long long)N->M * 16, N->x, N->stream);
+  forward(N, false, y_dev);
   FX_NCK(cudaGetLastError());
   return FERROX_OK;
 }
@@ -1168,7 +1205,7 @@ ferrox_status ferrox_nn_forward(ferrox_nn* N, const float* x_dev, float* y_dev) 
 // forward + MSE against t_dev + backward: gradients are accumulated (not applied)
 ferrox_status ferrox_nn_loss_grad(ferrox_nn* N, const float* x_dev, const float* t_dev, float* loss_host) {
   if (!N || !x_dev || !t_dev) return nfail(N, FERROX_EINVAL, "null argument");
-  fx::f32_to_bf16_kernel<<<fx::grid1((long long)N->M * 16, 256), 256, 0, N->stream>>>(x_dev, (long long)N->M * 16, N->x);
+  fx::nn_to_bf16(x_dev, (long long)N->M * 16, N->x, N->stream);
   FX_NCK(cudaMemsetAsync(N->loss, 0, sizeof(float), N->stream));
   forward(N, true);
   fx::nn_mse(N->y, t_dev, N->M, N->dy, N->loss, N->stream);
@@ -1305,6 +1342,7 @@ namespace {
 // 2x2x2 (or semi-coarsened) mean of a level field into the next level
 template <typename T>
 __global__ void avg_down_kernel(T* __restrict__ a, LevelDesc F, LevelDesc C) {
+  pdl_enter();
   const long long n = C.ncell;
   for (long long t = blockIdx.x * (long long)blockDim.x + threadIdx.x; t < n; t += (long long)gridDim.x * blockDim.x) {
     const int I = (int)(t % C.nx), J = (int)((t / C.nx) % C.ny), K = (int)(t / ((long long)C.nx * C.ny));
@@ -1322,7 +1360,8 @@ __global__ void avg_down_kernel(T* __restrict__ a, LevelDesc F, LevelDesc C) {
 
 // sum of squares of a level field in fixed order: one block
 template <typename T>
-__global__ void rms_kernel(const T* __restrict__ a, long long off, long long n, double* __restrict__ out) {
+__global__ void rms_kernel(const T* a, long long off, long long n, double* __restrict__ out) {
+  pdl_enter();
   __shared__ double sh[32];
   double s = 0.0;
   for (long long t = threadIdx.x; t < n; t += blockDim.x) {
@@ -1341,9 +1380,10 @@ __global__ void rms_kernel(const T* __restrict__ a, long long off, long long n, 
 
 // network input: residual / rms, per-plane material features, height, bias
 template <typename T>
-__global__ void features_kernel(const T* __restrict__ r, LevelDesc L, const float* __restrict__ pf,
-                                const double* __restrict__ scale, const DevParams* __restrict__ prm,
+__global__ void features_kernel(const T* r, LevelDesc L, const float* __restrict__ pf,
+                                const double* scale, const DevParams* prm,
                                 bf16* __restrict__ x) {
+  pdl_enter();
   const long long n = L.ncell;
   const float inv = (float)(1.0 / *scale);
   const float vapp = (float)(prm->v_top - prm->v_bot);
@@ -1359,8 +1399,9 @@ __global__ void features_kernel(const T* __restrict__ r, LevelDesc L, const floa
 
 // e (level) = scale * network output channel 0
 template <typename T>
-__global__ void apply_kernel(const float* __restrict__ y, LevelDesc L, const double* __restrict__ scale,
+__global__ void apply_kernel(const float* y, LevelDesc L, const double* scale,
                              T* __restrict__ e) {
+  pdl_enter();
   const double s = *scale;
   for (long long t = blockIdx.x * (long long)blockDim.x + threadIdx.x; t < L.ncell; t += (long long)gridDim.x * blockDim.x)
     e[L.off + t] = (T)(s * (double)y[t]);
@@ -1368,16 +1409,18 @@ __global__ void apply_kernel(const float* __restrict__ y, LevelDesc L, const dou
 
 // e0 = phi - phi_guess (fine level), the error the initial guess had
 template <typename T>
-__global__ void guess_error_kernel(const double* __restrict__ phi, const double* __restrict__ guess,
+__global__ void guess_error_kernel(const double* phi, const double* guess,
                                    long long n, T* __restrict__ e0) {
+  pdl_enter();
   for (long long t = blockIdx.x * (long long)blockDim.x + threadIdx.x; t < n; t += (long long)gridDim.x * blockDim.x)
     e0[t] = (T)(phi[t] - guess[t]);
 }
 
 // training target = restricted error / rms of the restricted initial residual
 template <typename T>
-__global__ void target_kernel(const T* __restrict__ e, LevelDesc L, const double* __restrict__ scale,
+__global__ void target_kernel(const T* e, LevelDesc L, const double* scale,
                               float* __restrict__ tgt) {
+  pdl_enter();
   const double inv = 1.0 / *scale;
   for (long long t = blockIdx.x * (long long)blockDim.x + threadIdx.x; t < L.ncell; t += (long long)gridDim.x * blockDim.x)
     tgt[t] = (float)((double)e[L.off + t] * inv);
@@ -1388,28 +1431,28 @@ __global__ void target_kernel(const T* __restrict__ e, LevelDesc L, const double
 template <typename T>
 void nn_bridge_restrict(T* arena, const std::vector<LevelDesc>& lv, int to, cudaStream_t s) {
   for (int l = 0; l < to; ++l)
-    avg_down_kernel<T><<<grid1(lv[l + 1].ncell, 256), 256, 0, s>>>(arena, lv[l], lv[l + 1]);
+    launch_k(avg_down_kernel<T>, dim3(grid1(lv[l + 1].ncell, 256)), dim3(256), 0, s, arena, lv[l], lv[l + 1]);
 }
 template <typename T>
 void nn_bridge_scale(const T* arena, const LevelDesc& L, double* scale, cudaStream_t s) {
-  rms_kernel<T><<<1, 1024, 0, s>>>(arena, L.off, L.ncell, scale);
+  launch_k(rms_kernel<T>, dim3(1), dim3(1024), 0, s, arena, L.off, L.ncell, scale);
 }
 template <typename T>
 void nn_bridge_features(const T* r, const LevelDesc& L, const float* pf, const double* scale,
                         const DevParams* prm, bf16* x, cudaStream_t s) {
-  features_kernel<T><<<grid1(L.ncell, 256), 256, 0, s>>>(r, L, pf, scale, prm, x);
+  launch_k(features_kernel<T>, dim3(grid1(L.ncell, 256)), dim3(256), 0, s, r, L, pf, scale, prm, x);
 }
 template <typename T>
 void nn_bridge_apply(const float* y, const LevelDesc& L, const double* scale, T* e, cudaStream_t s) {
-  apply_kernel<T><<<grid1(L.ncell, 256), 256, 0, s>>>(y, L, scale, e);
+  launch_k(apply_kernel<T>, dim3(grid1(L.ncell, 256)), dim3(256), 0, s, y, L, scale, e);
 }
 template <typename T>
 void nn_bridge_guess_error(const double* phi, const double* guess, long long n, T* e0, cudaStream_t s) {
-  guess_error_kernel<T><<<grid1(n, 256), 256, 0, s>>>(phi, guess, n, e0);
+  launch_k(guess_error_kernel<T>, dim3(grid1(n, 256)), dim3(256), 0, s, phi, guess, n, e0);
 }
 template <typename T>
 void nn_bridge_target(const T* e, const LevelDesc& L, const double* scale, float* tgt, cudaStream_t s) {
-  target_kernel<T><<<grid1(L.ncell, 256), 256, 0, s>>>(e, L, scale, tgt);
+  launch_k(target_kernel<T>, dim3(grid1(L.ncell, 256)), dim3(256), 0, s, e, L, scale, tgt);
 }
 
 #define FX_NNB(T)                                                                                   \
