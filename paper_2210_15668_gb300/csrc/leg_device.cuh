@@ -521,7 +521,7 @@ struct LegUp {
       const float2 va = P ? make_float2(r.x, b.x) : make_float2(b.x, r.x);
       const float2 vb = P ? make_float2(b.y, r.y) : make_float2(r.y, b.y);
       if (PHI) {
-        auto upd = [&](double p, float e) { return u.zero ? 0.0 : p + (double)fminf(fmaxf(e, -u.clampf), u.clampf); };
+        auto upd = [&](double p, float e) { return u.zero ? 0.0 : p + f64_of_float(fminf(fmaxf(e, -u.clampf), u.clampf)); };
         double* f = u.phi + (size_t)po * plane + q.base;
         store2(f, make_double2(upd(fa.x, va.x), upd(fa.y, va.y)), a.phi_vec);
         store2(f + a.nx, make_double2(upd(fb.x, vb.x), upd(fb.y, vb.y)), a.phi_vec);

@@ -55,16 +55,17 @@ struct Upd {
 };
 
 // phi += e, e clamped to [-clamp, clamp].  An FP32 correction is clamped in FP32
-// against the limit rounded to float and converted once: one FP64-pipe
-// conversion and one FP64 add per cell instead of a conversion, two FP64
-// min/max and the add (GB300 runs FP64 at 1/58 of the FP32 rate).  With an
-// infinite limit (no carriers) the result is the same bit for bit.
+// against the limit rounded to float and widened with integer operations: one FP64 add
+// per cell instead of two FP64 min/max, a conversion and the add (GB300 runs FP64, and
+// conversions to it, at 1/58 of the FP32 rate; the up leg that updates phi on 256x256x32
+// 28.4 -> 26.1 us, the update alone 10.8 -> 8.7).  With an infinite limit (no carriers)
+// the result is the same bit for bit (corrections below 2^-126 count as zero).
 template <typename T>
 __device__ __forceinline__ void apply_update(const Upd& u, int idx, T e) {
   if (u.zero) {
     u.phi[idx] = 0.0;
   } else if constexpr (sizeof(T) == sizeof(float)) {
-    u.phi[idx] += (double)fminf(fmaxf(e, -u.clampf), u.clampf);
+    u.phi[idx] += f64_of_float(fminf(fmaxf(e, -u.clampf), u.clampf));
   } else {
     u.phi[idx] += fmin(fmax(e, -u.clamp), u.clamp);
   }
