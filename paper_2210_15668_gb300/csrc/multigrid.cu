@@ -338,6 +338,57 @@ __device__ __forceinline__ double sum_partials(const double* P, int nblk, int ti
   return s;
 }
 
+// Residuals of the red children of coarse cell (I, J, K) of a level halved in all three
+// directions (the black ones vanish after a pre-smoothing, see black_residual_zero), with
+// the 2 x 2 x 2 children in registers: 20 loads in flight at once and 33 FP64 operations,
+// where a loop over the children serialises four loads-to-sum chains.
+struct RedChildren {
+  double res[2][2];        // [dk][dj]: the red cell of rows 2 J + dj, planes 2 K + dk
+  int base, plane;         // cell index of the first child, cells of a plane
+  // s: Newton shifts (null: none)
+  __device__ __forceinline__ void load(const double* e, const double* r, const double* s, const PlaneCoef<double>* coef,
+                                       const LevelDesc& F, const LevelDesc& C, int I, int J, int K) {
+    const int nx = F.nx;
+    plane = F.nx * F.ny;
+    // red cells at x = 2 I + p, p = (dj + dk) & 1
+    base = (2 * K * F.ny + 2 * J) * nx + 2 * I;
+    const int xl = I == 0 ? nx - 1 : -1, xr = I + 1 == C.nx ? 2 - nx : 2;
+    const int ym = J == 0 ? (F.ny - 1) * nx : -nx, yp = J + 1 == C.ny ? (2 - F.ny) * nx : 2 * nx;
+    double g[2][2][2], out_x[2][2], out_y[2][2], out_z[2][2], b[2][2], sh[2][2];
+#pragma unroll
+    for (int dk = 0; dk < 2; ++dk)
+#pragma unroll
+      for (int dj = 0; dj < 2; ++dj) {
+        const int p = (dj + dk) & 1, row = base + dk * plane + dj * nx;
+        g[dk][dj][0] = e[row];
+        g[dk][dj][1] = e[row + 1];
+        b[dk][dj] = r[row + p];
+        out_x[dk][dj] = e[row + (p ? xr : xl)];
+        out_y[dk][dj] = e[base + dk * plane + p + (dj ? yp : ym)];
+        const bool in = dk ? K + 1 < C.nz : K > 0;
+        out_z[dk][dj] = in ? e[row + p + (dk ? plane : -plane)] : 0.0;
+        sh[dk][dj] = s ? s[row + p] : 0.0;
+      }
+#pragma unroll
+    for (int dk = 0; dk < 2; ++dk) {
+      const PlaneCoef<double> c = ldg_struct(coef + F.coef_off + 2 * K + dk);
+#pragma unroll
+      for (int dj = 0; dj < 2; ++dj) {
+        const int p = (dj + dk) & 1;
+        const double x = out_x[dk][dj] + g[dk][dj][1 - p];
+        const double y = out_y[dk][dj] + g[dk][1 - dj][p];
+        const double z = g[1 - dk][dj][p], o = out_z[dk][dj];
+        double acc = fma(c.cx, x, b[dk][dj]);
+        acc = fma(c.cy, y, acc);
+        acc = fma(c.czlo, dk ? z : o, acc);
+        acc = fma(c.czhi, dk ? o : z, acc);
+        const double d = s && c.has_s ? c.diag + sh[dk][dj] : c.diag;
+        res[dk][dj] = fma(-d, g[dk][dj][p], acc);
+      }
+    }
+  }
+};
+
 // Direct FP64 form: the fine level's residual b - A phi after the pre-smoothing,
 // restricted to the first coarse level (8-child mean; the black residuals vanish, see
 // black_residual_zero) and its squared norm summed on the way; the last block sums the
@@ -349,9 +400,7 @@ __device__ __forceinline__ double sum_partials(const double* P, int nblk, int ti
 // (the FP64 -> FP32 conversion instruction runs on the FP64 pipe): the norms only scale
 // the stopping test, where a relative error of ~1e-6 in ||r|| is immaterial.
 //
-// A thread holds the 2 x 2 x 2 children of its coarse cell: 24 loads in flight at once and
-// 33 FP64 operations (a loop over the children serialised four loads-to-sum chains).
-// 256x256x32: 34.8 -> 28.6 us, 64x64x16: 16.3 -> 12.3 us (launches timed one by one, which
+// With the children in registers (RedChildren) 256x256x32: 34.8 -> 28.6 us, 64x64x16: 16.3 -> 12.3 us (launches timed one by one, which
 // adds about 3.5 us; the reduction's last block about as much).
 __global__ void __launch_bounds__(256) restrict_check_kernel(MGArgs<double> fa, double* rc, LevelDesc F,
                                                              LevelDesc C, CheckArgs ck) {
@@ -361,52 +410,24 @@ __global__ void __launch_bounds__(256) restrict_check_kernel(MGArgs<double> fa, 
   const int K = blockIdx.z;
   float rr = 0.0f, bb = 0.0f;
   if (I < C.nx && J < C.ny) {
-    const double *e = fa.e + F.off, *r = fa.r + F.off;
-    const int nx = F.nx, plane = F.nx * F.ny;
-    // rows 2 J and 2 J + 1 of planes 2 K and 2 K + 1; red cells at x = 2 I + p, p = (dj + dk) & 1
-    const int base = (2 * K * F.ny + 2 * J) * nx + 2 * I;
-    const int xl = I == 0 ? nx - 1 : -1, xr = I + 1 == C.nx ? 2 - nx : 2;
-    const int ym = J == 0 ? (F.ny - 1) * nx : -nx, yp = J + 1 == C.ny ? (2 - F.ny) * nx : 2 * nx;
-    double g[2][2][2], out_x[2][2], out_y[2][2], out_z[2][2], b[2][2], bk[2][2];
+    const double* r = fa.r + F.off;
+    RedChildren red;
+    red.load(fa.e + F.off, r, nullptr, fa.coef, F, C, I, J, K);
+    double sum = 0.0;
 #pragma unroll
     for (int dk = 0; dk < 2; ++dk)
 #pragma unroll
       for (int dj = 0; dj < 2; ++dj) {
-        const int p = (dj + dk) & 1, row = base + dk * plane + dj * nx;
-        g[dk][dj][0] = e[row];
-        g[dk][dj][1] = e[row + 1];
-        b[dk][dj] = r[row + p];
-        bk[dk][dj] = ck.first ? r[row + 1 - p] : 0.0;
-        out_x[dk][dj] = e[row + (p ? xr : xl)];
-        out_y[dk][dj] = e[base + dk * plane + p + (dj ? yp : ym)];
-        const bool in = dk ? K + 1 < C.nz : K > 0;
-        out_z[dk][dj] = in ? e[row + p + (dk ? plane : -plane)] : 0.0;
-      }
-    double sum = 0.0;
-#pragma unroll
-    for (int dk = 0; dk < 2; ++dk) {
-      const PlaneCoef<double> c = ldg_struct(fa.coef + F.coef_off + 2 * K + dk);
-#pragma unroll
-      for (int dj = 0; dj < 2; ++dj) {
-        const int p = (dj + dk) & 1;
-        const double x = out_x[dk][dj] + g[dk][dj][1 - p];
-        const double y = out_y[dk][dj] + g[dk][1 - dj][p];
-        const double z = g[1 - dk][dj][p], o = out_z[dk][dj];
-        double acc = fma(c.cx, x, b[dk][dj]);
-        acc = fma(c.cy, y, acc);
-        acc = fma(c.czlo, dk ? z : o, acc);
-        acc = fma(c.czhi, dk ? o : z, acc);
-        const double q = fma(-c.diag, g[dk][dj][p], acc);
-        sum += q;
-        const float qf = df_from_double(q).h;
+        sum += red.res[dk][dj];
+        const float qf = df_from_double(red.res[dk][dj]).h;
         rr = fmaf(qf, qf, rr);
-        if (ck.first) {   // in the order of the cells
-          const float b0 = df_from_double(p ? bk[dk][dj] : b[dk][dj]).h, b1 = df_from_double(p ? b[dk][dj] : bk[dk][dj]).h;
+        if (ck.first) {
+          const int row = red.base + dk * red.plane + dj * F.nx;
+          const float b0 = df_from_double(r[row]).h, b1 = df_from_double(r[row + 1]).h;
           bb = fmaf(b0, b0, bb);
           bb = fmaf(b1, b1, bb);
         }
       }
-    }
     rc[lidx(C, I, J, K)] = sum * 0.125;
   }
   block_sum2f(rr, bb);
@@ -435,6 +456,31 @@ __global__ void __launch_bounds__(256) restrict_check_kernel(MGArgs<double> fa, 
     if (ck.first) ck.stats->launches += ck.first_launches - 1;   // decide counted one
     if (ck.set_cond) cudaGraphSetConditional((cudaGraphConditionalHandle)ck.cond_handle, cond);
   }
+}
+
+// Restriction of an FP64 level halved in all three directions, one thread per coarse cell
+// (RedChildren), the residuals and shifts added in the order of restrict4_kernel: the
+// restrictions of 64^3 and 32^3 with a shift 17 -> 10 us together, of 128x128x16 and
+// 64x64x8 without one 15 -> 10.6.
+template <bool SC>
+__global__ void __launch_bounds__(128) restrict_red_kernel(MGArgs<double> a, LevelDesc F, LevelDesc C) {
+  pdl_enter();
+  const int I = blockIdx.x * blockDim.x + threadIdx.x;
+  const int J = blockIdx.y * blockDim.y + threadIdx.y, K = blockIdx.z;
+  if (I >= C.nx || J >= C.ny) return;
+  double u[2][2][2];
+  if (SC) {
+    const int plane = F.nx * F.ny, base = (2 * K * F.ny + 2 * J) * F.nx + 2 * I;
+#pragma unroll
+    for (int q = 0; q < 8; ++q) u[q >> 2][(q >> 1) & 1][q & 1] = a.s[F.off + base + (q >> 2) * plane + ((q >> 1) & 1) * F.nx + (q & 1)];
+  }
+  RedChildren red;
+  red.load(a.e + F.off, a.r + F.off, SC ? a.s + F.off : nullptr, a.coef, F, C, I, J, K);
+  const int c = lidx(C, I, J, K);
+  a.r[c] = ((red.res[0][0] + red.res[1][0]) + (red.res[1][1] + red.res[0][1])) * 0.125;
+  if (SC)
+    a.s[c] = (((u[0][0][0] + u[1][0][0]) + (u[0][0][1] + u[1][0][1])) +
+              ((u[0][1][0] + u[1][1][0]) + (u[0][1][1] + u[1][1][1]))) * 0.125;
 }
 
 // Restriction with four threads per coarse cell (consecutive lanes): each sums
@@ -885,6 +931,14 @@ void launch_restrict_check(const MGArgs<double>& fa, double* rc, const LevelDesc
 template <typename T>
 void launch_restrict(const MGArgs<T>& a, const LevelDesc& F, const LevelDesc& C, int nu1,
                      cudaStream_t s) {
+  if constexpr (sizeof(T) == sizeof(double)) {
+    if (black_residual_zero(F, nu1) && F.crx && F.cry && F.crz) {
+      dim3 block, grid;
+      check_shape(C, block, grid);
+      launch_k(a.s ? restrict_red_kernel<true> : restrict_red_kernel<false>, grid, block, 0, s, a, F, C);
+      return;
+    }
+  }
   if (sizeof(T) == sizeof(double) || C.ncell <= kSmallTransfer) {
     // four threads per coarse cell where latency bounds the restriction: FP64
     // levels, and FP32 levels up to kSmallTransfer coarse cells
