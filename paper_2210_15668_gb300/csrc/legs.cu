@@ -9,10 +9,6 @@
 
 namespace fx {
 
-#ifdef FX_LEG_BENCH
-LegPlan g_plan;
-#endif
-
 namespace {
 
 using namespace dev;
@@ -97,9 +93,6 @@ void up_tile(const LegArgs& a, const UpdateArgs* upd, cudaStream_t s) {
 // and with a shift the down leg that continues a correction (six registers more per
 // cell) the larger tile: 256x256x64 32x32/32 37, 32x16/32 50.
 LegPlan leg_plan(long long cells, int nx, int ny, int nz, bool wide) {
-#ifdef FX_LEG_BENCH
-  return g_plan;
-#endif
   if (cells < (1 << 17)) return {kLegTile16x16, 2};
   if (cells < (1 << 20)) return {kLegTile32x16, 4};
   const long long tiles = (long long)((nx + 31) / 32) * ((ny + 15) / 16);
