@@ -140,8 +140,8 @@ class ClockSampler:
 # FP64 pipe instructions per unit of work (the FP64 forms are bound by this pipe)
 FAST_INNER = -8  # fast and learned forms: V-cycles per FP64 residual chosen on the device (<= 8)
 
-FP64_INSTR = {"smooth_fine": 7.0, "smooth_coarse": 7.0, "resid": 10.0, "tdgl": 30.0, "restrict": 8.0,
-              "prolong": 4.5}
+FP64_INSTR = {"smooth_fine": 7.0, "smooth_coarse": 7.0, "resid": 10.0, "tdgl": 21.0, "restrict": 4.1,
+              "prolong": 1.8}
 # the direct FP64 form's fine sweeps run on b / diag with couplings divided by the
 # diagonal: two additions and four multiply-adds per cell
 FP64_INSTR_DIRECT_FINE = 6.0
@@ -177,8 +177,8 @@ def class_rooflines(prof, hbm_peak, fp64_classes=(), df_classes=()):
     """Per kernel class of one eager, event-timed step: time, launches, algorithmic
     bytes (from the library's own per-launch count), effective GB/s and fraction of
     the measured HBM peak; plus the whole step (sum over classes).  fp64_classes are
-    labelled bound by the FP64 pipe, df_classes (the mixed form's double-float outer
-    residual) by instruction issue on the FP32 and integer pipes."""
+    labelled bound by the FP64 pipe, df_classes (the mixed form's outer residual) as well,
+    with Boltzmann carriers on the FP32 and integer pipes beside it."""
     out = {}
     tb = tm = 0.0
     for k, (ms, n, by) in prof.items():
@@ -188,7 +188,7 @@ def class_rooflines(prof, hbm_peak, fp64_classes=(), df_classes=()):
         out[k] = {"ms": round(ms, 4), "launches": n, "bytes": by,
                   "gbs": gbs, "hbm_frac": gbs / hbm_peak if gbs else None}
         if k in df_classes:
-            out[k]["bound"] = "issue (double-float on the FP32 and integer pipes)"
+            out[k]["bound"] = "alu (FP64 pipe; carriers in double-float beside it)"
         elif k in fp64_classes:
             out[k]["bound"] = "alu (FP64 pipe)"
         tb += by
