@@ -354,7 +354,7 @@ enum { kLegTile32x32 = 0, kLegTile32x16 = 1, kLegTile16x16 = 2 };
 struct LegPlan {
   int tile, kz;
 };
-LegPlan leg_plan(long long cells, int nx, int ny, int nz, bool wide);
+LegPlan leg_plan(long long cells, int nx, int ny, int nz, bool wide, bool up = false);
 cudaError_t leg_prepare();
 void launch_leg_down(const LegArgs& a, cudaStream_t s);
 template <typename T>

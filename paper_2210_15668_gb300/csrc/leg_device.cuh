@@ -62,13 +62,13 @@ struct LegShape {
   static constexpr int PLANE = (2 * BY + 2) * PITCH;   // one published colour of one plane
 };
 
-// Blocks per SM the register allocation has to allow: with a Newton shift 16 warps
-// (128 registers instead of 130 to 150, one 240-thread block per SM otherwise); without
-// one the kernels keep the 72 to 124 registers they ask for (80 forced: 256x256x32
+// Blocks per SM the register allocation has to allow: with a Newton shift or the phi update
+// 16 warps (128 registers instead of 130 to 150, one 240-thread block per SM otherwise);
+// the others keep the 72 to 124 registers they ask for (80 forced: 256x256x32
 // mixed step 5.65 -> 6.14 ms for five solves)
-__host__ __device__ constexpr int leg_min_blocks(int threads, bool sc) {
+__host__ __device__ constexpr int leg_min_blocks(int threads, bool cap) {
   const int w = (threads + 31) / 32;
-  return sc && w < 16 ? 16 / w : 1;
+  return cap && w < 16 ? 16 / w : 1;
 }
 
 constexpr int kLegHaloZ = 6;      // planes recomputed below a z chunk at most (even)

@@ -21,7 +21,7 @@ __global__ void __launch_bounds__(LegDown<TX, TY, SC, CONT>::G::THREADS, leg_min
 }
 
 template <int TX, int TY, bool SC, bool PHI>
-__global__ void __launch_bounds__(LegUp<TX, TY, SC, PHI>::G::THREADS, leg_min_blocks(LegUp<TX, TY, SC, PHI>::G::THREADS, SC)) leg_up_kernel(LegArgs a, Upd u, const DevStats* st) {
+__global__ void __launch_bounds__(LegUp<TX, TY, SC, PHI>::G::THREADS, leg_min_blocks(LegUp<TX, TY, SC, PHI>::G::THREADS, SC || PHI)) leg_up_kernel(LegArgs a, Upd u, const DevStats* st) {
   extern __shared__ __align__(16) unsigned char leg_smem[];
   pdl_enter();
   if (PHI) u.zero = st->zero_phi;
@@ -92,12 +92,17 @@ void up_tile(const LegArgs& a, const UpdateArgs* upd, cudaStream_t s) {
 //   512x512x128 (shift)  32x16/128 297 / 217, 32x16/32 287 / 232, 32x16/16 325 / 281,
 // and with a shift the down leg that continues a correction (six registers more per
 // cell) the larger tile: 256x256x64 32x32/32 37, 32x16/32 50.
-LegPlan leg_plan(long long cells, int nx, int ny, int nz, bool wide) {
+// An up leg whose blocks would leave SMs idle takes 16 planes, two blocks to an SM (its
+// phi update waits on memory): 256x256x32, 256 blocks instead of 128: both fine legs, timed one
+// by one, 52 -> 45.5 us; the down leg gains nothing from it, and 256x256x64 (256 blocks
+// of 32 planes) loses.
+LegPlan leg_plan(long long cells, int nx, int ny, int nz, bool wide, bool up) {
   if (cells < (1 << 17)) return {kLegTile16x16, 2};
   if (cells < (1 << 20)) return {kLegTile32x16, 4};
   const long long tiles = (long long)((nx + 31) / 32) * ((ny + 15) / 16);
   int kz = 32;
   while (kz < 128 && tiles * ((nz + kz - 1) / kz) > 600) kz *= 2;
+  if (up && tiles * ((nz + kz - 1) / kz) < 152) kz = 16;
   return {wide ? kLegTile32x32 : kLegTile32x16, kz};
 }
 
@@ -121,7 +126,7 @@ void launch_leg_down(const LegArgs& a_in, cudaStream_t s) {
 
 void launch_leg_up(const LegArgs& a_in, const UpdateArgs* upd, cudaStream_t s) {
   LegArgs a = a_in;
-  const LegPlan p = leg_plan((long long)a.nx * a.ny * a.nz, a.nx, a.ny, a.nz, false);
+  const LegPlan p = leg_plan((long long)a.nx * a.ny * a.nz, a.nx, a.ny, a.nz, false, true);
   a.kz = std::min(p.kz, a.nz + (a.nz & 1));
   a.phi_vec = upd && reinterpret_cast<uintptr_t>(upd->phi) % 16 == 0;
   if (p.tile == kLegTile32x32) up_tile<32, 32>(a, upd, s);

@@ -57,8 +57,8 @@ struct Upd {
 // phi += e, e clamped to [-clamp, clamp].  An FP32 correction is clamped in FP32
 // against the limit rounded to float and widened with integer operations: one FP64 add
 // per cell instead of two FP64 min/max, a conversion and the add (GB300 runs FP64, and
-// conversions to it, at 1/58 of the FP32 rate; the up leg that updates phi on 256x256x32
-// 28.4 -> 26.1 us, the update alone 10.8 -> 8.7).  With an infinite limit (no carriers)
+// conversions to it, at 1/58 of the FP32 rate; both fine legs on 256x256x32, timed one by
+// one, 56 -> 52 us, the update alone 14.3 -> 12.2).  With an infinite limit (no carriers)
 // the result is the same bit for bit (corrections below 2^-126 count as zero).
 template <typename T>
 __device__ __forceinline__ void apply_update(const Upd& u, int idx, T e) {
