@@ -63,6 +63,9 @@ struct ferrox_ctx {
   size_t tail_smem = 0;
   int resid_blocks = 0;
   int resid_kchunk = 0;   // planes per z chunk of the residual kernel
+  std::vector<int> resid_zs;      // Fermi-Dirac carriers on a small grid: its chunks' first planes and the end
+  int* resid_zs_d = nullptr;
+  int resid_nzs = 0, resid_rows = 0;
   int resid_kchunk_df = 0;  // the same for its double-float form (longer columns per thread)
   bool direct = false;    // FP64 V-cycles on phi itself (see direct_form)
   int dense_lev = -1;     // tail level solved by its inverse (-1: none)
@@ -885,6 +888,9 @@ void enqueue_resid(ferrox_ctx* c, cudaStream_t s, int first, int set_cond,
   a.carriers_df = c->df_resid ? c->carriers_df : nullptr;
   a.partials = c->partials_d;
   a.kchunk = c->resid_kchunk;
+  a.zs = c->resid_zs_d;
+  a.nzs = c->resid_nzs;
+  a.rows = c->resid_rows;
   a.stats = c->stats_d;
   a.tol = c->num.tol;
   a.max_cycles = c->num.max_cycles;
@@ -1114,6 +1120,9 @@ void enqueue_nn_features(ferrox_ctx* c, cudaStream_t s, __nv_bfloat16* x) {
   a.partials = c->partials_d;
   a.norm_out = c->nn_scale + 1;   // ||r|| of the guess, for the check of the correction
   a.kchunk = c->resid_kchunk;
+  a.zs = c->resid_zs_d;
+  a.nzs = c->resid_nzs;
+  a.rows = c->resid_rows;
   launch_resid<T>(a, s);
   T* r = static_cast<T*>(c->r_arena);
   nn_bridge_restrict<T>(r, c->lv, c->nn_level, s);
@@ -1353,7 +1362,7 @@ void release(ferrox_ctx* c) {
   for (auto g : ge) if (g) cudaGraphExecDestroy(g);
   for (auto g : gr) if (g) cudaGraphDestroy(g);
   void* ptrs[] = {c->b, c->Pbuf, c->Fbuf, c->phi_prev, c->e_arena, c->eb_arena, c->e_alt, c->r_arena, c->s_arena, c->coef, c->coef0, c->coef0s, c->bs, c->sinv0, c->coef_df, c->carriers_df,
-                  c->planes_d, c->force_d, c->planes_f32_d, c->lv_d, c->lvt_d, c->lvm_d, c->nn_scale, c->phi_guess, c->nn_pf, c->nn_stats, c->params_d, c->stats_d, c->partials_d, c->charge_d,
+                  c->planes_d, c->force_d, c->planes_f32_d, c->lv_d, c->lvt_d, c->lvm_d, c->resid_zs_d, c->nn_scale, c->phi_guess, c->nn_pf, c->nn_stats, c->params_d, c->stats_d, c->partials_d, c->charge_d,
                   c->charge_part_d, c->dense_d, c->dense_wide_d};
   for (void* p : ptrs) if (p) cudaFree(p);
   if (c->host_pinned) cudaFreeHost(c->host_pinned);
@@ -1448,17 +1457,33 @@ ferrox_status ferrox_init_geometry(ferrox_ctx** out, const ferrox_geometry* geom
   const size_t tsz = mixed ? sizeof(float) : sizeof(double);
   plan_tail(ctx, tsz, true);
   {
-    // residual grid: split the columns into z chunks (halving, at least 4 planes each)
-    // until there are about four waves of blocks on 152 SMs; down to two planes where
-    // carriers in FP64 make the semiconductor's planes several times dearer than the
-    // others (64^3 cube with Fermi-Dirac carriers on 16 planes, launches timed one by one:
-    // 49 us with 4 planes, 43 with 2, 55 with 1)
+    // residual grid: split the columns into z chunks (halving, at least 4 planes each, two
+    // where carriers in FP64 make the semiconductor's planes several times dearer than the
+    // others) until there are about four waves of blocks on 152 SMs.  A small grid with
+    // Fermi-Dirac carriers does not reach them: its semiconductor planes keep such chunks,
+    // the others take four times as long ones, and a block has half the rows, so that the
+    // dear planes spread over the SMs and the rest costs few blocks.  64^3 cube, carriers
+    // on 16 planes, launches timed one by one: chunks of 4 planes 49 us, of 2 43, of 1 55;
+    // with half the rows 41, with longer chunks for the other planes as well 35 (eight
+    // times as long 47, twice 41).  128x128x48 (chunks of 3) loses 5% by it.
+    const int bx = (ctx->nx + kResidBX - 1) / kResidBX;
+    int bxy = bx * ((ctx->ny + kResidBY - 1) / kResidBY);
     const int least = carrier_kind(ctx) == 2 || (ctx->has_sc && !mixed) ? 2 : 4;
-    const int bxy = ((ctx->nx + kResidBX - 1) / kResidBX) * ((ctx->ny + kResidBY - 1) / kResidBY);
     int zc = 1;
     while ((long long)bxy * zc < 4LL * 152 * 3 && ctx->nz / (2 * zc) >= least) zc *= 2;
     ctx->resid_kchunk = (ctx->nz + zc - 1) / zc;
     ctx->resid_blocks = bxy * ((ctx->nz + ctx->resid_kchunk - 1) / ctx->resid_kchunk);
+    if (carrier_kind(ctx) == 2 && ctx->resid_kchunk <= 2) {
+      ctx->resid_rows = kResidBY / 2;
+      for (int z = 0; z < ctx->nz;) {
+        ctx->resid_zs.push_back(z);
+        const int sc = ctx->planes[z].sc, most = sc ? ctx->resid_kchunk : 4 * ctx->resid_kchunk;
+        for (int n = 0; z < ctx->nz && n < most && ctx->planes[z].sc == sc; ++n) ++z;
+      }
+      ctx->resid_nzs = (int)ctx->resid_zs.size();
+      ctx->resid_zs.push_back(ctx->nz);
+      ctx->resid_blocks = bx * ((ctx->ny + ctx->resid_rows - 1) / ctx->resid_rows) * ctx->resid_nzs;
+    }
     // the double-float form: at least 8 planes per thread (its block reduction and
     // per-column set-up cost more than the FP64 form's), about two waves
     int zd = 1;
@@ -1519,6 +1544,10 @@ ferrox_status ferrox_init_geometry(ferrox_ctx** out, const ferrox_geometry* geom
   FX_INIT_CK(cudaMalloc(&ctx->partials_d, std::max(3 * (size_t)ctx->resid_blocks,
                                                     2 * (size_t)ctx->check_blocks) *
                                                sizeof(double)));
+  if (ctx->resid_nzs > 0) {
+    FX_INIT_CK(cudaMalloc(&ctx->resid_zs_d, ctx->resid_zs.size() * sizeof(int)));
+    FX_INIT_CK(cudaMemcpy(ctx->resid_zs_d, ctx->resid_zs.data(), ctx->resid_zs.size() * sizeof(int), cudaMemcpyHostToDevice));
+  }
   FX_INIT_CK(cudaMalloc(&ctx->lvt_d, ctx->lv_tail.size() * sizeof(LevelDesc)));
   FX_INIT_CK(cudaMemcpy(ctx->lvt_d, ctx->lv_tail.data(), ctx->lv_tail.size() * sizeof(LevelDesc),
                         cudaMemcpyHostToDevice));

@@ -210,6 +210,8 @@ struct ResidArgs {
   int adapt_max;           // > 0: choose the next outer iteration's V-cycles (<= adapt_max)
   int launches_per_vcycle; // adaptive: kernels of one V-cycle and its countdown
   int kchunk;              // planes per z chunk of the multi-block kernel (grid.z chunks)
+  const int* zs;           // non-null: the chunks' first planes and the end (nzs chunks) instead
+  int nzs, rows;           // ... and the rows of a block (0: kResidBY)
   int inner_fixed;         // fixed V-cycles per outer iteration (when adapt_max == 0)
   double* norm_out;        // store ||r|| here instead of taking a decision
   const double* reject_ref;          // ||r|| of the guess before a learned correction: the

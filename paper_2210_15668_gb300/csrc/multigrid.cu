@@ -667,9 +667,9 @@ template <typename T, int SC, bool DFC, int R>
 __global__ void __launch_bounds__(kResidBX* kResidBY / R, DFC && SC == 1 ? 3 * R : 1) resid_kernel(ResidArgs a) {
   pdl_enter();
   const int i = blockIdx.x * kResidBX + threadIdx.x;
-  const int j = blockIdx.y * kResidBY + R * threadIdx.y;
-  const int k0 = blockIdx.z * a.kchunk;
-  const int k1 = min(a.nz, k0 + a.kchunk);
+  const int j = R * (blockIdx.y * blockDim.y + threadIdx.y);
+  const int k0 = a.zs ? __ldg(a.zs + blockIdx.z) : blockIdx.z * a.kchunk;
+  const int k1 = a.zs ? __ldg(a.zs + blockIdx.z + 1) : min(a.nz, k0 + a.kchunk);
   double acc_r = 0.0, acc_b = 0.0, acc_rho = 0.0;
   const bool in = i < a.nx && j < a.ny;
   if constexpr (sizeof(T) == sizeof(float)) {
@@ -1008,8 +1008,7 @@ template <typename T>
 void launch_resid(const ResidArgs& a_in, cudaStream_t s) {
   ResidArgs a = a_in;
   a.warp_rows = a.nx % 32 == 0;
-  const dim3 grid((a.nx + kResidBX - 1) / kResidBX, (a.ny + kResidBY - 1) / kResidBY,
-                  (a.nz + a.kchunk - 1) / a.kchunk);
+  dim3 grid((a.nx + kResidBX - 1) / kResidBX, (a.ny + kResidBY - 1) / kResidBY, (a.nz + a.kchunk - 1) / a.kchunk);
   // carriers: 0 none, 1 Boltzmann statistics only, 2 with Fermi-Dirac planes
   if constexpr (sizeof(T) == sizeof(double)) {
     if (a.coef_df) {   // the double-float diagnostic
@@ -1020,9 +1019,12 @@ void launch_resid(const ResidArgs& a_in, cudaStream_t s) {
       return;
     }
   }
+  const int by = a.rows ? a.rows : kResidBY;
+  grid.y = (a.ny + by - 1) / by;
+  if (a.zs) grid.z = a.nzs;
   auto go = [&](auto rows) {
     constexpr int R = decltype(rows)::value;
-    const dim3 block(kResidBX, kResidBY / R);
+    const dim3 block(kResidBX, by / R);
     if constexpr (sizeof(T) == sizeof(float)) {
       if (a.carriers_df) {
         if (a.carriers == 2) { launch_k(resid_kernel<T, 2, true, R>, grid, block, 0, s, a); return; }
