@@ -532,6 +532,18 @@ __device__ __forceinline__ T narrow_resid(double x) {
   return (T)x;
 }
 
+// The same to the nearest float (ties away from zero), half the error and no bias: a run
+// that takes several V-cycles per residual accepts corrections of about 1e-2 whose last
+// bits come from here.
+__device__ __forceinline__ float round_resid(double x) {
+  const unsigned long long u = (unsigned long long)__double_as_longlong(x), b = u + (1ull << 28);
+  const unsigned sign = (unsigned)(u >> 32) & 0x80000000u;
+  const int e = (int)((b >> 52) & 0x7ff) - 1023 + 127;
+  if (e >= 255 || ((u >> 52) & 0x7ff) == 0x7ff) return __uint_as_float(sign | 0x7f800000u);
+  if (e <= 0) return __uint_as_float(sign);
+  return __uint_as_float(sign | ((unsigned)e << 23) | (unsigned)((b >> 29) & 0x7fffffu));
+}
+
 // Fermi-Dirac integral of order 1/2 (normalised to e^eta for eta -> -inf) and its
 // derivative, by the approximation of Bednarczyk & Bednarczyk (1978) that the paper
 // uses for the carrier integrals: F = 1/(e^-eta + xi), xi = (3 sqrt(pi)/4) v^(-3/8),
@@ -705,9 +717,10 @@ __device__ __forceinline__ void resid_column(const ResidArgs& a, int i, int j, i
 //   DFC: Boltzmann carriers in double-float on the FP32 pipe, beside the FP64 stencil (the
 //     mixed form), added to the FP64 sum as pairs: FP32 and FP64 pipes overlap, and the
 //     exponentials cost no FP64 instruction.
+//   ROUND: the FP32 residual rounded to nearest (the single stack's mixed form).
 //   N: the type of the squared norms (float where they decide a tolerance from an FP32
 //     residual, as in resid_column_df).
-template <typename T, int SC, bool DFC, int R, typename N>
+template <typename T, int SC, bool DFC, int R, typename N, bool ROUND = false>
 __device__ __forceinline__ void resid_rows(const ResidArgs& a, int i, int j0, int k0, int k1, bool in, N& acc_r,
                                            N& acc_b, double& acc_rho) {
   const int nx = a.nx, ny = a.ny, nz = a.nz;
@@ -806,7 +819,9 @@ __device__ __forceinline__ void resid_rows(const ResidArgs& a, int i, int j0, in
         rf = df_add(df_from_double(r), rho_df).h;
         if (in) r_out[t] = (T)rf;
       } else {
-        const T rt = narrow_resid<T>(r);
+        T rt;
+        if constexpr (ROUND) rt = round_resid(r);
+        else rt = narrow_resid<T>(r);
         if (in) r_out[t] = rt;
         rf = (float)rt;
       }

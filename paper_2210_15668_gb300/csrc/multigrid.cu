@@ -674,7 +674,7 @@ __global__ void __launch_bounds__(kResidBX* kResidBY / R, DFC && SC == 1 ? 3 * R
   const bool in = i < a.nx && j < a.ny;
   if constexpr (sizeof(T) == sizeof(float)) {
     float fr = 0.0f, fb = 0.0f;
-    resid_rows<T, SC, DFC, R>(a, i, j, k0, k1, in, fr, fb, acc_rho);
+    resid_rows<T, SC, DFC, R, float, true>(a, i, j, k0, k1, in, fr, fb, acc_rho);
     if (a.no_stats) return;
     // the squared norms within the block in FP32 (no FP64 work per cell), across
     // blocks in FP64 below; ||rho||^2 in FP64
