@@ -18,12 +18,15 @@ namespace fx {
 
 // Programmatic dependent launch: each solver kernel is launched with the
 // programmatic-serialization attribute and first waits for the kernel before
-// it to complete (its memory visible).  No kernel triggers its dependents
-// early: they are released when it completes, so blocks of the next kernel
-// never sit on SMs waiting while this one still has blocks to place (measured:
-// an early trigger cost 3% in FP64, 2% in the mixed form); what remains is the
-// launch work the driver does ahead of time.  Without the attribute the wait
-// is a no-op.
+// it to complete (its memory visible), on every path: the kernels after it rely on that
+// wait for all that came before.  The solver's kernels do not trigger their dependents
+// early: they are released when a kernel completes, so blocks of the next one never sit
+// on SMs waiting while this one still has blocks to place (measured: an early trigger
+// cost 3% in FP64, 2% in the mixed form); what remains is the launch work the driver does
+// ahead of time.  The network's tensor-memory convolutions are the exception
+// (conv_tc_kernel): whatever is launched after one may start while it runs, so it reads
+// nothing that a kernel writes before its wait but the packed weights, and does not mark
+// its inputs __restrict__.  Without the attribute the wait is a no-op.
 __device__ __forceinline__ void pdl_enter() {
   asm volatile("griddepcontrol.wait;" ::: "memory");
 }

@@ -378,8 +378,12 @@ __global__ void __launch_bounds__(kTcThreads) conv_tc_kernel(
   // work done ahead, nine dependent launches of a forward pass on 8x64x64 take 44 us
   // instead of 68; inputs of kernels that may start early are not marked __restrict__,
   // which would allow their loads before the wait.
+  // The barrier puts every thread's trigger after warp 0's allocation: the successor starts
+  // once all blocks here have triggered, so all hold their columns by then.  Its blocks on
+  // the same SM may find none left and wait for this kernel; this kernel never waits for
+  // theirs, which they keep until it is done (an allocation has no time limit).
   for (int i = tid; i < WBYTES / 16; i += kTcThreads) tc_cp16(sw + 16u * i, wt + 8 * i, true);
-  __syncwarp();
+  __syncthreads();
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   pdl_enter();
   if (nmine > 0) tc_load_halo<CIN, UP>(in, s1, g, tc_tile(blockIdx.x, g, zt), zt, hb0, chunk_entries);
@@ -754,8 +758,10 @@ int grid1(long long n, int threads) {
 }
 
 // dynamic shared memory of a tensor-memory CTA (barriers, weights, two halo
-// buffers), padded so that the CTAs that fit on one SM never ask for more than
-// its 512 tensor-memory columns together
+// buffers), padded so that the CTAs of one launch that fit on one SM never ask for more
+// than its 512 tensor-memory columns together.  The launches of other layers that share
+// the SM are not counted: conv_tc_kernel lets the next one start only when all its own
+// blocks hold their columns.
 size_t tc_smem(int cin, int cout, int zt) {
   const size_t b = 128 + (size_t)27 * cin * cout * 2 + 2 * (size_t)(cin / 8) * kTcPlane * (zt + 2) * 16;
   const int per_sm = 512 / tc_cols(2 * zt * cout);
