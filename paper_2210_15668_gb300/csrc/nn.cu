@@ -723,18 +723,19 @@ __device__ __forceinline__ void pack_weight(int t, int cin, int cout, float w, b
   wbt[(((size_t)(26 - tap) * (cout / 8) + co / 8) * cin + ci) * 8 + co % 8] = val;
 }
 
-// Adam on every parameter (lr > 0) and the packed copies of the weights, all layers in one
-// launch
+// Adam on every parameter (update; a step size that rounds to zero still moves the moments and
+// clears the gradients) and the packed copies of the weights, all layers in one launch
 __global__ void __launch_bounds__(256) adam_pack_kernel(NNLayout L, float* __restrict__ p, float* __restrict__ g,
-                                                        float* __restrict__ m, float* __restrict__ v, float lr, float b1,
-                                                        float b2, float c1, float c2, float eps, bf16* __restrict__ wk,
+                                                        float* __restrict__ m, float* __restrict__ v, int update, float lr,
+                                                        float b1, float b2, float c1, float c2, float eps,
+                                                        bf16* __restrict__ wk,
                                                         bf16* __restrict__ wb, bf16* __restrict__ wkt,
                                                         bf16* __restrict__ wbt) {
   pdl_enter();
   const int t = blockIdx.x * blockDim.x + threadIdx.x;
   if (t >= L.b0[6]) return;
   float x = p[t];
-  if (lr > 0.f) {
+  if (update) {
     const float gr = g[t];
     const float mt = b1 * m[t] + (1.f - b1) * gr;
     const float vt = b2 * v[t] + (1.f - b2) * gr * gr;
@@ -922,11 +923,12 @@ void nn_skip_grad(const float* dcat, const float* dp, const bf16* s1, NNGrid f, 
 void nn_mse(const float* y, const float* tgt, int M, bf16* dy, float* loss, cudaStream_t s) {
   launch_k(mse_kernel, dim3(grid1(M, 256)), dim3(256), 0, s, y, tgt, M, dy, loss);
 }
-void nn_adam_pack(const NNLayout& L, float* p, float* g, float* m, float* v, float lr, int step, bf16* wk, bf16* wb,
-                  bf16* wkt, bf16* wbt, cudaStream_t s) {
+void nn_adam_pack(const NNLayout& L, float* p, float* g, float* m, float* v, bool update, float lr, int step, bf16* wk,
+                  bf16* wb, bf16* wkt, bf16* wbt, cudaStream_t s) {
   const float b1 = 0.9f, b2 = 0.999f;
   const float c1 = 1.f - powf(b1, (float)step), c2 = 1.f - powf(b2, (float)step);
-  launch_k(adam_pack_kernel, dim3((L.b0[6] + 255) / 256), dim3(256), 0, s, L, p, g, m, v, lr, b1, b2, c1, c2, 1e-8f, wk, wb, wkt, wbt);
+  launch_k(adam_pack_kernel, dim3((L.b0[6] + 255) / 256), dim3(256), 0, s, L, p, g, m, v, update ? 1 : 0, lr, b1, b2, c1, c2, 1e-8f,
+           wk, wb, wkt, wbt);
 }
 
 }  // namespace fx
@@ -1036,10 +1038,10 @@ cudaError_t nalloc(ferrox_nn* N, P** ptr, size_t bytes) {
   return e;
 }
 
-// one Adam update with step size lr (0: none) and the packed copies of the weights
-void adam_pack(ferrox_nn* N, float lr) {
-  fx::nn_adam_pack(N->lay, N->par, N->grad, N->mom1, N->mom2, lr, std::max(1, N->adam_step), N->wk0, N->wb0, N->wkt0,
-                   N->wbt0, N->stream);
+// one Adam update with step size lr (update) and the packed copies of the weights
+void adam_pack(ferrox_nn* N, bool update, float lr = 0.f) {
+  fx::nn_adam_pack(N->lay, N->par, N->grad, N->mom1, N->mom2, update, lr, std::max(1, N->adam_step), N->wk0, N->wb0,
+                   N->wkt0, N->wbt0, N->stream);
 }
 
 // one convolution of layer l: forward weights, or the adjoint's when adjoint is set
@@ -1191,7 +1193,7 @@ ferrox_status ferrox_nn_create(ferrox_nn** out, int D, int H, int W, int capacit
     if ((e = nalloc(N, &N->snap_x, (size_t)capacity * M * 16 * sizeof(bf16))) != cudaSuccess) return fail_alloc(e);
     if ((e = nalloc(N, &N->snap_t, (size_t)capacity * M * sizeof(float))) != cudaSuccess) return fail_alloc(e);
   }
-  adam_pack(N, 0.f);
+  adam_pack(N, false);
   if ((e = cudaDeviceSynchronize()) != cudaSuccess) {
     nn_release(N);
     return nfail(nullptr, FERROX_ECUDA, cudaGetErrorString(e));
@@ -1240,7 +1242,7 @@ ferrox_status ferrox_nn_set_params(ferrox_nn* N, const float* w, const float* b)
   const size_t nw = N->lay.w0[fx::kLayers], nb = N->lay.b0[fx::kLayers] - nw;
   FX_NCK(cudaMemcpyAsync(N->par, w, nw * sizeof(float), cudaMemcpyHostToDevice, N->stream));
   FX_NCK(cudaMemcpyAsync(N->par + nw, b, nb * sizeof(float), cudaMemcpyHostToDevice, N->stream));
-  adam_pack(N, 0.f);
+  adam_pack(N, false);
   FX_NCK(cudaStreamSynchronize(N->stream));
   return FERROX_OK;
 }
@@ -1248,7 +1250,7 @@ ferrox_status ferrox_nn_set_params(ferrox_nn* N, const float* w, const float* b)
 ferrox_status ferrox_nn_adam_step(ferrox_nn* N, double lr) {
   if (!N || !(lr > 0.0)) return nfail(N, FERROX_EINVAL, "bad argument");
   N->adam_step += 1;
-  adam_pack(N, (float)lr);
+  adam_pack(N, true, (float)lr);
   FX_NCK(cudaGetLastError());
   return FERROX_OK;
 }
@@ -1293,7 +1295,7 @@ ferrox_status ferrox_nn_train(ferrox_nn* N, int epochs, double lr, int batch, fl
         const double lr_k = lr * (0.1 + 0.45 * (1.0 + std::cos(3.141592653589793 * (double)k / (double)total)));
         ++k;
         N->adam_step += 1;
-        adam_pack(N, (float)lr_k);
+        adam_pack(N, true, (float)lr_k);
       }
     }
     FX_NCK(cudaGetLastError());
