@@ -140,7 +140,7 @@ class ClockSampler:
 # FP64 pipe instructions per unit of work (the FP64 forms are bound by this pipe)
 FAST_INNER = -8  # fast and learned forms: V-cycles per FP64 residual chosen on the device (<= 8)
 
-FP64_INSTR = {"smooth_fine": 7.0, "smooth_coarse": 7.0, "resid": 10.0, "tdgl": 21.0, "restrict": 4.1,
+FP64_INSTR = {"smooth_fine": 7.0, "smooth_coarse": 7.0, "resid": 10.0, "tdgl": 22.0, "restrict": 4.1,
               "prolong": 1.8}
 # the direct FP64 form's fine sweeps run on b / diag with couplings divided by the
 # diagonal: two additions and four multiply-adds per cell

@@ -112,9 +112,11 @@ struct PlaneTDGL {
 
 // What the FP64 update of P_z reads of a plane, with everything that is constant over a
 // run folded on the host (the update is bound by the FP64 pipe):
-//   dF = P (lin + beta P^2 + gamma P^4) + w_dn P_dn + w_up P_up + glat (sum of the four
-//        lateral neighbours) + (upper - lower face potential) / h,   f = -Gamma dF,
-// lin = alpha + 4 g44/h^2 - g11 wz_c; the face weights are those of the plane's lower face.
+//   dF = P (lin + beta P^2 + gamma P^4) + w_dn (P - P_dn) + w_up (P_up - P)
+//        + glat (sum of the four lateral neighbours - 4 P) + (upper - lower face potential) / h,
+//   f = -Gamma dF,   lin = alpha - g11 (wz_dn + wz_c + wz_up)
+// (alpha itself inside a layer, where d2/dz2 is a difference of steps); the face weights
+// are those of the plane's lower face.
 struct PlaneForce {
   int fe, pad;
   double lin, beta, gamma, w_dn, w_up, glat;
@@ -124,9 +126,9 @@ struct PlaneForce {
 __host__ __device__ inline PlaneForce plane_force(const PlaneTDGL& p, double inv_h2, double dt) {
   PlaneForce f;
   f.fe = p.fe; f.pad = 0;
-  f.lin = p.alpha + 4.0 * p.g44 * inv_h2 - p.g11 * p.wz_c;
+  f.lin = fma(-p.g11, (p.wz_c + p.wz_dn) + p.wz_up, p.alpha);
   f.beta = p.beta; f.gamma = p.gamma;
-  f.w_dn = -p.g11 * p.wz_dn; f.w_up = -p.g11 * p.wz_up;
+  f.w_dn = p.g11 * p.wz_dn; f.w_up = -p.g11 * p.wz_up;
   f.glat = -p.g44 * inv_h2;
   f.gam = -p.Gamma; f.gdt = -p.Gamma * dt;
   f.fw_L = p.fw_L; f.fw_R = p.fw_R; f.fpc = p.fpc;

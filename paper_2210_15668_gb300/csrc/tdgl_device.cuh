@@ -15,20 +15,22 @@ __device__ __forceinline__ double landau(double a, double b, double g, double P)
 }
 
 // The FP64 update of P_z along a column, plane by plane upwards.  The face potential,
-// polarization and potential that a plane shares with the next one are kept, so each is
-// computed and loaded once: 17 FP64 operations for the force and update of a cell and 4
+// polarization step and potential that a plane shares with the next one are kept, so each
+// is computed and loaded once: 18 FP64 operations for the force and update of a cell and 4
 // for its right-hand side (38 executed per cell before, with both faces of every cell
-// evaluated on their own).  Every rounding is spelled out: all kernels that march, from
-// whatever plane they start, agree bit for bit.
+// evaluated on their own).  The gradient terms are formed from differences of P, so their
+// roundings are relative to the terms and not to g/h^2 P, which is the larger by far in
+// smooth domains (one operation more than with P's coefficients collected in `lin`).
+// Every rounding is spelled out: all kernels that march, from whatever plane they start,
+// agree bit for bit.
 struct PzMarch {
-  double P, Pdn, ph, face;   // of the plane updated next: P, P below, potential, lower face potential
+  double P, dP, ph, face;    // of the plane updated next: P, its step from the plane below, potential, lower face potential
   bool ready = false;        // they are its own (the plane below was ferroelectric)
 };
 
-// potential of the face between planes k - 1 and k (f: plane k's table entry)
-__device__ __forceinline__ double face_potential(const PlaneForce& f, double ph_lo, double ph_hi, double P_lo,
-                                                 double P_hi) {
-  return fma(-f.fpc, __dadd_rn(P_hi, -P_lo), fma(f.fw_L, ph_lo, __dmul_rn(f.fw_R, ph_hi)));
+// potential of the face between planes k - 1 and k (f: plane k's table entry; dP: the step of P)
+__device__ __forceinline__ double face_potential(const PlaneForce& f, double ph_lo, double ph_hi, double dP) {
+  return fma(-f.fpc, dP, fma(f.fw_L, ph_lo, __dmul_rn(f.fw_R, ph_hi)));
 }
 
 // new P of ferroelectric plane k (cell t) of column (i, j)
@@ -40,12 +42,12 @@ __device__ __forceinline__ double advance_z(const TDGLArgs& a, PzMarch& m, const
   if (!m.ready) {
     m.P = Pz[t];
     m.ph = a.phi[t];
-    m.Pdn = k > 0 && __ldg(&a.force[k - 1].fe) ? Pz[t - plane] : 0.0;
-    m.face = k == 0 ? v_bot : face_potential(f, a.phi[t - plane], m.ph, m.Pdn, m.P);
+    m.dP = __dadd_rn(m.P, -(k > 0 && __ldg(&a.force[k - 1].fe) ? Pz[t - plane] : 0.0));
+    m.face = k == 0 ? v_bot : face_potential(f, a.phi[t - plane], m.ph, m.dP);
   }
   const double lat = __dadd_rn(__dadd_rn(Pz[t - i + im], Pz[t - i + ip]),
                                __dadd_rn(Pz[t + (long long)(jm - j) * a.nx], Pz[t + (long long)(jp - j) * a.nx]));
-  double Pup = 0.0, ph_up = 0.0, face_up = v_top;
+  double Pup = 0.0, dP_up = 0.0, ph_up = 0.0, face_up = v_top;
   bool fe_up = false;
   if (k < a.nz - 1) {
     const PlaneForce* u = a.force + k + 1;
@@ -54,13 +56,14 @@ __device__ __forceinline__ double advance_z(const TDGLArgs& a, PzMarch& m, const
     ph_up = a.phi[t + plane];
     PlaneForce fu;
     fu.fw_L = __ldg(&u->fw_L); fu.fw_R = __ldg(&u->fw_R); fu.fpc = __ldg(&u->fpc);
-    face_up = face_potential(fu, m.ph, ph_up, m.P, Pup);
+    dP_up = __dadd_rn(Pup, -m.P);
+    face_up = face_potential(fu, m.ph, ph_up, dP_up);
   }
   const double P2 = __dmul_rn(m.P, m.P);
   double dF = __dmul_rn(m.P, fma(P2, fma(f.gamma, P2, f.beta), f.lin));
-  dF = fma(f.w_dn, m.Pdn, dF);
-  dF = fma(f.w_up, Pup, dF);
-  dF = fma(f.glat, lat, dF);
+  dF = fma(f.w_dn, m.dP, dF);
+  dF = fma(f.w_up, dP_up, dF);
+  dF = fma(f.glat, fma(-4.0, m.P, lat), dF);
   dF = fma(__dadd_rn(face_up, -m.face), a.inv_h, dF);
   double pn;
   if (a.mode == 0) {
@@ -74,7 +77,7 @@ __device__ __forceinline__ double advance_z(const TDGLArgs& a, PzMarch& m, const
       pn = fma(0.5 * a.dt, __dadd_rn(a.F_store[ti], fz), a.P_base[ti]);
     }
   }
-  m.Pdn = m.P;
+  m.dP = dP_up;
   m.P = Pup;
   m.ph = ph_up;
   m.face = face_up;
