@@ -428,6 +428,16 @@ void fd_reference(double Nc, double Nv, double Eg_eV, double T, double N_A, doub
   *eta_p0 = -gap - *eta_e0;
 }
 
+// d2P/dz2 of a surface plane, weights of the plane and of its neighbour inside the layer.
+// The multiply-add is spelled out: compilers differ in what they contract, and the tables
+// are made on the host and in a kernel (1 - 2 kappa is the same either way).
+struct SurfaceWeights {
+  double c, n;
+};
+__host__ __device__ inline SurfaceWeights surface_weights(double kappa, double inv_h2) {
+  return {4.0 * fma(18.0, kappa, -3.0) / 3.0 * inv_h2, 4.0 * (1.0 - 2.0 * kappa) / 3.0 * inv_h2};
+}
+
 ferrox_status build_planes(ferrox_ctx* c) {
   const int nz = c->nz;
   c->planes.assign(nz, PlaneTDGL{});
@@ -486,11 +496,10 @@ ferrox_status build_planes(ferrox_ctx* c) {
       if (dn && up) {
         p.wz_dn = ih2; p.wz_c = -2.0 * ih2; p.wz_up = ih2;
       } else if (up || dn) {
-        const double wn = 4.0 * (1.0 - 2.0 * kappa) / 3.0 * ih2;
-        const double wc = 4.0 * (18.0 * kappa - 3.0) / 3.0 * ih2;
-        p.wz_c = wc;
-        p.wz_up = up ? wn : 0.0;
-        p.wz_dn = dn ? wn : 0.0;
+        const SurfaceWeights w = surface_weights(kappa, ih2);
+        p.wz_c = w.c;
+        p.wz_up = up ? w.n : 0.0;
+        p.wz_dn = dn ? w.n : 0.0;
       } else {
         return fail(nullptr, FERROX_EINVAL, "a ferroelectric layer must be at least 2 cells thick");
       }
@@ -3001,10 +3010,10 @@ __host__ __device__ inline PlaneTDGL static_plane(const ferrox_layer& L, const f
     if (fe_dn && fe_up) {
       p.wz_dn = ih2; p.wz_c = -2.0 * ih2; p.wz_up = ih2;
     } else {
-      const double wn = 4.0 * (1.0 - 2.0 * kappa) / 3.0 * ih2;
-      p.wz_c = 4.0 * (18.0 * kappa - 3.0) / 3.0 * ih2;
-      p.wz_up = fe_up ? wn : 0.0;
-      p.wz_dn = fe_dn ? wn : 0.0;
+      const SurfaceWeights w = surface_weights(kappa, ih2);
+      p.wz_c = w.c;
+      p.wz_up = fe_up ? w.n : 0.0;
+      p.wz_dn = fe_dn ? w.n : 0.0;
     }
   }
   if (dn) {
