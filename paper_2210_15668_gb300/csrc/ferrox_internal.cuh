@@ -465,7 +465,7 @@ bool nn_conv_uses_tc(int cin, int cout, NNGrid g);
 cudaError_t nn_tc_setup();
 void nn_conv_wgrad(const __nv_bfloat16* in, int cin, const __nv_bfloat16* dout, int cout, NNGrid g,
                    float* gw, float* gb, float* part, cudaStream_t s);
-size_t nn_wgrad_workspace(NNGrid g);
+size_t nn_wgrad_workspace();
 void nn_pool2(const __nv_bfloat16* in, NNGrid f, int C, __nv_bfloat16* out, cudaStream_t s);
 void nn_upcat(const __nv_bfloat16* a4, const __nv_bfloat16* s1, NNGrid f, __nv_bfloat16* cat, cudaStream_t s);
 void nn_up_grad(const float* dcat, const __nv_bfloat16* a4, NNGrid f, __nv_bfloat16* out, cudaStream_t s);

@@ -48,24 +48,18 @@ void up(const LegArgs& a, const UpdateArgs* upd, cudaStream_t s) {
   launch_k(leg_up_kernel<TX, TY, SC, PHI>, leg_grid<TX, TY>(a), dim3(K::G::THREADS), K::smem_bytes(a.kz), s, a, u, st);
 }
 
+cudaError_t allow_smem(const void* f) {
+  return cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024);
+}
+
 template <int TX, int TY>
 cudaError_t prepare_tile() {
-  const int lim = 227 * 1024;
-  const cudaFuncAttribute m = cudaFuncAttributeMaxDynamicSharedMemorySize;
-  cudaError_t e = cudaSuccess;
-  auto set = [&](const void* f) {
-    const cudaError_t r = cudaFuncSetAttribute(f, m, lim);
-    if (e == cudaSuccess) e = r;
-  };
-  set((const void*)leg_down_kernel<TX, TY, false, false>);
-  set((const void*)leg_down_kernel<TX, TY, false, true>);
-  set((const void*)leg_down_kernel<TX, TY, true, false>);
-  set((const void*)leg_down_kernel<TX, TY, true, true>);
-  set((const void*)leg_up_kernel<TX, TY, false, false>);
-  set((const void*)leg_up_kernel<TX, TY, false, true>);
-  set((const void*)leg_up_kernel<TX, TY, true, false>);
-  set((const void*)leg_up_kernel<TX, TY, true, true>);
-  return e;
+  for (const void* f : {(const void*)leg_down_kernel<TX, TY, false, false>, (const void*)leg_down_kernel<TX, TY, false, true>,
+                        (const void*)leg_down_kernel<TX, TY, true, false>, (const void*)leg_down_kernel<TX, TY, true, true>,
+                        (const void*)leg_up_kernel<TX, TY, false, false>, (const void*)leg_up_kernel<TX, TY, false, true>,
+                        (const void*)leg_up_kernel<TX, TY, true, false>, (const void*)leg_up_kernel<TX, TY, true, true>})
+    if (const cudaError_t e = allow_smem(f); e != cudaSuccess) return e;
+  return cudaSuccess;
 }
 
 template <int TX, int TY>
@@ -110,7 +104,7 @@ bool leg_level(const LevelDesc& L) { return L.crx && L.cry && !(L.nx & 1) && !(L
 
 cudaError_t leg_prepare() {
   cudaError_t e;
-  if ((e = prepare_tile<32, 32>()) != cudaSuccess) return e;
+  if ((e = allow_smem((const void*)leg_down_kernel<32, 32, true, true>)) != cudaSuccess) return e;
   if ((e = prepare_tile<32, 16>()) != cudaSuccess) return e;
   return prepare_tile<16, 16>();
 }
@@ -119,7 +113,7 @@ void launch_leg_down(const LegArgs& a_in, cudaStream_t s) {
   LegArgs a = a_in;
   const LegPlan p = leg_plan((long long)a.nx * a.ny * a.nz, a.nx, a.ny, a.nz, a.s && a.e_in);
   a.kz = std::min(p.kz, a.nz + (a.nz & 1));
-  if (p.tile == kLegTile32x32) down_tile<32, 32>(a, s);
+  if (p.tile == kLegTile32x32) down<32, 32, true, true>(a, s);   // wide levels only
   else if (p.tile == kLegTile32x16) down_tile<32, 16>(a, s);
   else down_tile<16, 16>(a, s);
 }
@@ -129,8 +123,7 @@ void launch_leg_up(const LegArgs& a_in, const UpdateArgs* upd, cudaStream_t s) {
   const LegPlan p = leg_plan((long long)a.nx * a.ny * a.nz, a.nx, a.ny, a.nz, false, true);
   a.kz = std::min(p.kz, a.nz + (a.nz & 1));
   a.phi_vec = upd && reinterpret_cast<uintptr_t>(upd->phi) % 16 == 0;
-  if (p.tile == kLegTile32x32) up_tile<32, 32>(a, upd, s);
-  else if (p.tile == kLegTile32x16) up_tile<32, 16>(a, upd, s);
+  if (p.tile == kLegTile32x16) up_tile<32, 16>(a, upd, s);
   else up_tile<16, 16>(a, upd, s);
 }
 

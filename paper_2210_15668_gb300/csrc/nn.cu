@@ -892,8 +892,8 @@ int wg_blocks(NNGrid g, int tz) {
   return (int)std::min<long long>(t, sm_count());
 }
 
-// floats of the weight gradients' workspace for a network whose finest grid is g
-size_t nn_wgrad_workspace(NNGrid) { return (size_t)sm_count() * wg_elems(32, 32); }
+// floats of the weight gradients' workspace: one block's sums of the largest layer per SM
+size_t nn_wgrad_workspace() { return (size_t)sm_count() * wg_elems(32, 32); }
 
 // gw and gb of one layer; part: the workspace (one layer at a time)
 void nn_conv_wgrad(const bf16* in, int cin, const bf16* dout, int cout, NNGrid g, float* gw,
@@ -999,8 +999,8 @@ struct ferrox_nn {
   bool tc = true;                // tensor-memory convolutions where the grid allows
   bf16 *x = nullptr, *a1 = nullptr, *s1 = nullptr, *p = nullptr, *a3 = nullptr, *a4 = nullptr,
        *cat = nullptr, *a5 = nullptr, *dy = nullptr, *t16a = nullptr, *t16b = nullptr,
-       *t32a = nullptr, *t32b = nullptr, *tcoarse16 = nullptr;
-  float *y = nullptr, *df = nullptr, *dcat = nullptr, *dpc = nullptr, *loss = nullptr;
+       *t32a = nullptr, *t32b = nullptr;
+  float *y = nullptr, *dcat = nullptr, *dpc = nullptr, *loss = nullptr;
   int cap = 0, count = 0, next = 0;
   bf16* snap_x = nullptr;     // [cap][M][16]
   float* snap_t = nullptr;    // [cap][M]
@@ -1164,7 +1164,7 @@ ferrox_status ferrox_nn_create(ferrox_nn** out, int D, int H, int W, int capacit
     if ((e = nalloc(N, p, np * sizeof(float))) != cudaSuccess) return fail_alloc(e);
   for (bf16** p : {&N->wk0, &N->wb0, &N->wkt0, &N->wbt0})
     if ((e = nalloc(N, p, nw * sizeof(bf16))) != cudaSuccess) return fail_alloc(e);
-  if ((e = nalloc(N, &N->part, fx::nn_wgrad_workspace(N->g) * sizeof(float))) != cudaSuccess) return fail_alloc(e);
+  if ((e = nalloc(N, &N->part, fx::nn_wgrad_workspace() * sizeof(float))) != cudaSuccess) return fail_alloc(e);
   for (int l = 0; l < fx::kLayers; ++l) {
     N->w[l] = N->par + L.w0[l];
     N->b[l] = N->par + L.b0[l];
@@ -1180,12 +1180,10 @@ ferrox_status ferrox_nn_create(ferrox_nn** out, int D, int H, int W, int capacit
   struct { bf16** p; size_t n; } bufs[] = {
       {&N->x, M * 16}, {&N->a1, M * 16}, {&N->s1, M * 16}, {&N->p, Mc * 16}, {&N->a3, Mc * 32},
       {&N->a4, Mc * 32}, {&N->cat, M * 48}, {&N->a5, M * 16}, {&N->dy, M * 16},
-      {&N->t16a, M * 16}, {&N->t16b, M * 16}, {&N->t32a, Mc * 32}, {&N->t32b, Mc * 32},
-      {&N->tcoarse16, Mc * 16}};
+      {&N->t16a, M * 16}, {&N->t16b, M * 16}, {&N->t32a, Mc * 32}, {&N->t32b, Mc * 32}};
   for (auto& bq : bufs)
     if ((e = nalloc(N, bq.p, bq.n * sizeof(bf16))) != cudaSuccess) return fail_alloc(e);
-  struct { float** p; size_t n; } fbufs[] = {{&N->y, M}, {&N->df, M * 48}, {&N->dcat, M * 48},
-                                              {&N->dpc, Mc * 16}, {&N->loss, 4}};
+  struct { float** p; size_t n; } fbufs[] = {{&N->y, M}, {&N->dcat, M * 48}, {&N->dpc, Mc * 16}, {&N->loss, 4}};
   for (auto& bq : fbufs)
     if ((e = nalloc(N, bq.p, bq.n * sizeof(float))) != cudaSuccess) return fail_alloc(e);
   if ((e = nalloc(N, &N->fault, sizeof(int))) != cudaSuccess) return fail_alloc(e);
