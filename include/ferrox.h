@@ -268,15 +268,22 @@ ferrox_status ferrox_fe_planes(const ferrox_ctx* ctx, int* fe_lo, int* fe_hi);
 ferrox_status ferrox_get_state_fe(ferrox_ctx* ctx, double* P_fe_host, double* phi_host);
 ferrox_status ferrox_set_state_fe(ferrox_ctx* ctx, const double* P_fe_host, const double* phi_host);
 
-/* Kernel classes reported by ferrox_profile_step. */
+/* Kernel classes reported by ferrox_profile_step.  A launch that does the work of several
+ * classes counts as one.  In the mixed form with two sweeps each way, a level's way down
+ * (two sweeps, residual, restriction) and its way up (prolongation + correction, two
+ * sweeps) are a launch each: SMOOTH0 both on the fine level, RESTRICT and PROLONG on the
+ * others, whose sweeps then show in no class of their own. */
 enum {
   FERROX_K_TDGL = 0,      /* fused TDGL update + right-hand side */
-  FERROX_K_RESID = 1,     /* FP64 outer residual, carrier charge, norms, convergence test */
-  FERROX_K_SMOOTH0 = 2,   /* red-black Gauss-Seidel colour sweep on the fine level */
+  FERROX_K_RESID = 1,     /* outer residual, carrier charge, norms, convergence test (direct FP64
+                             form: with the fine level's restriction) */
+  FERROX_K_SMOOTH0 = 2,   /* red-black Gauss-Seidel colour sweeps of the fine level, or its ways
+                             down and up */
   FERROX_K_SMOOTHC = 3,   /* colour sweeps on coarser multi-block levels */
-  FERROX_K_RESTRICT = 4,  /* residual + restriction */
-  FERROX_K_PROLONG = 5,   /* prolongation + correction */
-  FERROX_K_TAIL = 6,      /* single-CTA V-cycle over the smallest levels */
+  FERROX_K_RESTRICT = 4,  /* residual + restriction, or a coarser level's way down */
+  FERROX_K_PROLONG = 5,   /* prolongation + correction, or a coarser level's way up */
+  FERROX_K_TAIL = 6,      /* the smallest levels in one launch: a V-cycle of one CTA or a dense
+                             solve, or, with the levels above them, of a cluster of CTAs */
   FERROX_K_UPDATE = 7,    /* phi += correction */
   FERROX_K_COPY = 8,      /* copy of the new polarization; initial-guess extrapolation */
   FERROX_K_COUNT = 9

@@ -1468,13 +1468,17 @@ ferrox_status ferrox_init_geometry(ferrox_ctx** out, const ferrox_geometry* geom
   {
     // residual grid: split the columns into z chunks (halving, at least 4 planes each, two
     // where carriers in FP64 make the semiconductor's planes several times dearer than the
-    // others) until there are about four waves of blocks on 152 SMs.  A small grid with
-    // Fermi-Dirac carriers does not reach them: its semiconductor planes keep such chunks,
-    // the others take four times as long ones, and a block has half the rows, so that the
-    // dear planes spread over the SMs and the rest costs few blocks.  64^3 cube, carriers
+    // others) until there are about four waves of blocks on 152 SMs.  Where the halving ends
+    // at chunks of two planes with Fermi-Dirac carriers, the semiconductor's planes keep
+    // them, the others take four times as long ones, and a block has half the rows, so that
+    // the dear planes spread over the SMs and the rest costs few blocks.  64^3 cube, carriers
     // on 16 planes, launches timed one by one: chunks of 4 planes 49 us, of 2 43, of 1 55;
     // with half the rows 41, with longer chunks for the other planes as well 35 (eight
-    // times as long 47, twice 41).  128x128x48 (chunks of 3) loses 5% by it.
+    // times as long 47, twice 41); whole runs 6892 -> 6462 us, 32^3 3985 -> 3586.  Grids
+    // that end at chunks of three or four planes below four waves keep plain chunks: there it
+    // depends on the planes (whole runs, plain / split, us: 48^3 6816 / 6445, 96^3 15064 /
+    // 14570, 128x128x48 with 12 semiconductor planes in FP64 14042 / 14168, 128x128x24 9529 /
+    // 10575, in the mixed form 6411 / 7416).
     const int bx = (ctx->nx + kResidBX - 1) / kResidBX;
     int bxy = bx * ((ctx->ny + kResidBY - 1) / kResidBY);
     const int least = carrier_kind(ctx) == 2 || (ctx->has_sc && !mixed) ? 2 : 4;

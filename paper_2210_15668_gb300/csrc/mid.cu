@@ -13,7 +13,8 @@
 // same way, a tail of its own (a V-cycle of CTA 0 or the dense solve, its rows spread over
 // the cluster) goes through global memory as between launches.  Each cell sees the
 // operations of smooth_pair, cell_residual, restrict4_kernel (restrict_cell) and
-// prolong_fine in the same order: a V-cycle equals the separate launches bit for bit.
+// prolong_fine in the same order: a V-cycle equals the separate launches bit for bit (FP64
+// quotients by a shifted diagonal: over_recip).
 //
 // A colour phase is bound by its latencies, 0.35 to 0.5 us (a load from another SM, six
 // dependent FP64 operations of about 27 ns, 74 ns of barrier).  Measured: 64x64x16 FP64,
@@ -78,9 +79,13 @@ __device__ __forceinline__ T ld_at(unsigned a) {
 __device__ __forceinline__ double mul_rn(double a, double b) { return __dmul_rn(a, b); }
 __device__ __forceinline__ float mul_rn(float a, float b) { return __fmul_rn(a, b); }
 
-// x / d from ri = 1 / d rounded to nearest: one residual correction of x * ri gives the
-// rounded quotient (Markstein, IBM J. Res. Dev. 34, 1990), two operations instead of a
-// division's dozen in the chain of every shifted cell
+// x / d from ri = 1 / d rounded to nearest: x * ri with one residual correction, two
+// operations instead of a division's dozen in the chain of every shifted cell.  Markstein
+// (IBM J. Res. Dev. 34, 1990) proves the rounded quotient from a start within one unit in
+// the last place; x * ri may be 1.5 off, so a quotient next to a midpoint of two numbers
+// could still round the other way.  Two billion pairs, half of them made to lie there, gave
+// the division's bits.  Not so where the residual underflows (|x| below about 1e-290), and
+// an infinite x gives NaN (a solve that ends as not finite either way).
 __device__ __forceinline__ double over_recip(double x, double d, double ri) {
   const double t = __dmul_rn(x, ri);
   return fma(fma(-d, t, x), ri, t);

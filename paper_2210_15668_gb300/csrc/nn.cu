@@ -6,9 +6,11 @@
 // and y and zero-padded in z, like the device.  Gradients with respect to the
 // input use the same kernel with the taps flipped and the channel matrices
 // transposed (the adjoint convolution); gradients with respect to the weights
-// contract over voxels (M = input channels, N = output channels, K = voxels)
-// and are summed into FP32 with atomics.  Master weights, Adam moments and
-// gradients are FP32; the kernels read BF16 copies.
+// contract over voxels (M = input channels, N = output channels, K = voxels) into one
+// FP32 partial sum per block, and the partial sums are added in a fixed order.  Grids that
+// the tensor-memory convolution's tiles divide take that kernel instead of mma.sync
+// (conv_tc_kernel).  Master weights, Adam moments and gradients are FP32; the kernels read
+// BF16 copies.
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
 
@@ -879,7 +881,11 @@ bool nn_conv_upcat_tc(const bf16* a4, const bf16* s1, const bf16* wt, const floa
   return true;
 }
 
-// Planes per tile of the weight gradient: the most of {4, 2} that leaves every SM a tile.
+// Planes per tile of the weight gradient: the most of {4, 2} that leaves five of six SMs a
+// tile (128 of 152).  A whole training step, us, with a tile asked for 128 or for all 152 SMs:
+// 8x64x64 (two planes 128 tiles) 242 / 248, 16x48x48 (144) 256 / 260, 14x66x62 (four planes
+// 144) 383 / 390, 16x72x64 (144) 424 / 432, 16x64x64 (128) 284 / 284; for 64 SMs 8x64x64
+// takes 248 and 16x48x48 267: fewer, deeper tiles load less halo until SMs idle.
 int wg_tz(NNGrid g) {
   const long long t = (long long)((g.W + kWgX - 1) / kWgX) * ((g.H + kWgY - 1) / kWgY);
   for (int tz : {4, 2})
