@@ -110,7 +110,7 @@ __device__ __forceinline__ double rhs_of_f32(const TDGLArgs& a, int k, double pd
   return b;
 }
 
-// the FP64 update (tdgl_chunk).  256x256 columns of 10 ferroelectric planes: 49.8 -> 40.6 us,
+// the FP64 update (tdgl_chunk).  256x256 columns of 10 ferroelectric planes: 49.8 -> 42 us,
 // the FP64 pipe busy throughout
 __global__ void __launch_bounds__(kCX* kCY* kCZ) tdgl_chunk_kernel(TDGLArgs a) {
   pdl_enter();
